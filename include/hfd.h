@@ -246,7 +246,7 @@ hfd_status hfd_steps_profiled(hfd_mesh* mesh, double* U, double dt, int32_t nste
  * arrays in internal order), but the per-call scratch (state copy, vertex and edge fluxes) is a
  * fixed 8 MiB array compiled into the library, held on every GPU that loads the library until
  * the process exits.  That is room for about 32,000 vertices in FP64 (256 bytes each with their
- * ~3 flux edges) or 65,000 in FP32 bulk; larger meshes get HFD_ERR_ARG with the bytes needed.
+ * ~3 flux edges; above 28,000 the plain FP64 divergence runs, see hfd_mesh_set_fp64_div) or 65,000 in FP32 bulk; larger meshes get HFD_ERR_ARG with the bytes needed.
  * Every call looks up the array's device address (cudaGetSymbolAddress, with the mesh's device
  * current), so the address stays right across a cudaDeviceReset; the first call on a device
  * may also load the library's device code there, so make that first call before any stream
@@ -298,12 +298,12 @@ hfd_status hfd_mesh_set_launch(hfd_mesh* mesh, int32_t persistent, int32_t grid)
  * HFD_ERR_TIMEOUT in the error word and returns instead of waiting.  Drops captured graphs. */
 hfd_status hfd_mesh_set_barrier_limit(hfd_mesh* mesh, uint32_t polls);
 
-/* Lanes (threads) per vertex in the divergence gather: 1, 2, 4 or 8.  The defaults are 1 for
- * FP64 meshes (FP64-pipe bound: no cross-lane reduction) and 4 for FP32 meshes (memory bound:
- * coalesced groups); small meshes fill the GPU better with more lanes.  Each lane sums a
- * strided share of the entries and the shares are combined by a fixed reduce-scatter, so a lane
- * count gives deterministic results that agree with the other counts to rounding.  The
- * persistent form (hfd_mesh_set_launch) has kernels for 1, 2 and 4 lanes and runs 8 as 4.  Drops
+/* Lanes (threads) per vertex in the divergence gather: 1, 2, 4 or 8.  The default is 4 (coalesced
+ * groups), and 8 for FP64 meshes of fewer than 20,000 rows, which fill the GPU better so.  Each lane
+ * sums a strided share of the entries and the shares are combined by a fixed reduce-scatter, so a
+ * lane count gives deterministic results that agree with the other counts to rounding; the
+ * fixed-point FP64 divergence (hfd_mesh_set_fp64_div) has 4 and 8 lanes, runs 1 and 2 as 4, and
+ * gives the same bits with both.  The persistent form (hfd_mesh_set_launch) has kernels for 1, 2 and 4 lanes and runs 8 as 4.  Drops
  * captured graphs.  Errors: HFD_ERR_ARG (another count, or a persistent grid set by
  * hfd_mesh_set_launch that the new count's kernel cannot hold co-resident). */
 hfd_status hfd_mesh_set_lanes(hfd_mesh* mesh, int32_t lanes);
@@ -344,8 +344,14 @@ hfd_status hfd_check_conversions(int64_t n, const double* x, float* f_int, float
  * ~1e-11 relative there, against ~1e-12 for the plain form.  Speed on the four-quadrant
  * 1024x1024 mesh (GB300): the divergence 1.66 ms against 2.23 ms, the edge kernel 0.11 ms
  * slower (it forms dh), the step 11.05 ms against 12.45 ms.  The viscous rows stay FP64.
- * folded = 0: the plain form, 24 FP64 multiply-adds per stencil vertex and 12 per stencil edge
- * on the FP64 pipe, with the lane count of hfd_mesh_set_lanes.  Drops captured graphs.
+ * folded = 0: fixed point.  Each row's coefficients and the fluxes it reads are 57-bit integers
+ * relative to their largest, multiplied and summed exactly on the integer pipe (three 32x32+64-bit
+ * multiply-adds per product), so that only the factors are rounded: the sums are closer to the exact
+ * ones than those of FP64 multiply-adds (rms error 0.15 to 0.35 of theirs) and do not depend on
+ * the order of the entries or the lane count.  Rows that read a flux that is not finite are
+ * evaluated in FP64.  Meshes with a row of more than 400 products (2 per vertex, 1 per edge) take
+ * the plain FP64 form, as does the persistent launch: 24 FP64 multiply-adds per stencil vertex
+ * and 12 per stencil edge with the lane count of hfd_mesh_set_lanes.  Drops captured graphs.
  * Errors: HFD_ERR_ARG (folded not 0 or 1), HFD_ERR_UNSUPPORTED (folded = 1 on an FP32 mesh). */
 hfd_status hfd_mesh_set_fp64_div(hfd_mesh* mesh, int32_t folded);
 

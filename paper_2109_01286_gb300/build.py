@@ -29,7 +29,7 @@ def _nvcc():
 
 
 def _sources():
-    return [os.path.join(CSRC, f) for f in ("prep.cpp", "kernels.cu", "api.cu", "noalloc.cu",
+    return [os.path.join(CSRC, f) for f in ("prep.cpp", "kernels.cu", "div_fixed.cu", "api.cu", "noalloc.cu",
                                             "adjoint.cu", "peaks.cu", "prep3.cpp", "kernels3d.cu",
                                             "api3d.cu")]
 
@@ -37,7 +37,8 @@ def _sources():
 def _deps():
     return _sources() + [os.path.join(CSRC, f) for f in ("prep.hpp", "kernels.hpp", "mesh.hpp",
                                                          "adjoint_kernels.cuh", "linalg.hpp",
-                                                         "mesh3.hpp", "kernels3d.hpp", "fp_convert.cuh")] + \
+                                                         "mesh3.hpp", "kernels3d.hpp", "fp_convert.cuh",
+                                                         "fixed_point.cuh", "div_common.cuh", "mbar.cuh")] + \
         [os.path.join(INCLUDE, "hfd.h"), os.path.join(INCLUDE, "hfd3d.h"), os.path.abspath(__file__)]
 
 
@@ -68,10 +69,13 @@ def build(force=False, verbose=False):
         else:
             cmds.append([nvcc, ARCH, "-lineinfo", "-Xcompiler", "-fPIC,-ffp-contract=off"] +
                         common + ["-c", src, "-o", obj])
-    kcheck = os.path.join(bdir, "kernels_check.cu.o")
-    cmds.append([nvcc, ARCH, "-lineinfo", "-Xcompiler", "-fPIC,-ffp-contract=off", "-DHFD_CHECK=1"] +
-                common + ["-c", os.path.join(CSRC, "kernels.cu"), "-o", kcheck])
-    objs_check = [kcheck if o.endswith(os.sep + "kernels.cu.o") else o for o in objs]
+    checked = {}                    # the kernels with gathers, with every index tested
+    for name in ("kernels", "div_fixed"):
+        checked[os.path.join(bdir, name + ".cu.o")] = os.path.join(bdir, name + "_check.cu.o")
+        cmds.append([nvcc, ARCH, "-lineinfo", "-Xcompiler", "-fPIC,-ffp-contract=off", "-DHFD_CHECK=1"] +
+                    common + ["-c", os.path.join(CSRC, name + ".cu"), "-o",
+                              checked[os.path.join(bdir, name + ".cu.o")]])
+    objs_check = [checked.get(o, o) for o in objs]
     procs = [subprocess.Popen(c, stdout=subprocess.PIPE, stderr=subprocess.STDOUT, text=True)
              for c in cmds]
     failed = []

@@ -9,9 +9,12 @@
 #include <map>
 #include <new>
 #include <numeric>
+#include <thread>
 #include <type_traits>
 #include <vector>
 
+#include "fixed_point.cuh"
+#include "linalg.hpp"
 #include "kernels.hpp"
 #include "mesh.hpp"
 #include "prep.hpp"
@@ -104,6 +107,92 @@ hfd_status dev_alloc(hfd_mesh* m, void** dst, size_t bytes) {
     hfd_status s_ = (x);             \
     if (s_ != HFD_OK) return s_;     \
   } while (0)
+
+// The fixed-point form of an FP64 mesh's divergence (d.fx, d.div_fx): chunk pointers and tile
+// records here, the coefficients packed on the device from the uploaded rows.  Meshes whose rows
+// have no such form (a row of more than kFxRowMax28 products, coefficients outside the exponent
+// field, a tile too large for shared memory) keep the plain FP64 kernel.
+hfd_status build_div_fx(hfd_mesh* m, const std::vector<int32_t>& vptr, const std::vector<int32_t>& vidx,
+                        const std::vector<int32_t>& eptr, const std::vector<int32_t>& eidx) {
+  DevMesh& d = m->dm;
+  hfd::DivFx& f = d.fx;
+  const int A = d.A, C = hfd::kDivChunk;
+  d.div_fx = 0;
+  if (A == 0 || d.Ef == 0) return HFD_OK;
+  std::vector<int32_t> cv(A + 1, 0), ce(A + 1, 0);
+  for (int r = 0; r < A; ++r) {
+    const int N = vptr[r + 1] - vptr[r], M = eptr[r + 1] - eptr[r];
+    if (N == 0 || M == 0 || 2 * N + M > hfd::kFxRowMax28) return HFD_OK;
+    if (2 * N + M > hfd::kFxRowMax29) f.L = 28;
+    cv[r + 1] = cv[r] + (N + C - 1) / C;
+    ce[r + 1] = ce[r] + (M + C - 1) / C;
+  }
+  // tiles
+  f.rows = A < hfd::kFxSmallRows ? 8 : 16;
+  const int nt = (A + f.rows - 1) / f.rows;
+  std::vector<int4> head(nt);
+  std::vector<std::vector<int32_t>> recs(nt);
+  std::vector<int64_t> bytes(nt);
+  const int nth = m->opts.nthreads > 0 ? m->opts.nthreads : (int)std::max(1u, std::thread::hardware_concurrency());
+  hfd::parallel_for(nt, nth, [&](int64_t t, int) {
+    const int r0 = (int)t * f.rows, r1 = std::min(A, r0 + f.rows);
+    const std::vector<int32_t>* idx[2] = {&vidx, &eidx};
+    const int32_t* ptr[2] = {vptr.data(), eptr.data()};
+    std::vector<int32_t> list[2];
+    for (int k = 0; k < 2; ++k) {
+      list[k].assign(idx[k]->begin() + ptr[k][r0], idx[k]->begin() + ptr[k][r1]);
+      std::sort(list[k].begin(), list[k].end());
+      list[k].erase(std::unique(list[k].begin(), list[k].end()), list[k].end());
+    }
+    std::vector<uint16_t> pos;
+    for (int k = 0; k < 2; ++k)
+      for (int r = r0; r < r1; ++r) {
+        const size_t first = pos.size();
+        for (int j = ptr[k][r]; j < ptr[k][r + 1]; ++j)
+          pos.push_back((uint16_t)(std::lower_bound(list[k].begin(), list[k].end(), (*idx[k])[j]) - list[k].begin()));
+        while (pos.size() % C) pos.push_back(pos[first]);   // padding stays within the row's scale
+      }
+    while (pos.size() % 8) pos.push_back(0);
+    std::vector<int32_t>& rec = recs[t];
+    const size_t nv = list[0].size(), ne = list[1].size(), ids = (nv + ne + 3) & ~(size_t)3;
+    rec.assign(ids + pos.size() / 2, 0);
+    std::copy(list[0].begin(), list[0].end(), rec.begin());
+    std::copy(list[1].begin(), list[1].end(), rec.begin() + nv);
+    std::memcpy(&rec[ids], pos.data(), pos.size() * sizeof(uint16_t));
+    head[t] = make_int4(0, (int)rec.size() / 4, (int)nv, (int)ne);
+    bytes[t] = 4 * (int64_t)rec.size() + (d.viscous ? 144 : 72) * (int64_t)nv + 40 * (int64_t)ne;
+  });
+  std::vector<int32_t> rec;
+  int64_t most = 0;
+  for (int t = 0; t < nt; ++t) {
+    if (rec.size() / 4 > (size_t)INT32_MAX) return HFD_OK;
+    head[t].x = (int)(rec.size() / 4);
+    rec.insert(rec.end(), recs[t].begin(), recs[t].end());
+    most = std::max(most, bytes[t]);
+  }
+  if (most > hfd::kFxSmemMax) return HFD_OK;
+  f.smem = (int)((most + 15) & ~(int64_t)15);
+  const size_t nv = (size_t)cv[A], ne = (size_t)ce[A];
+  int32_t* flag = nullptr;
+  TRY(dev_upload(m, (void**)&f.head, head));
+  TRY(dev_upload(m, (void**)&f.rec, rec));
+  TRY(dev_upload(m, (void**)&f.vptr, cv));
+  TRY(dev_upload(m, (void**)&f.eptr, ce));
+  TRY(dev_alloc(m, (void**)&f.cv, nv * 192));
+  TRY(dev_alloc(m, (void**)&f.ce, ne * 96));
+  if (d.viscous) TRY(dev_alloc(m, (void**)&f.cvis, nv * 192));
+  TRY(dev_alloc(m, (void**)&f.cexp, (size_t)A * sizeof(int2)));
+  TRY(dev_alloc(m, (void**)&f.ex, (size_t)d.V * 2 * sizeof(unsigned)));
+  if (d.viscous) TRY(dev_alloc(m, (void**)&f.exv, (size_t)d.V * 2 * sizeof(unsigned)));
+  TRY(dev_alloc(m, (void**)&f.ee, (size_t)d.Ef * 2 * sizeof(unsigned)));
+  TRY(dev_alloc(m, (void**)&flag, sizeof(int32_t)));
+  CK(hfd::prepare_div_fx(d));
+  CK(hfd::pack_div_fx(d, flag, nullptr));
+  int32_t none = 0;
+  CK(cudaMemcpy(&none, flag, sizeof none, cudaMemcpyDeviceToHost));
+  d.div_fx = none ? 0 : 1;
+  return HFD_OK;
+}
 
 // Upload the coefficient streams in bulk precision T.
 template <typename T>
@@ -318,6 +407,7 @@ hfd_status upload_streams(hfd_mesh* m, const hfd::Prep& P, const std::vector<int
   TRY(dev_upload(m, &d.cv, cv));
   TRY(dev_upload(m, &d.ce, ce));
   if (P.opts.viscous) TRY(dev_upload(m, &d.cvis, cvis));
+  if (std::is_same<T, double>::value) TRY(build_div_fx(m, vptr, vidx, eptr, eidx));
   const size_t V = d.V;
   TRY(dev_alloc(m, &d.Ua, V * 12 * sizeof(T)));
   TRY(dev_alloc(m, &d.FG, V * 8 * sizeof(T)));
@@ -427,9 +517,10 @@ hfd_status upload(const hfd::Prep& P, int precision, hfd_mesh* m) {
   TRY(dev_alloc(m, (void**)&m->U1, (size_t)12 * V * sizeof(double)));
   TRY(dev_alloc(m, (void**)&m->U2, (size_t)12 * V * sizeof(double)));
   CK(cudaStreamCreateWithFlags(&m->cap, cudaStreamNonBlocking));
-  // lanes per vertex in the divergence: FP64 is bound by the FP64 pipe and runs best without a
-  // cross-lane reduction (1); the FP32 path is bound by memory and prefers coalesced groups (4)
-  m->lanes = m->opts.precision == 0 ? 1 : 4;
+  // lanes per vertex in the divergence: the fixed-point FP64 kernel and the FP32 one take coalesced
+  // groups of 4 (8 where the mesh is too small to fill the GPU, see div_fixed.cu); the plain FP64
+  // kernel is bound by the FP64 pipe and runs best without a cross-lane reduction (1)
+  m->lanes = m->opts.precision != 0 ? 4 : !d.div_fx ? 1 : d.fx.rows == 8 ? 8 : 4;
   if (const char* env = getenv("HFD_DIV_LANES")) {   // tuning override: 1, 2, 4 or 8
     int l = atoi(env);
     if (l == 1 || l == 2 || l == 4 || l == 8) m->lanes = l;

@@ -22,29 +22,13 @@
 
 #include <type_traits>
 
-#include "kernels.hpp"
+#include "div_common.cuh"
+#include "fixed_point.cuh"
 #include "fp_convert.cuh"
+#include "kernels.hpp"
+#include "mbar.cuh"
 
 namespace hfd {
-
-enum : unsigned { ERRBIT_NONFINITE = 1u, ERRBIT_POSITIVITY = 2u, ERRBIT_TIMEOUT = 4u, ERRBIT_INDEX = 8u };
-
-// Bounds-checked build (compiled with -DHFD_CHECK=1, the stand-in for a memory checker): every
-// gathered index is tested against its array's extent; one outside [0, n) records ERRBIT_INDEX
-// in the mesh's error word and is replaced by 0, so that the access stays in bounds (the result
-// is then wrong, and hfd_check reports it).  In the normal build this is the identity.
-#ifndef HFD_CHECK
-#define HFD_CHECK 0
-#endif
-__device__ __forceinline__ int chk_idx(int i, int n, unsigned* err) {
-#if HFD_CHECK
-  if ((unsigned)i >= (unsigned)n) {
-    atomicOr(err, ERRBIT_INDEX);
-    return 0;
-  }
-#endif
-  return i;
-}
 
 // ------------------------------------------------------------------ vector loads
 __device__ __forceinline__ void ld12(const double* p, double* o) {
@@ -423,10 +407,40 @@ __device__ __forceinline__ void smoothness(T u0, T u1, T u2, T u3, T u4, T* b) {
 }
 
 // ------------------------------------------------------------------ k_vertex
+// A vertex's two flux vectors: 8 values of T, or (FP64 with an array of exponent codes) the
+// fixed-point divergence's stored pairs and the vertex's exponent word.
+__device__ __forceinline__ void st_fluxes(float* FG, int v, const float* F, const float* G, uint2*,
+                                          int) {
+  st4(FG + (size_t)v * 8, F);
+  st4(FG + (size_t)v * 8 + 4, G);
+}
+__device__ __forceinline__ void st_fluxes(double* FG, int v, const double* F, const double* G,
+                                          uint2* ex, int L) {
+  if (!ex) {
+    st4(FG + (size_t)v * 8, F);
+    st4(FG + (size_t)v * 8 + 4, G);
+    return;
+  }
+  int E[4];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) E[q] = max(fx_code(F[q]), fx_code(G[q]));
+  int4* o = reinterpret_cast<int4*>(FG + (size_t)v * 8);
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    const int2 a = fx_encode(F[2 * i], E[2 * i], L), b = fx_encode(F[2 * i + 1], E[2 * i + 1], L);
+    const int2 c = fx_encode(G[2 * i], E[2 * i], L), d = fx_encode(G[2 * i + 1], E[2 * i + 1], L);
+    o[i] = make_int4(a.x, a.y, b.x, b.y);
+    o[2 + i] = make_int4(c.x, c.y, d.x, d.y);
+  }
+  ex[v] = make_uint2((unsigned)E[0] | ((unsigned)E[1] << 16), (unsigned)E[2] | ((unsigned)E[3] << 16));
+}
+
 template <typename T, bool VISC>
 __device__ __forceinline__ void vertex_body(int v, int V, const double* __restrict__ U, T* Ua,
                                             T* FG, T* FGv, const Phys& ph, float* wref,
-                                            const float* s0f, const double* s0d) {
+                                            const float* s0f, const double* s0d,
+                                            uint2* ex = nullptr, uint2* exv = nullptr,
+                                            int fxL = 0) {
   if (v >= V) return;
   double w[12];
 #pragma unroll
@@ -468,8 +482,7 @@ __device__ __forceinline__ void vertex_body(int v, int V, const double* __restri
     T p = pressure(q, g1);
     T F[4] = {q[1], q[1] * u + p, q[2] * u, (q[3] + p) * u};
     T Gf[4] = {q[2], q[1] * vv, q[2] * vv + p, (q[3] + p) * vv};
-    st4(FG + (size_t)v * 8, F);
-    st4(FG + (size_t)v * 8 + 4, Gf);
+    st_fluxes(FG, v, F, Gf, ex, fxL);
   }
   if (VISC) {   // viscous flux from w, w_x, w_y (Sec. 2.3; chain rule for the primitives)
     double rho = w[0], uu = w[1] / rho, vw = w[2] / rho;
@@ -488,8 +501,7 @@ __device__ __forceinline__ void vertex_body(int v, int V, const double* __restri
     double txy = mu * (uy + vx);
     T Fv[4] = {T(0), T(txx), T(txy), T(uu * txx + vw * txy + ph.kappa * Tx)};
     T Gv[4] = {T(0), T(txy), T(tyy), T(uu * txy + vw * tyy + ph.kappa * Ty)};
-    st4(FGv + (size_t)v * 8, Fv);
-    st4(FGv + (size_t)v * 8 + 4, Gv);
+    st_fluxes(FGv, v, Fv, Gv, exv, fxL);
   }
 }
 
@@ -507,11 +519,13 @@ __device__ __forceinline__ void block_reference(const double* __restrict__ U, in
 
 template <typename T, bool VISC>
 __global__ void __launch_bounds__(256) k_vertex(int V, const double* __restrict__ U, T* Ua, T* FG,
-                                                T* FGv, Phys ph, float* wref) {
+                                                T* FGv, Phys ph, float* wref, uint2* ex,
+                                                uint2* exv, int fxL) {
   __shared__ float s0f[4];
   __shared__ double s0d[4];
   if constexpr (std::is_same<T, float>::value) block_reference(U, V, s0f, s0d);
-  vertex_body<T, VISC>(blockIdx.x * blockDim.x + threadIdx.x, V, U, Ua, FG, FGv, ph, wref, s0f, s0d);
+  vertex_body<T, VISC>(blockIdx.x * blockDim.x + threadIdx.x, V, U, Ua, FG, FGv, ph, wref, s0f, s0d,
+                       ex, exv, fxL);
 }
 
 // ------------------------------------------------------------------ k_edge
@@ -557,7 +571,9 @@ __device__ __forceinline__ void edge_body(int e, int Ef, int V, const int32_t* _
                                           const T* __restrict__ w3, const T* __restrict__ Ua,
                                           T* __restrict__ h, const Phys& ph, unsigned* err,
                                           uint8_t* __restrict__ dbg, const float* __restrict__ wref,
-                                          const double* __restrict__ FGd = nullptr) {
+                                          const double* __restrict__ FGd = nullptr,
+                                          const uint2* __restrict__ ex = nullptr,
+                                          uint2* __restrict__ ee = nullptr, int fxL = 0) {
   if (e >= Ef) return;
   const T g1 = phys_g1<T>(ph);
   int s[6];
@@ -739,6 +755,21 @@ __device__ __forceinline__ void edge_body(int e, int Ef, int V, const int32_t* _
       o[1] = make_float4(t[2].hi, t[2].lo, t[3].hi, t[3].lo);
       return;
     }
+    if (ee) {
+      // fixed-point divergence: the stored pairs, at a scale that covers the end vertices' fluxes
+      const uint2 a = __ldg(ex + s[2]);
+      const uint2 b = __ldg(ex + s[3]);
+      const uint2 m = make_uint2(__vmaxu2(a.x, b.x), __vmaxu2(a.y, b.y));
+      const int E[4] = {max((int)(m.x & 0xffff), fx_code(hq[0])), max((int)(m.x >> 16), fx_code(hq[1])),
+                        max((int)(m.y & 0xffff), fx_code(hq[2])), max((int)(m.y >> 16), fx_code(hq[3]))};
+      const int2 p0 = fx_encode(hq[0], E[0], fxL), p1 = fx_encode(hq[1], E[1], fxL);
+      const int2 p2 = fx_encode(hq[2], E[2], fxL), p3 = fx_encode(hq[3], E[3], fxL);
+      int4* o = reinterpret_cast<int4*>(h + (size_t)e * 4);
+      o[0] = make_int4(p0.x, p0.y, p1.x, p1.y);
+      o[1] = make_int4(p2.x, p2.y, p3.x, p3.y);
+      ee[e] = make_uint2((unsigned)E[0] | ((unsigned)E[1] << 16), (unsigned)E[2] | ((unsigned)E[3] << 16));
+      return;
+    }
   }
   st4(h + (size_t)e * 4, hq);
 }
@@ -757,64 +788,13 @@ __global__ void __launch_bounds__(128, EdgeOcc<T>::kMinBlocks) k_edge(int Ef, in
                                               const T* __restrict__ w3, const T* __restrict__ Ua,
                                               T* __restrict__ h, Phys ph, unsigned* err,
                                               uint8_t* __restrict__ dbg, const float* __restrict__ wref,
-                                              const double* __restrict__ FGd) {
+                                              const double* __restrict__ FGd,
+                                              const uint2* __restrict__ ex, uint2* __restrict__ ee, int fxL) {
   edge_body<T>(blockIdx.x * blockDim.x + threadIdx.x, Ef, V, sten, nrm, w5, w3, Ua, h, ph, err, dbg,
-               wref, FGd);
+               wref, FGd, ex, ee, fxL);
 }
 
 // ------------------------------------------------------------------ k_div
-// G lanes per active vertex (G in {1, 2, 4}); lanes stride over the CSR entries; the 12 partial
-// sums are combined by a fixed reduce-scatter over the group (each level halves the values a
-// lane holds), so the result is deterministic and every add is useful.  acc = div(f) -
-// div(f_vis) for the 12 rows; R = -acc.
-template <int G, typename T>
-__device__ __forceinline__ void reduce_scatter12(T* acc, int lane) {
-  // after the loop lane `lane` holds rows base .. base + 12/G - 1 in acc[0 .. 12/G - 1]
-  if (G >= 2) {
-    const int o = G / 2;
-    bool hi = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < 6; ++i) {
-      T keep = hi ? acc[6 + i] : acc[i];
-      T send = hi ? acc[i] : acc[6 + i];
-      acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o, G);
-    }
-  }
-  if (G >= 4) {
-    const int o = G / 4;
-    bool hi = (lane & o) != 0;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-      T keep = hi ? acc[3 + i] : acc[i];
-      T send = hi ? acc[i] : acc[3 + i];
-      acc[i] = keep + __shfl_xor_sync(0xffffffffu, send, o, G);
-    }
-  }
-  if (G >= 8) {
-    // three values left: the lane with bit 0 clear keeps rows 0-1, its partner keeps row 2
-    bool hi = (lane & 1) != 0;
-    T r0 = __shfl_xor_sync(0xffffffffu, acc[0], 1, G);
-    T r1 = __shfl_xor_sync(0xffffffffu, acc[1], 1, G);
-    T r2 = __shfl_xor_sync(0xffffffffu, acc[2], 1, G);
-    if (hi) {
-      acc[0] = acc[2] + r2;
-    } else {
-      acc[0] += r0;
-      acc[1] += r1;
-    }
-  }
-}
-
-// Per-stage arguments of the divergence: out = R (residual) or a*Un + b*(Us + dt*R) (stage).
-struct StageArgs {
-  const double* Us;
-  const double* Un;
-  double* out;
-  int mode;
-  double a, b, dt_fixed;
-  const double* dt_member;   // per-mesh step of a batch (dt_fixed <= 0), or nullptr
-};
-
 // FP32-bulk gather of one vertex's divergence rows over the chunked layout: lane `lane` of
 // the group takes chunks lane, lane + G, ...; per chunk one int4 of indices, 6 (3 for edges)
 // float4 coefficient rows and 4 flux gathers, all independent loads.  Padding entries carry
@@ -896,16 +876,8 @@ __device__ __forceinline__ void div_gather_chunked(
   }
 }
 
-// Finite (not inf or NaN) by the exponent field, on the integer pipe (GB300's FP64 pipe is
-// the limit of the FP64 divergence).
-__device__ __forceinline__ bool finite_bits(double x) {
-  return ((unsigned)(__double_as_longlong(x) >> 52) & 0x7ffu) != 0x7ffu;
-}
-
 // Combines the lanes' partial sums of vertex r (every lane of the warp must call this: the
-// reduce-scatter shuffles over the whole warp) and writes R = -acc, or the Runge-Kutta stage
-// combination a*Un + b*(Us + dt*R), for the rows this lane holds; flags non-finite values and
-// non-positive densities in the error word.
+// reduce-scatter shuffles over the whole warp) and writes the rows this lane then holds.
 template <typename T, int G>
 __device__ __forceinline__ void div_finish(int r, int lane, bool live, T* acc, int V,
                                            const StageArgs& sa, const int32_t* __restrict__ vmem,
@@ -913,45 +885,14 @@ __device__ __forceinline__ void div_finish(int r, int lane, bool live, T* acc, i
                                            double* dt_last, unsigned* err) {
   reduce_scatter12<G>(acc, lane);
   if (!live) return;
-  const double* __restrict__ Us = sa.Us;
-  const double* __restrict__ Un = sa.Un;
-  double* out = sa.out;
-  const int mode = sa.mode;
-  const double a = sa.a, b = sa.b, dt_fixed = sa.dt_fixed;
-  // time step of this vertex's mesh (a batch holds several meshes, each with its own CFL step)
-  const int mem = vmem ? __ldg(vmem + r) : 0;
-  double dt = dt_fixed > 0.0 ? dt_fixed
-               : sa.dt_member ? __ldg(sa.dt_member + mem)
-                              : cfl * __longlong_as_double((long long)dtbits[mem]);
-  if (mode == DIV_STAGE && lane == 0 && dt_last && (r == 0 || (vmem && __ldg(vmem + r - 1) != mem)))
-    dt_last[mem] = dt;
-  // rows held by this lane after the reduce-scatter: base .. base + per - 1
-  int per = G == 1 ? 12 : G == 2 ? 6 : 3;
-  int base = (G >= 2 && (lane & (G / 2)) ? 6 : 0) + (G >= 4 && (lane & (G / 4)) ? 3 : 0);
-  if (G >= 8) {
-    if (lane & 1) { base += 2; per = 1; } else { per = 2; }
-  }
-  unsigned bad = 0;
+  double R[RowShare<G>::kMax];
 #pragma unroll
-  for (int i = 0; i < 12 / (G >= 8 ? 4 : G); ++i) {
-    if (i >= per) break;
-    int k = base + i;
-    double R = -(double)acc[i];
-    size_t idx = (size_t)k * V + r;
-    double o;
-    if (mode == DIV_RESIDUAL) {
-      o = R;
-    } else {
-      // explicit roundings, so that every kernel holding this code (four-launch, staged,
-      // persistent) gives the same bits: one FMA, one multiply, one FMA
-      o = __dmul_rn(b, __fma_rn(dt, R, Us[idx]));
-      if (a != 0.0) o = __fma_rn(a, Un[idx], o);   // the first stage does not read the base state
-    }
-    out[idx] = o;
-    if (!finite_bits(o)) bad |= ERRBIT_NONFINITE;
-    if (mode == DIV_STAGE && k == 0 && !(o > 0.0)) bad |= ERRBIT_POSITIVITY;
-  }
-  if (bad) atomicOr(err, bad);
+  for (int i = 0; i < RowShare<G>::kMax; ++i) R[i] = -(double)acc[i];
+  int row[RowShare<G>::kMax];
+#pragma unroll
+  for (int i = 0; i < RowShare<G>::kMax; ++i) row[i] = RowShare<G>::first(lane) + i;
+  finish_rows<RowShare<G>::kMax>(r, lane, RowShare<G>::count(lane), row, R, V, sa, vmem, dtbits, cfl,
+                                 dt_last, err);
 }
 
 template <typename T, int G, bool VISC>
@@ -1320,49 +1261,7 @@ __global__ void __launch_bounds__(256, 2) k_div_df(int A, int V, int Ef, const i
 constexpr int kStageG = 8;                                  // lanes per vertex
 constexpr int kStageCW = 8;                                 // consumer warps
 constexpr int kStageThreads = 32 * (kStageCW + 1);          // + one producer warp
-constexpr unsigned kMbarPolls = 1u << 22;                   // bound of an mbarrier wait
 static_assert(kStageCW * 32 / kStageG == kStageTileVerts, "one group of lanes per tile vertex");
-
-__device__ __forceinline__ unsigned smem_addr(const void* p) {
-  return (unsigned)__cvta_generic_to_shared(p);
-}
-__device__ __forceinline__ void mbar_init(unsigned long long* bar, unsigned count) {
-  asm volatile("mbarrier.init.shared::cta.b64 [%0], %1;" ::"r"(smem_addr(bar)), "r"(count) : "memory");
-}
-__device__ __forceinline__ void mbar_init_fence() {
-  asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
-}
-__device__ __forceinline__ void mbar_arrive(unsigned long long* bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(smem_addr(bar)) : "memory");
-}
-__device__ __forceinline__ void mbar_expect_tx(unsigned long long* bar, unsigned bytes) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(smem_addr(bar)), "r"(bytes)
-               : "memory");
-}
-// 1D bulk copy global -> shared, completing `bytes` transactions on `bar` (16-byte aligned
-// addresses, size a multiple of 16).
-__device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned bytes,
-                                         unsigned long long* bar) {
-  asm volatile(
-      "cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
-          smem_addr(dst)),
-      "l"(src), "r"(bytes), "r"(smem_addr(bar))
-      : "memory");
-}
-// Bounded wait for the phase of `bar` with parity `parity`; false if the bound ran out.
-__device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity) {
-  const unsigned a = smem_addr(bar);
-  for (unsigned i = 0; i < kMbarPolls; ++i) {
-    unsigned done;
-    asm volatile(
-        "{\n .reg .pred p;\n mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n selp.u32 %0, 1, 0, p;\n}"
-        : "=r"(done)
-        : "r"(a), "r"(parity)
-        : "memory");
-    if (done) return true;
-  }
-  return false;
-}
 
 // Byte layout of one staged tile: two row-pointer slots (vptr and eptr from the 16-byte aligned
 // vertex pb = r0 & ~3 on), index chunks, vertex coefficient chunks (6 float4 rows), viscous
@@ -1798,19 +1697,21 @@ cudaError_t launch_ghost(const DevMesh& m, double* U, const double* base, cudaSt
 cudaError_t launch_vertex(const DevMesh& m, const double* U, const Phys& ph, cudaStream_t s) {
   int nb = blocks(m.V, 256);
   if (m.precision == 0) {
+    const bool fx = m.div_fx && !m.div_df;
     if (m.viscous)
-      k_vertex<double, true><<<nb, 256, 0, s>>>(m.V, U, (double*)m.Ua, (double*)m.FG,
-                                                (double*)m.FGv, ph, nullptr);
+      k_vertex<double, true><<<nb, 256, 0, s>>>(m.V, U, (double*)m.Ua, (double*)m.FG, (double*)m.FGv,
+                                                ph, nullptr, fx ? m.fx.ex : nullptr,
+                                                fx ? m.fx.exv : nullptr, m.fx.L);
     else
       k_vertex<double, false><<<nb, 256, 0, s>>>(m.V, U, (double*)m.Ua, (double*)m.FG, nullptr, ph,
-                                                 nullptr);
+                                                 nullptr, fx ? m.fx.ex : nullptr, nullptr, m.fx.L);
   } else {
     if (m.viscous)
       k_vertex<float, true><<<nb, 256, 0, s>>>(m.V, U, (float*)m.Ua, (float*)m.FG, (float*)m.FGv, ph,
-                                               m.wref);
+                                               m.wref, nullptr, nullptr, 0);
     else
       k_vertex<float, false><<<nb, 256, 0, s>>>(m.V, U, (float*)m.Ua, (float*)m.FG, nullptr, ph,
-                                                m.wref);
+                                                m.wref, nullptr, nullptr, 0);
   }
   return cudaGetLastError();
 }
@@ -1818,15 +1719,18 @@ cudaError_t launch_vertex(const DevMesh& m, const double* U, const Phys& ph, cud
 cudaError_t launch_edge(const DevMesh& m, const Phys& ph, cudaStream_t s) {
   if (m.Ef == 0) return cudaSuccess;
   int nb = blocks(m.Ef, 128);
-  if (m.precision == 0)
+  if (m.precision == 0) {
+    const bool fx = m.div_fx && !m.div_df;
     k_edge<double><<<nb, 128, 0, s>>>(m.Ef, m.V, m.sten, (const double*)m.nrm, (const double*)m.w5,
                                       (const double*)m.w3, (const double*)m.Ua, (double*)m.h, ph,
                                       m.err, m.dbg_branch, nullptr,
-                                      m.div_df ? (const double*)m.FG : nullptr);
-  else
+                                      m.div_df ? (const double*)m.FG : nullptr,
+                                      fx ? m.fx.ex : nullptr, fx ? m.fx.ee : nullptr, m.fx.L);
+  } else {
     k_edge<float><<<nb, 128, 0, s>>>(m.Ef, m.V, m.sten, (const float*)m.nrm, (const float*)m.w5,
                                      (const float*)m.w3, (const float*)m.Ua, (float*)m.h, ph, m.err,
-                                     m.dbg_branch, m.wref, nullptr);
+                                     m.dbg_branch, m.wref, nullptr, nullptr, nullptr, 0);
+  }
   return cudaGetLastError();
 }
 
@@ -1898,6 +1802,8 @@ cudaError_t launch_div(const DevMesh& m, const double* Us, const double* Un, dou
                                          nullptr, (const double*)m.FG, nullptr,
                                          (const float*)m.h, sa, m.vmem, m.dtbits, ph.cfl,
                                          m.dt_last, m.err);
+  } else if (m.precision == 0 && m.div_fx) {
+    return launch_div_fx(m, sa, ph, lanes, s);
   } else if (m.precision == 0) {
     switch (lanes) {
       case 1: div_dispatch<double, 1>(m, sa, ph, s); break;

@@ -51,6 +51,29 @@ constexpr int kStages = 3;
 constexpr int kStageTileBytes = 36 * 1024;
 constexpr int kStagePtrSlot = 160;     // 36 row pointers of a tile (pb .. r1, whole int4s) + slack
 
+// FP64 meshes: the fixed-point form of the divergence (div_fixed.cu).  Rows in chunks of four
+// entries (vptr, eptr count chunks), coefficients as limb pairs with 3 exponents per row (cexp.x,
+// and cexp.y for the viscous rows), fluxes in the stored form of fixed_point.cuh with exponent
+// codes of the 4 components per vertex (ex, exv) and per edge (ee), 16 bits each.
+//
+// Rows go in tiles of `rows` consecutive ones.  A tile's record (rec from head.x on, head.y units of
+// 16 bytes) lists the distinct vertices (head.z) and edges (head.w) that its rows read, and for every
+// entry of its chunks, vertices first, the position in that list as 16 bits.
+struct DivFx {
+  int A = 0, V = 0, Ef = 0;
+  int L = 29;                 // bits of a limb
+  int rows = 16;              // rows per tile: 8 or 16
+  int smem = 0;               // bytes of the tile that stages the most
+  int32_t *vptr = nullptr, *eptr = nullptr;
+  int4 *cv = nullptr, *cvis = nullptr;
+  unsigned char* ce = nullptr;
+  int2* cexp = nullptr;
+  int4 *head = nullptr, *rec = nullptr;
+  uint2 *ex = nullptr, *exv = nullptr, *ee = nullptr;
+  const int4 *FG = nullptr, *FGv = nullptr, *h = nullptr;   // set at launch, with the plain rows:
+  const int32_t *nvptr = nullptr, *nvidx = nullptr, *neptr = nullptr, *neidx = nullptr;
+};
+
 // Device arrays of one mesh in internal numbering.  Coefficient and flux arrays hold elements
 // of the path's bulk precision T (double or float), addressed through void pointers here.
 struct DevMesh {
@@ -114,6 +137,10 @@ struct DevMesh {
   void* cvdf = nullptr;
   void* cedf = nullptr;
   double* sig = nullptr;
+  // FP64 meshes: the divergence in fixed point (div_fx = 1, unless div_df is set); k_vertex and
+  // k_edge then write FG, FGv and h in its stored form
+  int div_fx = 0;
+  DivFx fx;
   // testing aid: when set, k_edge writes per flux edge the Alg. 1 branch it took (bit side*4+q
   // set: the WENO-weighted 3-node value of characteristic component q on side L (0) or R (1))
   uint8_t* dbg_branch = nullptr;
@@ -122,6 +149,16 @@ struct DevMesh {
 };
 
 enum DivMode { DIV_RESIDUAL = 0, DIV_STAGE = 1 };
+
+// Per-stage arguments of the divergence: out = R (residual) or a*Un + b*(Us + dt*R) (stage).
+struct StageArgs {
+  const double* Us;
+  const double* Un;
+  double* out;
+  int mode;
+  double a, b, dt_fixed;
+  const double* dt_member;   // per-mesh step of a batch (dt_fixed <= 0), or nullptr
+};
 
 // Everything the persistent stage kernel reads, passed by value.
 struct KernelArgs {
@@ -156,6 +193,15 @@ cudaError_t launch_edge(const DevMesh& m, const Phys& ph, cudaStream_t s);
 cudaError_t launch_div(const DevMesh& m, const double* Us, const double* Un, double* out,
                        int mode, double a, double b, double dt_fixed, const Phys& ph,
                        int lanes, cudaStream_t s, const double* dt_member = nullptr);
+// Packs the FP64 rows of m into m.fx (allocated, chunk pointers set); *flag (device, zeroed by
+// the caller) becomes nonzero when a row has no fixed-point form.
+cudaError_t pack_div_fx(const DevMesh& m, int* flag, cudaStream_t s);
+// Raises the kernels' shared-memory limit for m.fx.smem (at most kFxSmemMax).
+constexpr int kFxSmallRows = 20000;     // meshes of fewer rows take tiles of 8 rows
+constexpr int kFxSmemMax = 128 * 1024;
+cudaError_t prepare_div_fx(const DevMesh& m);
+cudaError_t launch_div_fx(const DevMesh& m, const StageArgs& sa, const Phys& ph, int lanes,
+                          cudaStream_t s);
 cudaError_t launch_dtmin(const DevMesh& m, const double* U, const Phys& ph, cudaStream_t s);
 // One cooperative launch running ghost refresh (optional), vertex fluxes, edge fluxes and the
 // divergence + stage update of one RK stage, phases separated by bounded grid barriers.

@@ -70,6 +70,8 @@ extern "C" hfd_status hfd_residual_static(hfd_mesh* m, double* U, double* R, voi
                    need, V, Ef, (unsigned)HFD_STATIC_SCRATCH_BYTES);
     return HFD_ERR_ARG;
   }
+  const size_t b_x = round256(V * 2 * sizeof(unsigned)), b_e = round256(Ef * 2 * sizeof(unsigned));
+  const size_t b_fx = b_x + (src.viscous ? b_x : 0) + b_e;
   void* base = nullptr;
   hfd_status st = static_scratch_address(&base);
   if (st != HFD_OK) return st;
@@ -79,6 +81,15 @@ extern "C" hfd_status hfd_residual_static(hfd_mesh* m, double* U, double* R, voi
   d.FG = p + b_ua;
   d.FGv = src.viscous ? p + b_ua + b_fg : nullptr;
   d.h = p + b_ua + b_fg + b_fgv;
+  // the fixed-point divergence needs its exponent words too; a mesh that leaves no room for them
+  // takes the plain FP64 divergence
+  if (d.div_fx && need + b_fx <= HFD_STATIC_SCRATCH_BYTES) {
+    d.fx.ex = reinterpret_cast<uint2*>(p + need);
+    d.fx.ee = reinterpret_cast<uint2*>(p + need + b_x);
+    if (src.viscous) d.fx.exv = reinterpret_cast<uint2*>(p + need + b_x + b_e);
+  } else {
+    d.div_fx = 0;
+  }
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e = hfd::launch_ghost(d, U, U, s);
   if (e == cudaSuccess) e = hfd::launch_vertex(d, U, m->ph, s);
