@@ -245,8 +245,9 @@ hfd_status hfd_steps_profiled(hfd_mesh* mesh, double* U, double dt, int32_t nste
  * output and result as hfd_residual (U in/out for its ghost columns, R out, both 12*nv device
  * arrays in internal order), but the per-call scratch (state copy, vertex and edge fluxes) is a
  * fixed 8 MiB array compiled into the library, held on every GPU that loads the library until
- * the process exits.  That is room for about 32,000 vertices in FP64 (256 bytes each with their
- * ~3 flux edges; above 28,000 the plain FP64 divergence runs, see hfd_mesh_set_fp64_div) or 65,000 in FP32 bulk; larger meshes get HFD_ERR_ARG with the bytes needed.
+ * the process exits, and for FP64 meshes a further scratch set that the mesh allocates when it is
+ * created.  That is room for about 32,000 vertices in FP64 (256 bytes each with their
+ * ~3 flux edges) or 65,000 in FP32 bulk; larger meshes get HFD_ERR_ARG with the bytes needed.
  * Every call looks up the array's device address (cudaGetSymbolAddress, with the mesh's device
  * current), so the address stays right across a cudaDeviceReset; the first call on a device
  * may also load the library's device code there, so make that first call before any stream

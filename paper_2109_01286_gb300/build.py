@@ -38,7 +38,8 @@ def _deps():
     return _sources() + [os.path.join(CSRC, f) for f in ("prep.hpp", "kernels.hpp", "mesh.hpp",
                                                          "adjoint_kernels.cuh", "linalg.hpp",
                                                          "mesh3.hpp", "kernels3d.hpp", "fp_convert.cuh",
-                                                         "fixed_point.cuh", "div_common.cuh", "mbar.cuh")] + \
+                                                         "fixed_point.cuh", "div_common.cuh", "mbar.cuh",
+                                                         "fp64_roots.cuh")] + \
         [os.path.join(INCLUDE, "hfd.h"), os.path.join(INCLUDE, "hfd3d.h"), os.path.abspath(__file__)]
 
 

@@ -191,6 +191,34 @@ hfd_status build_div_fx(hfd_mesh* m, const std::vector<int32_t>& vptr, const std
   int32_t none = 0;
   CK(cudaMemcpy(&none, flag, sizeof none, cudaMemcpyDeviceToHost));
   d.div_fx = none ? 0 : 1;
+  if (!d.div_fx) return HFD_OK;
+  // the edge kernel's 5-node sums in fixed point
+  TRY(dev_alloc(m, (void**)&f.w5f, (size_t)30 * d.Ef * sizeof(int2)));
+  TRY(dev_alloc(m, (void**)&f.w5e, (size_t)d.Ef * sizeof(int2)));
+  CK(hfd::pack_w5_fx(d, flag, nullptr));
+  CK(cudaMemcpy(&none, flag, sizeof none, cudaMemcpyDeviceToHost));
+  if (none) return HFD_OK;
+  TRY(dev_alloc(m, (void**)&f.uf, (size_t)d.V * 12 * sizeof(int2)));
+  TRY(dev_alloc(m, (void**)&f.uc, (size_t)d.V * sizeof(uint4)));
+  return HFD_OK;
+}
+
+// hfd_residual_static's scratch beside its fixed array, for FP64 meshes that the array holds.
+hfd_status static_scratch(hfd_mesh* m) {
+  const DevMesh& d = m->dm;
+  const size_t V = d.V, Ef = d.Ef;
+  if (V * 160 + (d.viscous ? V * 64 : 0) + Ef * 32 > hfd::kStaticScratchBytes) return HFD_OK;
+  TRY(dev_alloc(m, (void**)&m->static_list, Ef * sizeof(int2)));
+  TRY(dev_alloc(m, (void**)&m->static_count, sizeof(int)));
+  if (d.div_fx) {
+    TRY(dev_alloc(m, (void**)&m->static_fx.ex, V * sizeof(uint2)));
+    if (d.viscous) TRY(dev_alloc(m, (void**)&m->static_fx.exv, V * sizeof(uint2)));
+    TRY(dev_alloc(m, (void**)&m->static_fx.ee, Ef * sizeof(uint2)));
+  }
+  if (d.fx.uf) {
+    TRY(dev_alloc(m, (void**)&m->static_fx.uf, V * 12 * sizeof(int2)));
+    TRY(dev_alloc(m, (void**)&m->static_fx.uc, V * sizeof(uint4)));
+  }
   return HFD_OK;
 }
 
@@ -407,7 +435,12 @@ hfd_status upload_streams(hfd_mesh* m, const hfd::Prep& P, const std::vector<int
   TRY(dev_upload(m, &d.cv, cv));
   TRY(dev_upload(m, &d.ce, ce));
   if (P.opts.viscous) TRY(dev_upload(m, &d.cvis, cvis));
-  if (std::is_same<T, double>::value) TRY(build_div_fx(m, vptr, vidx, eptr, eidx));
+  if (std::is_same<T, double>::value) {
+    TRY(dev_alloc(m, (void**)&d.weno_list, (size_t)Ef * sizeof(int2)));
+    TRY(dev_alloc(m, (void**)&d.weno_count, sizeof(int)));
+    TRY(build_div_fx(m, vptr, vidx, eptr, eidx));
+    TRY(static_scratch(m));
+  }
   const size_t V = d.V;
   TRY(dev_alloc(m, &d.Ua, V * 12 * sizeof(T)));
   TRY(dev_alloc(m, &d.FG, V * 8 * sizeof(T)));

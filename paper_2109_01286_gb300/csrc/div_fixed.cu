@@ -422,6 +422,44 @@ cudaError_t pack_div_fx(const DevMesh& m, int* flag, cudaStream_t s) {
   return cudaGetLastError();
 }
 
+// One thread per flux edge: the 30 weights of its sides (side * 15 + node * 3 + {value, x, y}) as limbs.
+// Exponents: one per side for the values, and one offset for the derivatives of both sides.
+__global__ void k_pack_w5(int Ef, const double* __restrict__ w5, int2* w5f, int2* w5e, int* flag) {
+  constexpr int L = 29;
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e >= Ef) return;
+  int ev[2] = {-10000, -10000}, off = -10000;
+  bool bad = false;
+  for (int s = 0; s < 2; ++s) {
+    int ed = -10000;
+    for (int j = 0; j < 15; ++j) {
+      const double w = w5[(size_t)(15 * s + j) * Ef + e];
+      bad |= !isfinite(w);
+      if (j % 3 == 0) ev[s] = max(ev[s], exp_above(w));
+      else ed = max(ed, exp_above(w));
+    }
+    bad |= ev[s] == -10000 || abs(ev[s]) > 500;
+    if (ed != -10000) off = max(off, ed - ev[s]);
+  }
+  if (off == -10000) off = 0;
+  if (bad || abs(off) > 500) {
+    *flag = 1;
+    return;
+  }
+  for (int s = 0; s < 2; ++s)
+    for (int j = 0; j < 15; ++j) {
+      const size_t i = (size_t)(15 * s + j) * Ef + e;
+      w5f[i] = coef_limbs(w5[i], ev[s] + (j % 3 ? off : 0), L);
+    }
+  w5e[e] = make_int2((ev[0] & 0xffff) | (int)((unsigned)ev[1] << 16), off);
+}
+
+cudaError_t pack_w5_fx(const DevMesh& m, int* flag, cudaStream_t s) {
+  if (m.Ef == 0) return cudaSuccess;
+  k_pack_w5<<<(m.Ef + 63) / 64, 64, 0, s>>>(m.Ef, (const double*)m.w5, m.fx.w5f, m.fx.w5e, flag);
+  return cudaGetLastError();
+}
+
 template <int G, int L>
 static const void* fx_kernel(bool visc) {
   return visc ? (const void*)&k_div_fx<G, L, true> : (const void*)&k_div_fx<G, L, false>;

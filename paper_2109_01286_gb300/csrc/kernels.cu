@@ -24,6 +24,7 @@
 
 #include "div_common.cuh"
 #include "fixed_point.cuh"
+#include "fp64_roots.cuh"
 #include "fp_convert.cuh"
 #include "kernels.hpp"
 #include "mbar.cuh"
@@ -192,6 +193,74 @@ __device__ __forceinline__ void roe_flux(const T* wl, const T* wr, T nx, T ny, T
   T fr[4] = {wr[0] * unr, wr[1] * unr + pr * nx, wr[2] * unr + pr * ny, (wr[3] + pr) * unr};
 #pragma unroll
   for (int i = 0; i < 4; ++i) hq[i] = T(0.5) * (fl[i] + fr[i]) - diss[i];
+}
+
+// FP64 forms of the Roe average and flux, arranged for few FP64 instructions (one FP64 warp
+// instruction takes an SM 16 clocks): 120 for a flux with its two states' primitive quantities, where
+// the generic form with the CUDA library's roots takes about 185.
+struct Prim64 {       // of a state w: 1/rho, sqrt(rho), velocity, pressure, E + p, enthalpy
+  double ir, r, u, v, p, Ep, H;
+};
+__device__ __forceinline__ Prim64 prim64(const double* w, double g1) {
+  Prim64 q;
+  const double s = rsqrt64(w[0]);
+  q.ir = s * s;
+  q.r = w[0] * s;
+  q.u = w[1] * q.ir;
+  q.v = w[2] * q.ir;
+  q.p = g1 * fma(-0.5, fma(w[1], q.u, w[2] * q.v), w[3]);
+  q.Ep = w[3] + q.p;
+  q.H = q.Ep * q.ir;
+  return q;
+}
+// Roe-averaged u, v, K = u^2 + v^2, H, c, 1/c of two states (the right state's weight from one
+// reciprocal, the averages from the differences du, dv).
+struct Roe64 {
+  double u, v, K, H, c, ic, du, dv;
+};
+__device__ __forceinline__ Roe64 roe64(const Prim64& L, const Prim64& R, double g1) {
+  Roe64 a;
+  const double f = R.r * rcp64(L.r + R.r);
+  a.du = R.u - L.u;
+  a.dv = R.v - L.v;
+  a.u = fma(f, a.du, L.u);
+  a.v = fma(f, a.dv, L.v);
+  a.H = fma(f, R.H - L.H, L.H);
+  a.K = fma(a.u, a.u, a.v * a.v);
+  const double c2 = g1 * fma(-0.5, a.K, a.H);
+  a.ic = rsqrt64(c2);
+  a.c = c2 * a.ic;
+  return a;
+}
+__device__ __forceinline__ void roe_flux64(const double* wl, const double* wr, const Prim64& L,
+                                           const Prim64& R, double nx, double ny, double g1,
+                                           double harten, double half_inv_harten, double* hq) {
+  const Roe64 a = roe64(L, R, g1);
+  const double qn = fma(a.u, nx, a.v * ny), qt = fma(a.v, nx, -a.u * ny);
+  // wave strengths with the factor 1/2 of the flux, from the primitive jumps (see roe_flux)
+  const double dun = fma(a.du, nx, a.dv * ny), dut = fma(a.dv, nx, -a.du * ny);
+  const double hrho = 0.5 * (L.r * R.r), dp = R.p - L.p, ic2 = a.ic * a.ic;
+  const double hp = 0.25 * (dp * ic2), rc = (hrho * 0.5) * (a.ic * dun);
+  const double a0 = hp - rc, a3 = hp + rc, a1 = fma(0.5, wr[0] - wl[0], -2.0 * hp), a2 = hrho * dut;
+  const double lam[3] = {qn - a.c, qn, qn + a.c};
+  const double del = harten * a.c;
+  double al[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i) {
+    al[i] = fabs(lam[i]);
+    if (al[i] < del) al[i] = fma(lam[i], lam[i], del * del) * (half_inv_harten * a.ic);
+  }
+  const double k0 = al[0] * a0, k1 = al[1] * a1, k2 = al[1] * a2, k3 = al[2] * a3;
+  // R k
+  const double s03 = k0 + k3, s = s03 + k1, d = (k3 - k0) * a.c;
+  const double dx = fma(d, nx, -ny * k2), dy = fma(d, ny, nx * k2);
+  const double unl = fma(L.u, nx, L.v * ny), unr = fma(R.u, nx, R.v * ny);
+  const double ml = wl[0] * unl, mr = wr[0] * unr, ps = L.p + R.p;
+  hq[0] = fma(0.5, ml + mr, -s);
+  hq[1] = fma(0.5, fma(ps, nx, fma(mr, R.u, ml * L.u)), -fma(a.u, s, dx));
+  hq[2] = fma(0.5, fma(ps, ny, fma(mr, R.v, ml * L.v)), -fma(a.v, s, dy));
+  hq[3] = fma(0.5, fma(R.Ep, unr, L.Ep * unl),
+              -fma(a.H, s03, fma(d, qn, fma(0.5 * a.K, k1, qt * k2))));
 }
 
 // Rusanov's (local Lax-Friedrichs) flux along n: the mean of the two normal fluxes minus half
@@ -435,12 +504,41 @@ __device__ __forceinline__ void st_fluxes(double* FG, int v, const double* F, co
   ex[v] = make_uint2((unsigned)E[0] | ((unsigned)E[1] << 16), (unsigned)E[2] | ((unsigned)E[3] << 16));
 }
 
+// What the FP64 vertex kernel writes for the fixed-point kernels (null: not used): codes of the vertex
+// fluxes and the viscous ones, and the nodes' pairs and codes for the edge kernel.
+struct VertexFx {
+  uint2 *ex = nullptr, *exv = nullptr;
+  int4* uf = nullptr;
+  uint4* uc = nullptr;
+  int L = 0;
+  int* count = nullptr;            // zeroed: the edge kernel's list starts empty
+};
+
+__device__ __forceinline__ void st_nodes(int v, const double* w, const VertexFx& fx) {
+  if (!fx.uf) return;
+  constexpr int L = 29;
+  int E[8];
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    E[q] = fx_code(w[q]);
+    E[4 + q] = max(fx_code(w[4 + q]), fx_code(w[8 + q]));
+  }
+  int4* o = fx.uf + 6 * (size_t)v;
+#pragma unroll
+  for (int i = 0; i < 6; ++i) {
+    const int q = 2 * (i & 1) + (i >= 2 ? 4 : 0);
+    const int2 a = fx_encode(w[2 * i], E[q], L), b = fx_encode(w[2 * i + 1], E[q + 1], L);
+    o[i] = make_int4(a.x, a.y, b.x, b.y);
+  }
+  fx.uc[v] = make_uint4((unsigned)E[0] | ((unsigned)E[1] << 16), (unsigned)E[2] | ((unsigned)E[3] << 16),
+                        (unsigned)E[4] | ((unsigned)E[5] << 16), (unsigned)E[6] | ((unsigned)E[7] << 16));
+}
+
 template <typename T, bool VISC>
 __device__ __forceinline__ void vertex_body(int v, int V, const double* __restrict__ U, T* Ua,
                                             T* FG, T* FGv, const Phys& ph, float* wref,
                                             const float* s0f, const double* s0d,
-                                            uint2* ex = nullptr, uint2* exv = nullptr,
-                                            int fxL = 0) {
+                                            const VertexFx& fx = VertexFx()) {
   if (v >= V) return;
   double w[12];
 #pragma unroll
@@ -482,7 +580,8 @@ __device__ __forceinline__ void vertex_body(int v, int V, const double* __restri
     T p = pressure(q, g1);
     T F[4] = {q[1], q[1] * u + p, q[2] * u, (q[3] + p) * u};
     T Gf[4] = {q[2], q[1] * vv, q[2] * vv + p, (q[3] + p) * vv};
-    st_fluxes(FG, v, F, Gf, ex, fxL);
+    st_fluxes(FG, v, F, Gf, fx.ex, fx.L);
+    st_nodes(v, w, fx);
   }
   if (VISC) {   // viscous flux from w, w_x, w_y (Sec. 2.3; chain rule for the primitives)
     double rho = w[0], uu = w[1] / rho, vw = w[2] / rho;
@@ -501,7 +600,7 @@ __device__ __forceinline__ void vertex_body(int v, int V, const double* __restri
     double txy = mu * (uy + vx);
     T Fv[4] = {T(0), T(txx), T(txy), T(uu * txx + vw * txy + ph.kappa * Tx)};
     T Gv[4] = {T(0), T(txy), T(tyy), T(uu * txy + vw * tyy + ph.kappa * Ty)};
-    st_fluxes(FGv, v, Fv, Gv, exv, fxL);
+    st_fluxes(FGv, v, Fv, Gv, fx.exv, fx.L);
   }
 }
 
@@ -519,13 +618,12 @@ __device__ __forceinline__ void block_reference(const double* __restrict__ U, in
 
 template <typename T, bool VISC>
 __global__ void __launch_bounds__(256) k_vertex(int V, const double* __restrict__ U, T* Ua, T* FG,
-                                                T* FGv, Phys ph, float* wref, uint2* ex,
-                                                uint2* exv, int fxL) {
+                                                T* FGv, Phys ph, float* wref, VertexFx fx) {
   __shared__ float s0f[4];
   __shared__ double s0d[4];
   if constexpr (std::is_same<T, float>::value) block_reference(U, V, s0f, s0d);
-  vertex_body<T, VISC>(blockIdx.x * blockDim.x + threadIdx.x, V, U, Ua, FG, FGv, ph, wref, s0f, s0d,
-                       ex, exv, fxL);
+  if (fx.count && blockIdx.x == 0 && threadIdx.x == 0) *fx.count = 0;
+  vertex_body<T, VISC>(blockIdx.x * blockDim.x + threadIdx.x, V, U, Ua, FG, FGv, ph, wref, s0f, s0d, fx);
 }
 
 // ------------------------------------------------------------------ k_edge
@@ -565,16 +663,388 @@ __device__ __forceinline__ void sensor64(T u0, T u1, T u2, T u3, T u4, const Phy
   S = t[0] + t[1] + t[2];
 }
 
+// ---- FP64 edges
+// What the FP64 edge kernel reads and writes beside the plain arrays (null: not used): the vertex
+// fluxes of the folded double-float divergence; the fixed-point divergence's vertex codes and edge
+// codes; the nodes' stored pairs and codes and the 5-node weights in fixed point.
+struct EdgeFx {
+  const double* FGd = nullptr;
+  const uint2* ex = nullptr;
+  uint2* ee = nullptr;
+  const int4* uf = nullptr;        // [V][12] pairs: w, w_x, w_y
+  const uint4* uc = nullptr;       // [V] 8 codes of 16 bits: w (4), w_x and w_y together (4)
+  const int2* w5f = nullptr;       // [30][Ef] limb pairs, order of w5
+  const int2* w5e = nullptr;       // [Ef] exponents (see pack_w5)
+  int L = 0;
+  int2* list = nullptr;            // edges left to k_edge_weno: {edge, components}
+  int* count = nullptr;
+};
+
+// Characteristic values of the conservative values a: rows q_n - c, entropy, shear, q_n + c of the
+// left eigenvectors (left_ev), with the shared parts formed once (13 FP64 instructions).
+struct Left64 {
+  double h0, hu, hv, h3;           // halves of b2, b1 u, b1 v, b1
+  double n0, n1, n2;               // halves of q_n / c, n_x / c, n_y / c
+  double qt, nx, ny;
+  __device__ __forceinline__ Left64(const Roe64& a, double nx_, double ny_, double g1) : nx(nx_), ny(ny_) {
+    h3 = 0.5 * g1 * (a.ic * a.ic);
+    hu = h3 * a.u;
+    hv = h3 * a.v;
+    h0 = 0.5 * h3 * a.K;
+    const double hic = 0.5 * a.ic;
+    n1 = nx * hic;
+    n2 = ny * hic;
+    n0 = fma(a.u, n1, a.v * n2);
+    qt = fma(a.v, nx, -a.u * ny);
+  }
+  __device__ __forceinline__ void apply(const double* a, double* C) const {
+    const double A = fma(h0, a[0], fma(-hu, a[1], fma(-hv, a[2], h3 * a[3])));
+    const double N = fma(n0, a[0], fma(-n1, a[1], -n2 * a[2]));
+    C[0] = A + N;
+    C[1] = fma(-2.0, A, a[0]);
+    C[2] = fma(nx, a[2], fma(-ny, a[1], -qt * a[0]));
+    C[3] = A - N;
+  }
+};
+
+// One side whose sensor asks for the 3-node value in the components `mine` (or must be asked again in
+// FP64): weights and 3-node values of the four components side by side (their chains overlap in the
+// FP64 pipe, whose latency bounds this branch), selected per component.  Returns the components that
+// took the 3-node value; w: the side's state, replaced when there is one.
+__device__ __forceinline__ unsigned weno_side64(const Left64& L, const Roe64& a, unsigned mine, int side,
+                                                const int* s, const double* __restrict__ Ua,
+                                                const double* __restrict__ w3, int Ef, int e, const Phys& ph,
+                                                double* w) {
+  double c[5][4], C[4];
+  L.apply(w, C);
+#pragma unroll
+  for (int j = 0; j < 5; ++j) {
+    double v[4];
+    ld4(Ua + (size_t)(side == 0 ? s[j] : s[5 - j]) * 12, v);
+    L.apply(v, c[j]);
+  }
+  double k3[9];
+#pragma unroll
+  for (int i = 0; i < 9; ++i) k3[i] = ld_stream(w3 + (size_t)(9 * side + i) * Ef + e);
+  unsigned taken = 0;
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    double t[3], S;
+    sensor64(c[0][q], c[1][q], c[2][q], c[3][q], c[4][q], ph, t, S);
+    const bool smooth = (t[0] > ph.sens_lo * S) && (t[0] < ph.sens_hi * S);
+    const double c1 = k3[0] * c[0][q] + k3[1] * c[1][q] + k3[2] * c[2][q];
+    const double c2 = k3[3] * c[1][q] + k3[4] * c[2][q] + k3[5] * c[3][q];
+    const double c3 = k3[6] * c[2][q] + k3[7] * c[3][q] + k3[8] * c[4][q];
+    const double weighted = (t[0] * c1 + t[1] * c2 + t[2] * c3) * rcp64(S);
+    if (((mine >> q) & 1u) && !(smooth && ph.force_branch != 2)) {
+      C[q] = weighted;
+      taken |= 1u << q;
+    }
+  }
+  if (taken) {
+    const double qn = fma(a.u, L.nx, a.v * L.ny), s03 = C[0] + C[3], sum = s03 + C[1], d = (C[3] - C[0]) * a.c;
+    w[0] = sum;
+    w[1] = fma(a.u, sum, fma(d, L.nx, -L.ny * C[2]));
+    w[2] = fma(a.v, sum, fma(d, L.ny, L.nx * C[2]));
+    w[3] = fma(a.H, s03, fma(d, qn, fma(0.5 * a.K, C[1], L.qt * C[2])));
+  }
+  return taken;
+}
+
+// The sensor in FP32 on one component's five differences: the 3-node branch, and the guard band.
+__device__ __forceinline__ void sensor_bits(float u0, float u1, float u2, float u3, float u4, const Phys& ph,
+                                            bool& rough, bool& amb) {
+  float b[3];
+  smoothness(u0, u1, u2, u3, u4, b);
+  const float eps = ph.epsf;
+  float s0 = eps + b[0], s1 = eps + b[1], s2 = eps + b[2];
+  s0 *= s0; s1 *= s1; s2 *= s2;
+  const float t0 = 0.0625f * s1 * s2, t1 = 0.625f * s0 * s2, t2 = 0.3125f * s0 * s1;
+  const float S = t0 + t1 + t2;
+  const float mlo = t0 - ph.sens_lof * S, mhi = ph.sens_hif * S - t0;
+  rough = !(mlo > 0.f && mhi > 0.f);
+  amb = !(fabsf(mlo) > kGuard * S && fabsf(mhi) > kGuard * S);
+}
+
+// Bits (side*4+q) of the sensor in FP32 on the characteristic values cf of the nodes' differences from
+// the tail state: the 3-node branch, and the guard band.
+__device__ __forceinline__ void sensor32(const float (*cf)[4], const Phys& ph, unsigned& rough, unsigned& amb) {
+  rough = amb = 0;
+#pragma unroll
+  for (int side = 0; side < 2; ++side)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      float u0, u1, u2, u3, u4;
+      if (side == 0) { u0 = cf[0][q]; u1 = cf[1][q]; u2 = cf[2][q]; u3 = cf[3][q]; u4 = cf[4][q]; }
+      else           { u0 = cf[5][q]; u1 = cf[4][q]; u2 = cf[3][q]; u3 = cf[2][q]; u4 = cf[1][q]; }
+      bool r, m;
+      sensor_bits(u0, u1, u2, u3, u4, ph, r, m);
+      const unsigned bit = 1u << (side * 4 + q);
+      if (r) rough |= bit;
+      if (m) amb |= bit;
+    }
+  if (ph.force_branch == 1) rough = amb = 0u;                 // every side 5-node
+  else if (ph.force_branch == 2) { rough = 0xffu; amb = 0u; } // every side 3-node WENO
+}
+
+// The 5-node sums of both sides in fixed point (fixed_point.cuh): 120 DFMA, half of the smooth edge's
+// FP64 instructions, become 360 integer multiply-adds.  The nodes' 12 values are stored as pairs with
+// two codes per component (values; derivatives), the weights as limbs with one exponent per side
+// for the values (we.x: 16 bits each) and d = we.y above it for the derivatives (one d for both
+// sides, so that one alignment of the nodes serves both).  All products of component q then share the
+// scale top_q = max(value code, derivative code + d).  Also the sensor's characteristic values of
+// the differences from the tail state: the integer differences, rounded to FP32.  False: some value
+// is not finite, and nothing is written.
+__device__ __forceinline__ bool edge_fixed64(int e, int Ef, const int* s, const EdgeFx& fx, float nx, float ny,
+                                             const Phys& ph, double (*W)[4], float (*cf)[4]) {
+  constexpr int L = 29;
+  uint4 E = __ldg(fx.uc + s[0]);
+#pragma unroll
+  for (int k = 1; k < 6; ++k) {
+    const uint4 c = __ldg(fx.uc + s[k]);
+    E = make_uint4(__vmaxu2(E.x, c.x), __vmaxu2(E.y, c.y), __vmaxu2(E.z, c.z), __vmaxu2(E.w, c.w));
+  }
+  const int2 we = __ldg(fx.w5e + e);
+  const int Ew[4] = {(int)(E.x & 0xffffu), (int)(E.x >> 16), (int)(E.y & 0xffffu), (int)(E.y >> 16)};
+  const int Ed[4] = {(int)(E.z & 0xffffu), (int)(E.z >> 16), (int)(E.w & 0xffffu), (int)(E.w >> 16)};
+  if (max(max(max(Ew[0], Ew[1]), max(Ew[2], Ew[3])), max(max(Ed[0], Ed[1]), max(Ed[2], Ed[3]))) == kFxRaw)
+    return false;
+  int top[4];
+  float unit[4];                                   // FP32 value of 2^-(L-1) of the scale
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    top[q] = max(Ew[q], Ed[q] + we.y);
+    unit[q] = __int_as_float((min(max(top[q] - 1022, -98), 127) - (L - 1) + 127) << 23);
+  }
+  // a node's codes, read again where they are used (L1) rather than held for all six nodes; its shifts;
+  // and the limbs of its four values (g = 0), x derivatives (1) or y derivatives (2)
+  auto shifts = [&](int k, int* dw, int* dd) {
+    uint4 c;
+    asm volatile("ld.global.nc.v4.u32 {%0, %1, %2, %3}, [%4];"
+                 : "=r"(c.x), "=r"(c.y), "=r"(c.z), "=r"(c.w) : "l"(fx.uc + s[k]));
+    dw[0] = top[0] - (int)(c.x & 0xffffu);
+    dw[1] = top[1] - (int)(c.x >> 16);
+    dw[2] = top[2] - (int)(c.y & 0xffffu);
+    dw[3] = top[3] - (int)(c.y >> 16);
+    dd[0] = top[0] - we.y - (int)(c.z & 0xffffu);
+    dd[1] = top[1] - we.y - (int)(c.z >> 16);
+    dd[2] = top[2] - we.y - (int)(c.w & 0xffffu);
+    dd[3] = top[3] - we.y - (int)(c.w >> 16);
+    return ((dw[0] | dw[1] | dw[2] | dw[3] | dd[0] | dd[1] | dd[2] | dd[3]) & ~31) != 0;
+  };
+  auto group = [&](int k, int g, const int* d0, bool far, int* bh, int* bl) {
+    const int4* src = fx.uf + 6 * (size_t)s[k] + 2 * g;
+    const int4 a = __ldg(src), b = __ldg(src + 1);
+    int d[4] = {d0[0], d0[1], d0[2], d0[3]};
+    bh[0] = a.x; bl[0] = a.y; bh[1] = a.z; bl[1] = a.w;
+    bh[2] = b.x; bl[2] = b.y; bh[3] = b.z; bl[3] = b.w;
+    if (far) {
+#pragma unroll
+      for (int q = 0; q < 4; ++q) fx_far(bh[q], bl[q], d[q]);
+    }
+#pragma unroll
+    for (int q = 0; q < 4; ++q) fx_limbs(bh[q], bl[q], d[q], L);
+  };
+  constexpr float kLow = 1.0f / (1 << L);
+  int ih[4], il[4];
+  float Lf[4][4];
+  {
+    int jh[4], jl[4], dw[4], dd[4];
+    bool far = shifts(2, dw, dd);
+    group(2, 0, dw, far, ih, il);
+    far = shifts(3, dw, dd);
+    group(3, 0, dw, far, jh, jl);
+    float fi[4], fj[4], u, v, H, cs;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      fi[q] = fmaf((float)il[q], kLow, (float)ih[q]) * unit[q];
+      fj[q] = fmaf((float)jl[q], kLow, (float)jh[q]) * unit[q];
+    }
+    roe_avg(fi, fj, ph.g1f, u, v, H, cs);
+    left_ev(u, v, cs, nx, ny, ph.g1f, Lf);
+  }
+  long long hh[2][4], x[2][4];
+#pragma unroll
+  for (int i = 0; i < 2; ++i)
+#pragma unroll
+    for (int q = 0; q < 4; ++q) hh[i][q] = x[i][q] = 0;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    int dw[4], dd[4];
+    const bool far = shifts(k, dw, dd);
+#pragma unroll
+    for (int g = 0; g < 3; ++g) {
+      int bh[4], bl[4];
+      group(k, g, g ? dd : dw, far, bh, bl);
+      if (g == 0) {
+        float d[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          d[q] = fmaf((float)(bl[q] - il[q]), kLow, (float)(bh[q] - ih[q])) * unit[q];
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+          cf[k][q] = Lf[q][0] * d[0] + Lf[q][1] * d[1] + Lf[q][2] * d[2] + Lf[q][3] * d[3];
+      }
+#pragma unroll
+      for (int side = 0; side < 2; ++side) {
+        if (k < side || k > 4 + side) continue;
+        const int2 w = __ldg(fx.w5f + (size_t)(15 * side + 3 * (k - side) + g) * Ef + e);
+#pragma unroll
+        for (int q = 0; q < 4; ++q) fx_fma(hh[side][q], x[side][q], w.x, w.y, bh[q], bl[q]);
+      }
+    }
+  }
+#pragma unroll
+  for (int side = 0; side < 2; ++side) {
+    const int ew = side == 0 ? (we.x << 16) >> 16 : we.x >> 16;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const unsigned lo = fx_carry(hh[side][q], x[side][q], L);
+      W[side][q] = fx_to_double(hh[side][q], lo, top[q] + ew + L - 1022 - 2 * (2 * L - 1), L);
+    }
+  }
+  return true;
+}
+
+// Writes an FP64 edge's flux (end vertices i, j) in the form the divergence reads.
+__device__ __forceinline__ void store_flux64(int e, int i, int j, const double* hq, double nx, double ny,
+                                             double* __restrict__ h, const EdgeFx& fx) {
+  if (fx.FGd) {
+    // folded divergence: the flux minus the average of the end vertices' projected fluxes
+    // (O(h^2) on smooth data), as float pairs
+    double fa[8], fb[8];
+    ld8(fx.FGd + (size_t)i * 8, fa);
+    ld8(fx.FGd + (size_t)j * 8, fb);
+    F2x t[4];
+#pragma unroll
+    for (int q = 0; q < 4; ++q)
+      t[q] = split_df(hq[q] - 0.5 * ((fa[q] + fb[q]) * nx + (fa[4 + q] + fb[4 + q]) * ny));
+    float4* o = reinterpret_cast<float4*>(h + (size_t)e * 4);
+    o[0] = make_float4(t[0].hi, t[0].lo, t[1].hi, t[1].lo);
+    o[1] = make_float4(t[2].hi, t[2].lo, t[3].hi, t[3].lo);
+  } else if (fx.ee) {
+    // fixed-point divergence: the stored pairs, at a scale that covers the end vertices' fluxes
+    const uint2 a = __ldg(fx.ex + i), b = __ldg(fx.ex + j);
+    const uint2 m = make_uint2(__vmaxu2(a.x, b.x), __vmaxu2(a.y, b.y));
+    const int E[4] = {max((int)(m.x & 0xffff), fx_code(hq[0])), max((int)(m.x >> 16), fx_code(hq[1])),
+                      max((int)(m.y & 0xffff), fx_code(hq[2])), max((int)(m.y >> 16), fx_code(hq[3]))};
+    const int2 p0 = fx_encode(hq[0], E[0], fx.L), p1 = fx_encode(hq[1], E[1], fx.L);
+    const int2 p2 = fx_encode(hq[2], E[2], fx.L), p3 = fx_encode(hq[3], E[3], fx.L);
+    int4* o = reinterpret_cast<int4*>(h + (size_t)e * 4);
+    o[0] = make_int4(p0.x, p0.y, p1.x, p1.y);
+    o[1] = make_int4(p2.x, p2.y, p3.x, p3.y);
+    fx.ee[e] = make_uint2((unsigned)E[0] | ((unsigned)E[1] << 16), (unsigned)E[2] | ((unsigned)E[3] << 16));
+  } else {
+    st4(h + (size_t)e * 4, hq);
+  }
+}
+
+// The flux of an FP64 edge from its two sides (R16: a side that is not admissible takes its end state).
+__device__ __forceinline__ void flux64(double* wl, double* wr, Prim64 pl, Prim64 pr, const double* wi,
+                                       const double* wj, double nx, double ny, const Phys& ph, double* hq) {
+  if (!(positive_bits(wl[0]) && positive_bits(pl.p))) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) wl[q] = wi[q];
+    pl = prim64(wi, ph.g1);
+  }
+  if (!(positive_bits(wr[0]) && positive_bits(pr.p))) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) wr[q] = wj[q];
+    pr = prim64(wj, ph.g1);
+  }
+  if (ph.flux == 1)
+    rusanov_flux(wl, wr, nx, ny, ph.g1, hq);
+  else
+    roe_flux64(wl, wr, pl, pr, nx, ny, ph.g1, ph.harten, ph.half_inv_harten, hq);
+}
+
+// LIST: edges with a 3-node (or re-decided) component are only listed, for k_edge_weno.
+template <bool LIST>
+__device__ __forceinline__ void edge_body64(int e, int Ef, int V, const int32_t* __restrict__ sten,
+                                            const double* __restrict__ nrm, const double* __restrict__ w5,
+                                            const double* __restrict__ w3, const double* __restrict__ Ua,
+                                            double* __restrict__ h, const Phys& ph, unsigned* err,
+                                            uint8_t* __restrict__ dbg, const EdgeFx& fx) {
+  const double g1 = ph.g1;
+  int s[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) s[k] = chk_idx(ld_stream(sten + (size_t)k * Ef + e), V, err);
+  const double nx = ld_stream(nrm + e), ny = ld_stream(nrm + Ef + e);
+  double wi[4], wj[4];
+  ld4(Ua + (size_t)s[2] * 12, wi);
+  ld4(Ua + (size_t)s[3] * 12, wj);
+  double W[2][4];
+  float cf[6][4];
+  if (!fx.uf || !edge_fixed64(e, Ef, s, fx, d2f_rn(nx), d2f_rn(ny), ph, W, cf)) {
+#pragma unroll
+    for (int r = 0; r < 4; ++r) W[0][r] = W[1][r] = 0.0;
+    // FP32 left eigenvectors at the Roe state of the edge ends (sensor only)
+    float Lf[4][4];
+    {
+      float fi[4], fj[4];
+#pragma unroll
+      for (int q = 0; q < 4; ++q) { fi[q] = d2f_rn(wi[q]); fj[q] = d2f_rn(wj[q]); }
+      float u, v, H, c;
+      roe_avg(fi, fj, ph.g1f, u, v, H, c);
+      left_ev(u, v, c, d2f_rn(nx), d2f_rn(ny), ph.g1f, Lf);
+    }
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      double a[12];
+      ld12(Ua + (size_t)s[k] * 12, a);
+#pragma unroll
+      for (int side = 0; side < 2; ++side) {
+        if (k < side || k > 4 + side) continue;
+        const double* c = w5 + (size_t)(15 * side + 3 * (k - side)) * Ef + e;
+        const double wv = ld_stream(c), wx = ld_stream(c + Ef), wy = ld_stream(c + 2 * (size_t)Ef);
+#pragma unroll
+        for (int r = 0; r < 4; ++r)
+          W[side][r] = fma(wv, a[r], fma(wx, a[4 + r], fma(wy, a[8 + r], W[side][r])));
+      }
+      // end-state differences formed in FP64 and rounded once to FP32
+      float d[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) d[r] = d2f_rn(a[r] - wi[r]);
+#pragma unroll
+      for (int q = 0; q < 4; ++q)
+        cf[k][q] = Lf[q][0] * d[0] + Lf[q][1] * d[1] + Lf[q][2] * d[2] + Lf[q][3] * d[3];
+    }
+  }
+  unsigned rough, amb;
+  sensor32(cf, ph, rough, amb);
+  unsigned taken = 0;
+  if (LIST) {
+    if (rough | amb) {
+      fx.list[atomicAdd(fx.count, 1)] = make_int2(e, (int)(rough | amb));
+      return;
+    }
+  } else if (rough | amb) {
+    const Roe64 a = roe64(prim64(wi, g1), prim64(wj, g1), g1);
+    const Left64 L(a, nx, ny, g1);
+#pragma unroll
+    for (int side = 0; side < 2; ++side) {
+      const unsigned mine = ((rough | amb) >> (side * 4)) & 15u;
+      if (mine) taken |= weno_side64(L, a, mine, side, s, Ua, w3, Ef, e, ph, W[side]) << (side * 4);
+    }
+  }
+  if (dbg) dbg[e] = (uint8_t)taken;
+  double hq[4];
+  flux64(W[0], W[1], prim64(W[0], g1), prim64(W[1], g1), wi, wj, nx, ny, ph, hq);
+  store_flux64(e, s[2], s[3], hq, nx, ny, h, fx);
+}
+
 template <typename T>
 __device__ __forceinline__ void edge_body(int e, int Ef, int V, const int32_t* __restrict__ sten,
                                           const T* __restrict__ nrm, const T* __restrict__ w5,
                                           const T* __restrict__ w3, const T* __restrict__ Ua,
                                           T* __restrict__ h, const Phys& ph, unsigned* err,
                                           uint8_t* __restrict__ dbg, const float* __restrict__ wref,
-                                          const double* __restrict__ FGd = nullptr,
-                                          const uint2* __restrict__ ex = nullptr,
-                                          uint2* __restrict__ ee = nullptr, int fxL = 0) {
+                                          const EdgeFx& fx) {
   if (e >= Ef) return;
+  if constexpr (std::is_same<T, double>::value) {
+    edge_body64<false>(e, Ef, V, sten, nrm, w5, w3, Ua, h, ph, err, dbg, fx);
+    return;
+  }
   const T g1 = phys_g1<T>(ph);
   int s[6];
 #pragma unroll
@@ -740,58 +1210,211 @@ __device__ __forceinline__ void edge_body(int e, int Ef, int V, const int32_t* _
       rusanov_flux(wside[0], wside[1], nx, ny, g1, hq);
     else
       roe_flux(wside[0], wside[1], nx, ny, g1, phys_harten<T>(ph), phys_half_inv_harten<T>(ph), hq);
-    if (FGd) {
-      // folded divergence: the flux minus the average of the end vertices' projected fluxes
-      // (O(h^2) on smooth data), as float pairs
-      double fa[8], fb[8];
-      ld8(FGd + (size_t)s[2] * 8, fa);
-      ld8(FGd + (size_t)s[3] * 8, fb);
-      F2x t[4];
-#pragma unroll
-      for (int q = 0; q < 4; ++q)
-        t[q] = split_df(hq[q] - 0.5 * ((fa[q] + fb[q]) * nx + (fa[4 + q] + fb[4 + q]) * ny));
-      float4* o = reinterpret_cast<float4*>(h + (size_t)e * 4);
-      o[0] = make_float4(t[0].hi, t[0].lo, t[1].hi, t[1].lo);
-      o[1] = make_float4(t[2].hi, t[2].lo, t[3].hi, t[3].lo);
-      return;
-    }
-    if (ee) {
-      // fixed-point divergence: the stored pairs, at a scale that covers the end vertices' fluxes
-      const uint2 a = __ldg(ex + s[2]);
-      const uint2 b = __ldg(ex + s[3]);
-      const uint2 m = make_uint2(__vmaxu2(a.x, b.x), __vmaxu2(a.y, b.y));
-      const int E[4] = {max((int)(m.x & 0xffff), fx_code(hq[0])), max((int)(m.x >> 16), fx_code(hq[1])),
-                        max((int)(m.y & 0xffff), fx_code(hq[2])), max((int)(m.y >> 16), fx_code(hq[3]))};
-      const int2 p0 = fx_encode(hq[0], E[0], fxL), p1 = fx_encode(hq[1], E[1], fxL);
-      const int2 p2 = fx_encode(hq[2], E[2], fxL), p3 = fx_encode(hq[3], E[3], fxL);
-      int4* o = reinterpret_cast<int4*>(h + (size_t)e * 4);
-      o[0] = make_int4(p0.x, p0.y, p1.x, p1.y);
-      o[1] = make_int4(p2.x, p2.y, p3.x, p3.y);
-      ee[e] = make_uint2((unsigned)E[0] | ((unsigned)E[1] << 16), (unsigned)E[2] | ((unsigned)E[3] << 16));
-      return;
-    }
   }
   st4(h + (size_t)e * 4, hq);
 }
 
-// Resident blocks of 128 threads the compiler must allow: 3 for FP64 data (<= 170 registers; an
-// explicit bound of 1 lets it take ~214 and lose a block), 5 for FP32 data (96 registers, an
-// 8-byte spill; 4 percent faster than 4 blocks on the four-quadrant 1024x1024 step).
+// FP32 edges: 5 resident blocks of 128 threads (96 registers, an 8-byte spill; 4 percent faster than 4
+// blocks on the four-quadrant 1024x1024 step).
 template <typename T>
-struct EdgeOcc { static constexpr int kMinBlocks = 3; };
-template <>
-struct EdgeOcc<float> { static constexpr int kMinBlocks = 5; };
-
-template <typename T>
-__global__ void __launch_bounds__(128, EdgeOcc<T>::kMinBlocks) k_edge(int Ef, int V, const int32_t* __restrict__ sten,
+__global__ void __launch_bounds__(128, 5) k_edge(int Ef, int V, const int32_t* __restrict__ sten,
                                               const T* __restrict__ nrm, const T* __restrict__ w5,
                                               const T* __restrict__ w3, const T* __restrict__ Ua,
                                               T* __restrict__ h, Phys ph, unsigned* err,
                                               uint8_t* __restrict__ dbg, const float* __restrict__ wref,
-                                              const double* __restrict__ FGd,
-                                              const uint2* __restrict__ ex, uint2* __restrict__ ee, int fxL) {
+                                              EdgeFx fx) {
   edge_body<T>(blockIdx.x * blockDim.x + threadIdx.x, Ef, V, sten, nrm, w5, w3, Ua, h, ph, err, dbg,
-               wref, FGd, ex, ee, fxL);
+               wref, fx);
+}
+
+// FP64 edges whose two sides take the 5-node branch; the others are listed.
+// 128 registers (some spilled): 4 blocks of 128 an SM; 3 or 5 measured 4 and 2 percent slower.
+__global__ void __launch_bounds__(128, 4) k_edge64(int Ef, int V, const int32_t* __restrict__ sten,
+                                                   const double* __restrict__ nrm,
+                                                   const double* __restrict__ w5,
+                                                   const double* __restrict__ w3,
+                                                   const double* __restrict__ Ua, double* __restrict__ h,
+                                                   Phys ph, unsigned* err, uint8_t* __restrict__ dbg,
+                                                   EdgeFx fx) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < Ef) edge_body64<true>(e, Ef, V, sten, nrm, w5, w3, Ua, h, ph, err, dbg, fx);
+}
+
+// edge_fixed64's 5-node sum of one side's component q (the same integers, so the same bits).
+__device__ __forceinline__ bool lane_fixed64(int e, int Ef, const int* s, int side, int q, const EdgeFx& fx,
+                                             double& W5) {
+  constexpr int L = 29;
+  uint4 c[6], E = make_uint4(0, 0, 0, 0);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    c[k] = __ldg(fx.uc + s[k]);
+    E = make_uint4(__vmaxu2(E.x, c[k].x), __vmaxu2(E.y, c[k].y), __vmaxu2(E.z, c[k].z), __vmaxu2(E.w, c[k].w));
+  }
+  const unsigned all = __vmaxu2(__vmaxu2(E.x, E.y), __vmaxu2(E.z, E.w));
+  if ((all & 0xffffu) == kFxRaw || (all >> 16) == kFxRaw) return false;
+  auto code = [&](const uint4& v, bool deriv) {
+    const unsigned w = deriv ? (q & 2 ? v.w : v.z) : (q & 2 ? v.y : v.x);
+    return (int)(w >> (16 * (q & 1))) & 0xffff;
+  };
+  const int2 we = __ldg(fx.w5e + e);
+  const int top = max(code(E, false), code(E, true) + we.y);
+  long long hh = 0, x = 0;
+#pragma unroll
+  for (int j = 0; j < 5; ++j) {
+    const int v = side == 0 ? s[j] : s[j + 1];
+    const uint4 cj = side == 0 ? c[j] : c[j + 1];
+    const int2* u = reinterpret_cast<const int2*>(fx.uf) + 12 * (size_t)v + q;
+#pragma unroll
+    for (int g = 0; g < 3; ++g) {
+      int2 b = __ldg(u + 4 * g);
+      int d = g ? top - we.y - code(cj, true) : top - code(cj, false);
+      fx_far(b.x, b.y, d);
+      fx_limbs(b.x, b.y, d, L);
+      const int2 w = __ldg(fx.w5f + (size_t)(15 * side + 3 * j + g) * Ef + e);
+      fx_fma(hh, x, w.x, w.y, b.x, b.y);
+    }
+  }
+  const unsigned lo = fx_carry(hh, x, L);
+  const int ew = side == 0 ? (we.x << 16) >> 16 : we.x >> 16;
+  W5 = fx_to_double(hh, lo, top + ew + L - 1022 - 2 * (2 * L - 1), L);
+  return true;
+}
+
+// The value of a lane `o` lanes away (double).
+__device__ __forceinline__ double lane_xor(double x, int o) { return __shfl_xor_sync(0xffffffffu, x, o, 8); }
+__device__ __forceinline__ double lane_of(double x, int l) { return __shfl_sync(0xffffffffu, x, l, 8); }
+
+// The listed edges (ALL: every edge of a small mesh), 8 lanes each: lane side * 4 + q holds component q of one side, so that Alg. 1's FP64
+// chain is an eighth as long.  An SM partition takes 64 clocks for one FP64 warp instruction, and in a
+// warp of the edge kernel a few listed edges would hold up all (690 FP64 instructions for both sides
+// and all components; 240 here).
+template <bool ALL>
+__global__ void __launch_bounds__(128) k_edge_weno(int Ef, int V, const int32_t* __restrict__ sten,
+                                                   const double* __restrict__ nrm,
+                                                   const double* __restrict__ w5,
+                                                   const double* __restrict__ w3,
+                                                   const double* __restrict__ Ua, double* __restrict__ h,
+                                                   Phys ph, unsigned* err, uint8_t* __restrict__ dbg,
+                                                   EdgeFx fx) {
+  const int n = ALL ? Ef : *fx.count;
+  const int l8 = threadIdx.x & 7, side = l8 >> 2, q = l8 & 3;
+  const double g1 = ph.g1;
+  const int groups = gridDim.x * (blockDim.x >> 3);
+  // whole warps run the same number of rounds (shuffles)
+  for (int i0 = (blockIdx.x * blockDim.x + (threadIdx.x & ~31)) >> 3; i0 < n; i0 += groups) {
+    const int i = i0 + ((threadIdx.x & 31) >> 3);
+    const bool live = i < n;
+    const int2 rec = ALL ? make_int2(live ? i : i0, 0) : fx.list[live ? i : i0];
+    const int e = rec.x;
+    bool mine = ((unsigned)rec.y >> l8) & 1u;        // this component, by the FP32 sensor
+    int s[6];
+#pragma unroll
+    for (int k = 0; k < 6; ++k) s[k] = chk_idx(ld_stream(sten + (size_t)k * Ef + e), V, err);
+    const double nx = ld_stream(nrm + e), ny = ld_stream(nrm + Ef + e);
+    double wi[4], wj[4];
+    ld4(Ua + (size_t)s[2] * 12, wi);
+    ld4(Ua + (size_t)s[3] * 12, wj);
+    // this side's nodes (in WENO order: the right side from its far end) and its 5-node sum of component q
+    double c[5][4], W5;
+#pragma unroll
+    for (int j = 0; j < 5; ++j) ld4(Ua + (size_t)(side == 0 ? s[j] : s[5 - j]) * 12, c[j]);
+    if (!fx.uf || !lane_fixed64(e, Ef, s, side, q, fx, W5)) {
+      W5 = 0.0;
+#pragma unroll
+      for (int j = 0; j < 5; ++j) {
+        const double* a = Ua + (size_t)(side == 0 ? s[j] : s[j + 1]) * 12 + q;
+        const double* c5 = w5 + (size_t)(15 * side + 3 * j) * Ef + e;
+        W5 = fma(ld_stream(c5), __ldg(a), fma(ld_stream(c5 + Ef), __ldg(a + 4),
+                 fma(ld_stream(c5 + 2 * (size_t)Ef), __ldg(a + 8), W5)));
+      }
+    }
+    double w[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) w[r] = lane_of(W5, (l8 & 4) + r);
+    auto swap_sides = [&](const Prim64& p) {
+      Prim64 o;
+      o.ir = lane_xor(p.ir, 4); o.r = lane_xor(p.r, 4); o.u = lane_xor(p.u, 4); o.v = lane_xor(p.v, 4);
+      o.p = lane_xor(p.p, 4); o.Ep = lane_xor(p.Ep, 4); o.H = lane_xor(p.H, 4);
+      return o;
+    };
+    if (ALL) {
+      // the edge kernel's FP32 sensor, one component and side per lane
+      float fi[4], fj[4], u, v, H, cs, Lf[4][4], cf[5];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) { fi[r] = d2f_rn(wi[r]); fj[r] = d2f_rn(wj[r]); }
+      roe_avg(fi, fj, ph.g1f, u, v, H, cs);
+      left_ev(u, v, cs, d2f_rn(nx), d2f_rn(ny), ph.g1f, Lf);
+      const double base = q == 0 ? wi[0] : q == 1 ? wi[1] : q == 2 ? wi[2] : wi[3];
+#pragma unroll
+      for (int j = 0; j < 5; ++j) {
+        const float d = d2f_rn((q == 0 ? c[j][0] : q == 1 ? c[j][1] : q == 2 ? c[j][2] : c[j][3]) - base);
+        float sum = 0.f;
+#pragma unroll
+        for (int r = 0; r < 4; ++r) {
+          const float lr = q == 0 ? Lf[0][r] : q == 1 ? Lf[1][r] : q == 2 ? Lf[2][r] : Lf[3][r];
+          sum += lr * __shfl_sync(0xffffffffu, d, (l8 & 4) + r, 8);
+        }
+        cf[j] = sum;
+      }
+      bool rough, amb;
+      sensor_bits(cf[0], cf[1], cf[2], cf[3], cf[4], ph, rough, amb);
+      mine = ph.force_branch == 1 ? false : ph.force_branch == 2 ? true : rough || amb;
+    }
+    unsigned taken = 0;
+    if (__any_sync(0xffffffffu, mine)) {
+      double end[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) end[r] = side == 0 ? wi[r] : wj[r];
+      const Prim64 pe = prim64(end, g1), po = swap_sides(pe);
+      const Roe64 a = roe64(side == 0 ? pe : po, side == 0 ? po : pe, g1);
+      // row q of the left eigenvectors
+      const double h3 = 0.5 * g1 * (a.ic * a.ic), hic = 0.5 * a.ic, n1 = nx * hic, n2 = ny * hic;
+      const double qt = fma(a.v, nx, -a.u * ny);
+      const double sA = q == 1 ? -2.0 : 1.0, sN = q == 0 ? 1.0 : q == 3 ? -1.0 : 0.0;
+      double l[4];
+      l[3] = sA * h3;
+      l[0] = fma(sN, fma(a.u, n1, a.v * n2), fma(l[3], 0.5 * a.K, q == 1 ? 1.0 : 0.0));
+      l[1] = -fma(sN, n1, l[3] * a.u);
+      l[2] = -fma(sN, n2, l[3] * a.v);
+      if (q == 2) { l[0] = -qt; l[1] = -ny; l[2] = nx; l[3] = 0.0; }
+      auto charac = [&](const double* v) { return fma(l[0], v[0], fma(l[1], v[1], fma(l[2], v[2], l[3] * v[3]))); };
+      double u[5];
+#pragma unroll
+      for (int j = 0; j < 5; ++j) u[j] = charac(c[j]);
+      double C = charac(w), t[3], S;
+      sensor64(u[0], u[1], u[2], u[3], u[4], ph, t, S);
+      const bool smooth = (t[0] > ph.sens_lo * S) && (t[0] < ph.sens_hi * S);
+      const bool three = mine && !(smooth && ph.force_branch != 2);
+      double k3[9];
+#pragma unroll
+      for (int k = 0; k < 9; ++k) k3[k] = ld_stream(w3 + (size_t)(9 * side + k) * Ef + e);
+      const double c1 = k3[0] * u[0] + k3[1] * u[1] + k3[2] * u[2];
+      const double c2 = k3[3] * u[1] + k3[4] * u[2] + k3[5] * u[3];
+      const double c3 = k3[6] * u[2] + k3[7] * u[3] + k3[8] * u[4];
+      const double weighted = (t[0] * c1 + t[1] * c2 + t[2] * c3) * rcp64(S);
+      if (three) C = weighted;
+      taken = (__ballot_sync(0xffffffffu, three) >> (threadIdx.x & 24)) & 0xffu;
+      double Cs[4];
+#pragma unroll
+      for (int r = 0; r < 4; ++r) Cs[r] = lane_of(C, (l8 & 4) + r);
+      if ((taken >> (side * 4)) & 15u) {
+        const double qn = fma(a.u, nx, a.v * ny), s03 = Cs[0] + Cs[3], sum = s03 + Cs[1], d = (Cs[3] - Cs[0]) * a.c;
+        w[0] = sum;
+        w[1] = fma(a.u, sum, fma(d, nx, -ny * Cs[2]));
+        w[2] = fma(a.v, sum, fma(d, ny, nx * Cs[2]));
+        w[3] = fma(a.H, s03, fma(d, qn, fma(0.5 * a.K, Cs[1], qt * Cs[2])));
+      }
+    }
+    const Prim64 pw = prim64(w, g1), px = swap_sides(pw);
+    double x[4], hq[4];
+#pragma unroll
+    for (int r = 0; r < 4; ++r) x[r] = lane_xor(w[r], 4);
+    if (side == 0 && q == 0 && live) {
+      flux64(w, x, pw, px, wi, wj, nx, ny, ph, hq);
+      if (dbg) dbg[e] = (uint8_t)taken;
+      store_flux64(e, s[2], s[3], hq, nx, ny, h, fx);
+    }
+  }
 }
 
 // ------------------------------------------------------------------ k_div
@@ -1647,11 +2270,11 @@ __global__ void __launch_bounds__(128) k_stage(KernelArgs ka, StageArgs sa, Phys
   for (int v = tid; v < ka.V; v += stride)
     vertex_body<T, VISC>(v, ka.V, sa.Us, (T*)ka.Ua, (T*)ka.FG, (T*)ka.FGv, ph, ka.wref, s0f, s0d);
   if (!grid_barrier(ka.bar, nb, ka.err, ka.spins)) return;
-  const double* FGd = nullptr;
-  if constexpr (std::is_same<T, double>::value) FGd = ka.div_df ? (const double*)ka.FG : nullptr;
+  EdgeFx fx;
+  if constexpr (std::is_same<T, double>::value) fx.FGd = ka.div_df ? (const double*)ka.FG : nullptr;
   for (int e = tid; e < ka.Ef; e += stride)
     edge_body<T>(e, ka.Ef, ka.V, ka.sten, (const T*)ka.nrm, (const T*)ka.w5, (const T*)ka.w3,
-                 (const T*)ka.Ua, (T*)ka.h, ph, ka.err, nullptr, ka.wref, FGd);
+                 (const T*)ka.Ua, (T*)ka.h, ph, ka.err, nullptr, ka.wref, fx);
   if (!grid_barrier(ka.bar, nb, ka.err, ka.spins)) return;
   if constexpr (std::is_same<T, double>::value) {
     if (ka.div_df) {        // folded double-float divergence, one lane per vertex
@@ -1696,40 +2319,79 @@ cudaError_t launch_ghost(const DevMesh& m, double* U, const double* base, cudaSt
 
 cudaError_t launch_vertex(const DevMesh& m, const double* U, const Phys& ph, cudaStream_t s) {
   int nb = blocks(m.V, 256);
+  VertexFx fx;
   if (m.precision == 0) {
-    const bool fx = m.div_fx && !m.div_df;
+    fx.count = m.weno_count;
+    if (m.div_fx && !m.div_df) {
+      fx.ex = m.fx.ex;
+      fx.exv = m.fx.exv;
+      fx.uf = m.fx.uf;
+      fx.uc = m.fx.uc;
+      fx.L = m.fx.L;
+    }
     if (m.viscous)
       k_vertex<double, true><<<nb, 256, 0, s>>>(m.V, U, (double*)m.Ua, (double*)m.FG, (double*)m.FGv,
-                                                ph, nullptr, fx ? m.fx.ex : nullptr,
-                                                fx ? m.fx.exv : nullptr, m.fx.L);
+                                                ph, nullptr, fx);
     else
       k_vertex<double, false><<<nb, 256, 0, s>>>(m.V, U, (double*)m.Ua, (double*)m.FG, nullptr, ph,
-                                                 nullptr, fx ? m.fx.ex : nullptr, nullptr, m.fx.L);
+                                                 nullptr, fx);
   } else {
     if (m.viscous)
       k_vertex<float, true><<<nb, 256, 0, s>>>(m.V, U, (float*)m.Ua, (float*)m.FG, (float*)m.FGv, ph,
-                                               m.wref, nullptr, nullptr, 0);
+                                               m.wref, fx);
     else
       k_vertex<float, false><<<nb, 256, 0, s>>>(m.V, U, (float*)m.Ua, (float*)m.FG, nullptr, ph,
-                                                m.wref, nullptr, nullptr, 0);
+                                                m.wref, fx);
   }
   return cudaGetLastError();
 }
 
+// FP64 edges: one thread each where they fill the GPU (k_edge64, the edges with a 3-node component
+// listed for k_edge_weno), 8 lanes each in meshes of few edges, whose time is the chain of one warp:
+// 1728 edges 15 us with 8 lanes and 43 us in one pass of one thread each, 7800 edges 28 and 30 us, 12300
+// edges 36 and 30 us.  Before (one kernel, sums in FP64, 341 FP64 instructions a smooth edge): 45 us for
+// 1728 edges, 125 us for 196,600 (now 97 us, 128 FP64 instructions), 330 us for 512,000 (246 us).
+// Threads per block: an SM partition has its own FP64 unit, so blocks of 32 spread a small mesh best.
+constexpr int kEdge8Max = 8000;
+static int edge_threads(int Ef) { return Ef <= 152 * 64 ? 32 : Ef <= 152 * 128 ? 64 : 128; }
+
 cudaError_t launch_edge(const DevMesh& m, const Phys& ph, cudaStream_t s) {
   if (m.Ef == 0) return cudaSuccess;
-  int nb = blocks(m.Ef, 128);
+  EdgeFx fx;
   if (m.precision == 0) {
-    const bool fx = m.div_fx && !m.div_df;
-    k_edge<double><<<nb, 128, 0, s>>>(m.Ef, m.V, m.sten, (const double*)m.nrm, (const double*)m.w5,
-                                      (const double*)m.w3, (const double*)m.Ua, (double*)m.h, ph,
-                                      m.err, m.dbg_branch, nullptr,
-                                      m.div_df ? (const double*)m.FG : nullptr,
-                                      fx ? m.fx.ex : nullptr, fx ? m.fx.ee : nullptr, m.fx.L);
+    if (m.div_df) {
+      fx.FGd = (const double*)m.FG;
+    } else if (m.div_fx) {
+      fx.ex = m.fx.ex;
+      fx.ee = m.fx.ee;
+      fx.L = m.fx.L;
+      fx.uf = m.fx.uf;
+      fx.uc = m.fx.uc;
+      fx.w5f = m.fx.w5f;
+      fx.w5e = m.fx.w5e;
+    }
+    fx.list = m.weno_list;
+    fx.count = m.weno_count;
+    if (m.Ef <= kEdge8Max) {
+      k_edge_weno<true><<<blocks((long long)m.Ef * 8, 32), 32, 0, s>>>(
+          m.Ef, m.V, m.sten, (const double*)m.nrm, (const double*)m.w5, (const double*)m.w3,
+          (const double*)m.Ua, (double*)m.h, ph, m.err, m.dbg_branch, fx);
+      return cudaGetLastError();
+    }
+    const int nt = edge_threads(m.Ef);
+    k_edge64<<<blocks(m.Ef, nt), nt, 0, s>>>(m.Ef, m.V, m.sten, (const double*)m.nrm, (const double*)m.w5,
+                                             (const double*)m.w3, (const double*)m.Ua, (double*)m.h, ph,
+                                             m.err, m.dbg_branch, fx);
+    // the list's length is known on the device only: enough blocks for a full GPU, or the whole mesh
+    const int nb = std::min(blocks((long long)m.Ef * 8, nt), 152 * 4 * (128 / nt));
+    k_edge_weno<false><<<nb, nt, 0, s>>>(m.Ef, m.V, m.sten, (const double*)m.nrm, (const double*)m.w5,
+                                         (const double*)m.w3, (const double*)m.Ua, (double*)m.h, ph,
+                                         m.err, m.dbg_branch, fx);
   } else {
-    k_edge<float><<<nb, 128, 0, s>>>(m.Ef, m.V, m.sten, (const float*)m.nrm, (const float*)m.w5,
-                                     (const float*)m.w3, (const float*)m.Ua, (float*)m.h, ph, m.err,
-                                     m.dbg_branch, m.wref, nullptr, nullptr, nullptr, 0);
+    k_edge<float><<<blocks(m.Ef, 128), 128, 0, s>>>(m.Ef, m.V, m.sten, (const float*)m.nrm,
+                                                    (const float*)m.w5, (const float*)m.w3,
+                                                    (const float*)m.Ua, (float*)m.h, ph, m.err,
+                                                    m.dbg_branch, m.wref, fx);
   }
   return cudaGetLastError();
 }

@@ -70,6 +70,11 @@ struct DivFx {
   int2* cexp = nullptr;
   int4 *head = nullptr, *rec = nullptr;
   uint2 *ex = nullptr, *exv = nullptr, *ee = nullptr;
+  // the edge kernel's 5-node weights [30][Ef] and exponents [Ef], the nodes' pairs [V][12] and codes
+  // [V] (null: the weights have no fixed-point form)
+  int2 *w5f = nullptr, *w5e = nullptr;
+  int4* uf = nullptr;
+  uint4* uc = nullptr;
   const int4 *FG = nullptr, *FGv = nullptr, *h = nullptr;   // set at launch, with the plain rows:
   const int32_t *nvptr = nullptr, *nvidx = nullptr, *neptr = nullptr, *neidx = nullptr;
 };
@@ -141,12 +146,19 @@ struct DevMesh {
   // k_edge then write FG, FGv and h in its stored form
   int div_fx = 0;
   DivFx fx;
+  // FP64 meshes: the edges that k_edge64 leaves to k_edge_weno ({edge, components}) and their number,
+  // which k_vertex zeroes
+  int2* weno_list = nullptr;
+  int* weno_count = nullptr;
   // testing aid: when set, k_edge writes per flux edge the Alg. 1 branch it took (bit side*4+q
   // set: the WENO-weighted 3-node value of characteristic component q on side L (0) or R (1))
   uint8_t* dbg_branch = nullptr;
   void* FGv = nullptr;
   void* h = nullptr;
 };
+
+// Bytes of hfd_residual_static's array (noalloc.cu).
+constexpr size_t kStaticScratchBytes = 8u << 20;
 
 enum DivMode { DIV_RESIDUAL = 0, DIV_STAGE = 1 };
 
@@ -193,8 +205,9 @@ cudaError_t launch_edge(const DevMesh& m, const Phys& ph, cudaStream_t s);
 cudaError_t launch_div(const DevMesh& m, const double* Us, const double* Un, double* out,
                        int mode, double a, double b, double dt_fixed, const Phys& ph,
                        int lanes, cudaStream_t s, const double* dt_member = nullptr);
-// Packs the FP64 rows of m into m.fx (allocated, chunk pointers set); *flag (device, zeroed by
-// the caller) becomes nonzero when a row has no fixed-point form.
+// Packs the FP64 rows (5-node weights) of m into m.fx (allocated, chunk pointers set); *flag
+// (device, zeroed by the caller) becomes nonzero when one has no fixed-point form.
+cudaError_t pack_w5_fx(const DevMesh& m, int* flag, cudaStream_t s);
 cudaError_t pack_div_fx(const DevMesh& m, int* flag, cudaStream_t s);
 // Raises the kernels' shared-memory limit for m.fx.smem (at most kFxSmemMax).
 constexpr int kFxSmallRows = 20000;     // meshes of fewer rows take tiles of 8 rows

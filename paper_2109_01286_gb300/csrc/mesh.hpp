@@ -41,6 +41,9 @@ struct hfd_mesh {
   double* U2 = nullptr;
   double* Uin = nullptr;                // end-to-end staging (input order)
   double* Uint = nullptr;               // end-to-end staging (internal order)
+  hfd::DivFx static_fx;                 // hfd_residual_static: its own codes, pairs and edge list
+  int2* static_list = nullptr;
+  int* static_count = nullptr;
   cudaStream_t cap = nullptr;           // private stream used for graph capture
   std::map<std::pair<const double*, double>, GraphEntry> graphs;
   hfd_mesh_stats stats{};

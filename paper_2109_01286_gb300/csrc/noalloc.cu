@@ -8,7 +8,7 @@
 // up and then evaluates residuals without any further allocation.
 //
 // The scratch -- the AoS copy of the state, the vertex fluxes and the edge fluxes -- lives in
-// g_static_scratch below, HFD_STATIC_SCRATCH_BYTES per device.  Every GPU that loads the
+// g_static_scratch below, kStaticScratchBytes per device.  Every GPU that loads the
 // library holds that array until the process exits.  All calls on a device share the one
 // array: calls whose work overlaps on the GPU (different streams, or different host threads)
 // race on it and must be serialised by the caller.  Each call fully overwrites the parts of
@@ -22,9 +22,8 @@
 #include "mesh.hpp"
 #include "prep.hpp"
 
-#define HFD_STATIC_SCRATCH_BYTES (8u << 20)
 
-static __device__ __align__(256) unsigned char g_static_scratch[HFD_STATIC_SCRATCH_BYTES];
+static __device__ __align__(256) unsigned char g_static_scratch[hfd::kStaticScratchBytes];
 
 namespace {
 
@@ -64,14 +63,12 @@ extern "C" hfd_status hfd_residual_static(hfd_mesh* m, double* U, double* R, voi
   const size_t b_ua = round256(V * 12 * T), b_fg = round256(V * 8 * T);
   const size_t b_fgv = src.viscous ? round256(V * 8 * T) : 0, b_h = round256(Ef * 4 * T);
   const size_t need = b_ua + b_fg + b_fgv + b_h;
-  if (need > HFD_STATIC_SCRATCH_BYTES) {
+  if (need > hfd::kStaticScratchBytes) {
     hfd::set_error("hfd_residual_static: mesh needs %zu bytes of scratch (%zu vertices, %zu flux "
                    "edges), above the fixed %u-byte array; use hfd_residual",
-                   need, V, Ef, (unsigned)HFD_STATIC_SCRATCH_BYTES);
+                   need, V, Ef, (unsigned)hfd::kStaticScratchBytes);
     return HFD_ERR_ARG;
   }
-  const size_t b_x = round256(V * 2 * sizeof(unsigned)), b_e = round256(Ef * 2 * sizeof(unsigned));
-  const size_t b_fx = b_x + (src.viscous ? b_x : 0) + b_e;
   void* base = nullptr;
   hfd_status st = static_scratch_address(&base);
   if (st != HFD_OK) return st;
@@ -81,15 +78,14 @@ extern "C" hfd_status hfd_residual_static(hfd_mesh* m, double* U, double* R, voi
   d.FG = p + b_ua;
   d.FGv = src.viscous ? p + b_ua + b_fg : nullptr;
   d.h = p + b_ua + b_fg + b_fgv;
-  // the fixed-point divergence needs its exponent words too; a mesh that leaves no room for them
-  // takes the plain FP64 divergence
-  if (d.div_fx && need + b_fx <= HFD_STATIC_SCRATCH_BYTES) {
-    d.fx.ex = reinterpret_cast<uint2*>(p + need);
-    d.fx.ee = reinterpret_cast<uint2*>(p + need + b_x);
-    if (src.viscous) d.fx.exv = reinterpret_cast<uint2*>(p + need + b_x + b_e);
-  } else {
-    d.div_fx = 0;
-  }
+  // the FP64 kernels' further scratch is the mesh's, allocated with it for these calls alone
+  d.fx.ex = m->static_fx.ex;
+  d.fx.exv = m->static_fx.exv;
+  d.fx.ee = m->static_fx.ee;
+  d.fx.uf = m->static_fx.uf;
+  d.fx.uc = m->static_fx.uc;
+  d.weno_list = m->static_list;
+  d.weno_count = m->static_count;
   cudaStream_t s = (cudaStream_t)stream;
   cudaError_t e = hfd::launch_ghost(d, U, U, s);
   if (e == cudaSuccess) e = hfd::launch_vertex(d, U, m->ph, s);

@@ -110,3 +110,21 @@ def test_nonfinite_fluxes_reach_the_same_rows(value):
     assert not torch.isfinite(b).all() and torch.isfinite(b).any()
     with pytest.raises(pkg.HfdError):
         mesh.check()
+
+
+def test_edge_kernels_of_small_and_large_meshes_give_the_same_bits():
+    """A mesh of few edges gives every edge 8 lanes; a batch of copies has one thread an edge and lists
+    the edges with a 3-node component.  Sums are exact and the rest is the same code: equal bits."""
+    pkg = _pkg()
+    m = synth.jittered_grid(40, 33, 4.0, 3.3, seed=1)          # 3,960 edges; shocked part of the box
+    U = synth.isentropic_vortex(m, center=(2.0, 1.6))
+    U[:4, np.hypot(m["x"] - 1.0, m["y"] - 1.0) < 0.6] *= 2.0
+    prep = pkg.Prep(m)
+    one, many = prep.upload(), pkg.Prep.concat([prep] * 4).upload()
+    a = one.import_state(torch.from_numpy(U).cuda())
+    b = many.import_state(torch.from_numpy(np.concatenate([U] * 4, 1)).cuda())
+    assert one.edge_branches(a.clone()).any() and not one.edge_branches(a.clone()).all()
+    Ra = one.export_state(one.residual(a))
+    Rb = many.export_state(many.residual(b))
+    for k in range(4):
+        assert torch.equal(Rb[:, k * len(m["x"]):(k + 1) * len(m["x"])], Ra)
