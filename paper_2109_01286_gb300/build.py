@@ -39,7 +39,7 @@ def _deps():
                                                          "adjoint_kernels.cuh", "linalg.hpp",
                                                          "mesh3.hpp", "kernels3d.hpp", "fp_convert.cuh",
                                                          "fixed_point.cuh", "div_common.cuh", "mbar.cuh",
-                                                         "fp64_roots.cuh")] + \
+                                                         "fp64_roots.cuh", "edge64.cuh")] + \
         [os.path.join(INCLUDE, "hfd.h"), os.path.join(INCLUDE, "hfd3d.h"), os.path.abspath(__file__)]
 
 

@@ -26,6 +26,7 @@
 #include <vector>
 
 #include "adjoint_kernels.cuh"
+#include "edge64.cuh"
 #include "kernels.hpp"
 #include "mesh.hpp"
 #include "prep.hpp"
@@ -74,37 +75,51 @@ __device__ __forceinline__ void right_apply_d(double u, double v, double H, doub
   w[3] = (H - c * qn) * C[0] + 0.5 * (u * u + v * v) * C[1] + qt * C[2] + (H + c * qn) * C[3];
 }
 
-__device__ __forceinline__ double press(const double* w, double g1) {
-  return g1 * (w[3] - 0.5 * (w[1] * w[1] + w[2] * w[2]) / w[0]);
+// rho > 0 and p > 0: p rho / (gamma - 1) = E rho - |m|^2 / 2.
+__device__ __forceinline__ bool admissible_d(const double* w) {
+  return w[0] > 0.0 && fma(w[3], w[0], -0.5 * fma(w[1], w[1], w[2] * w[2])) > 0.0;
 }
 
-// Shared front of the edge reverse pass: hbar = -(D^T mu) at the edge, the stencil, the end
+// FP64 5-node sums of both sides in conservative variables (the forward interpolation).
+__device__ __forceinline__ void adj_edge_w5(int e, int Ef, const int* s, const double* __restrict__ w5,
+                                            const double* __restrict__ Ua, double (*W5)[4]) {
+  // ---- forward in FP64: 5-node conservative sums, sides with re-decided / 3-node components
+  for (int side = 0; side < 2; ++side)
+    for (int r = 0; r < 4; ++r) W5[side][r] = 0.0;
+  for (int k = 0; k < 6; ++k) {
+    const double* a = Ua + (size_t)s[k] * 12;
+    for (int side = 0; side < 2; ++side) {
+      int j = k - side;
+      if (j < 0 || j > 4) continue;
+      double wv = w5[(size_t)(15 * side + 3 * j) * Ef + e];
+      double wx = w5[(size_t)(15 * side + 3 * j + 1) * Ef + e];
+      double wy = w5[(size_t)(15 * side + 3 * j + 2) * Ef + e];
+      for (int r = 0; r < 4; ++r) W5[side][r] += wv * a[r] + wx * a[4 + r] + wy * a[8 + r];
+    }
+  }
+}
+
+// Shared front of the edge reverse pass: hbar at the edge (k_adj_hbar), the stencil, the end
 // states and the FP32 sensor decisions exactly as k_edge takes them (bit side*4+q of `rough`:
 // 3-node branch; of `amb`: inside the guard band, re-decided in FP64).
 __device__ __forceinline__ void adj_edge_front(
-    int e, int Ef, int V, const int32_t* __restrict__ sten, const double* __restrict__ nrm,
-    const double* __restrict__ Ua, const int32_t* __restrict__ eptr,
-    const double* __restrict__ ce, const int32_t* __restrict__ te_ptr,
-    const int32_t* __restrict__ te_row, const int32_t* __restrict__ te_pos,
-    const double* __restrict__ mu, const Phys& ph, double* hb, int* s, double& nx, double& ny,
-    double* wi, double* wj, unsigned& rough, unsigned& amb) {
+    int e, int Ef, const int32_t* __restrict__ sten, const double* __restrict__ nrm,
+    const double* __restrict__ w5, const double* __restrict__ Ua, const double* __restrict__ hbar,
+    const Phys& ph, const EdgeFx& fx, double* hb, int* s, double& nx, double& ny, double* wi, double* wj,
+    double (*W5)[4], unsigned& rough, unsigned& amb) {
   const double g1 = ph.g1;
-  // ---- hbar = -(D^T mu)_e
-  for (int q = 0; q < 4; ++q) hb[q] = 0.0;
-  for (int t = te_ptr[e]; t < te_ptr[e + 1]; ++t) {
-    int r = te_row[t], j = te_pos[t];
-    int m0 = eptr[r], M = eptr[r + 1] - m0;
-    const double* d = ce + 3 * (size_t)m0;
-    double d0 = d[j], dx = d[M + j], dy = d[2 * M + j];
-    for (int q = 0; q < 4; ++q)
-      hb[q] -= d0 * mu[(size_t)q * V + r] + dx * mu[(size_t)(4 + q) * V + r] +
-               dy * mu[(size_t)(8 + q) * V + r];
-  }
+  for (int q = 0; q < 4; ++q) hb[q] = hbar[(size_t)e * 4 + q];
   for (int k = 0; k < 6; ++k) s[k] = sten[(size_t)k * Ef + e];
   nx = nrm[e];
   ny = nrm[Ef + e];
   for (int r = 0; r < 4; ++r) { wi[r] = Ua[(size_t)s[2] * 12 + r]; wj[r] = Ua[(size_t)s[3] * 12 + r]; }
-  // ---- forward: FP32 sensor exactly as k_edge
+  // ---- forward: the 5-node sums and the FP32 sensor exactly as the edge kernel takes them
+  float cf6[6][4];
+  if (fx.uf && edge_fixed64(e, Ef, s, fx, (float)nx, (float)ny, ph, W5, cf6)) {
+    sensor32(cf6, ph, rough, amb);
+    return;
+  }
+  adj_edge_w5(e, Ef, s, w5, Ua, W5);
   rough = 0;
   amb = 0;
   {
@@ -152,54 +167,29 @@ __device__ __forceinline__ void adj_edge_front(
   }
 }
 
-// FP64 5-node sums of both sides in conservative variables (the forward interpolation).
-__device__ __forceinline__ void adj_edge_w5(int e, int Ef, const int* s, const double* __restrict__ w5,
-                                            const double* __restrict__ Ua, double (*W5)[4]) {
-  // ---- forward in FP64: 5-node conservative sums, sides with re-decided / 3-node components
-  for (int side = 0; side < 2; ++side)
-    for (int r = 0; r < 4; ++r) W5[side][r] = 0.0;
-  for (int k = 0; k < 6; ++k) {
-    const double* a = Ua + (size_t)s[k] * 12;
-    for (int side = 0; side < 2; ++side) {
-      int j = k - side;
-      if (j < 0 || j > 4) continue;
-      double wv = w5[(size_t)(15 * side + 3 * j) * Ef + e];
-      double wx = w5[(size_t)(15 * side + 3 * j + 1) * Ef + e];
-      double wy = w5[(size_t)(15 * side + 3 * j + 2) * Ef + e];
-      for (int r = 0; r < 4; ++r) W5[side][r] += wv * a[r] + wx * a[4 + r] + wy * a[8 + r];
-    }
-  }
-}
-
 // One thread per flux edge, edges whose sides both took the 5-node branch: the reverse of the
 // Roe flux and of the 5-node sums; each node's 12 sensitivities are formed in registers and
 // stored once to Ge[e][72].  Edges with a 3-node or re-decided component are appended to
 // `list` for k_adj_edge_full (the order of the list does not matter: each edge writes only
 // its own Ge row).
 __global__ void __launch_bounds__(128, 3) k_adj_edge(
-    int Ef, int V, const int32_t* __restrict__ sten, const double* __restrict__ nrm,
+    int Ef, const int32_t* __restrict__ sten, const double* __restrict__ nrm,
     const double* __restrict__ w5, const double* __restrict__ w3, const double* __restrict__ Ua,
-    const int32_t* __restrict__ eptr, const double* __restrict__ ce,
-    const int32_t* __restrict__ te_ptr, const int32_t* __restrict__ te_row,
-    const int32_t* __restrict__ te_pos, const double* __restrict__ mu, double* __restrict__ Ge,
-    Phys ph, int32_t* __restrict__ list, int32_t* __restrict__ count) {
+    const double* __restrict__ hbar, double* __restrict__ Ge, Phys ph, EdgeFx fx, int32_t* __restrict__ list, int32_t* __restrict__ count) {
   int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= Ef) return;
   double hb[4], nx, ny, wi[4], wj[4];
   int s[6];
   unsigned rough, amb;
-  adj_edge_front(e, Ef, V, sten, nrm, Ua, eptr, ce, te_ptr, te_row, te_pos, mu, ph, hb, s, nx, ny,
-                 wi, wj, rough, amb);
+  double W5[2][4];
+  adj_edge_front(e, Ef, sten, nrm, w5, Ua, hbar, ph, fx, hb, s, nx, ny, wi, wj, W5, rough, amb);
   if (rough | amb) {
     list[atomicAdd(count, 1)] = e;
     return;
   }
   double* ge = Ge + (size_t)e * 72;
-  const double g1 = ph.g1;
-  double W5[2][4];
-  adj_edge_w5(e, Ef, s, w5, Ua, W5);
-  bool fb0 = !(W5[0][0] > 0.0) || !(press(W5[0], g1) > 0.0);
-  bool fb1 = !(W5[1][0] > 0.0) || !(press(W5[1], g1) > 0.0);
+  bool fb0 = !admissible_d(W5[0]);
+  bool fb1 = !admissible_d(W5[1]);
   double wl[4], wr[4];
 #pragma unroll
   for (int r = 0; r < 4; ++r) {
@@ -256,24 +246,19 @@ __global__ void __launch_bounds__(128, 3) k_adj_edge(
 // reverse of Alg. 1 and the Roe flux; writes the sensitivities of the 12 values of the 6
 // stencil nodes to Ge[e][72].
 __global__ void __launch_bounds__(128) k_adj_edge_full(
-    int Ef, int V, const int32_t* __restrict__ sten, const double* __restrict__ nrm,
+    int Ef, const int32_t* __restrict__ sten, const double* __restrict__ nrm,
     const double* __restrict__ w5, const double* __restrict__ w3, const double* __restrict__ Ua,
-    const int32_t* __restrict__ eptr, const double* __restrict__ ce,
-    const int32_t* __restrict__ te_ptr, const int32_t* __restrict__ te_row,
-    const int32_t* __restrict__ te_pos, const double* __restrict__ mu, double* __restrict__ Ge,
-    Phys ph, const int32_t* __restrict__ list, const int32_t* __restrict__ count) {
+    const double* __restrict__ hbar, double* __restrict__ Ge, Phys ph, EdgeFx fx, const int32_t* __restrict__ list, const int32_t* __restrict__ count) {
   int li = blockIdx.x * blockDim.x + threadIdx.x;
   if (li >= *count) return;
   int e = list[li];
   double hb[4], nx, ny, wi[4], wj[4];
   int s[6];
   unsigned rough, amb;
-  adj_edge_front(e, Ef, V, sten, nrm, Ua, eptr, ce, te_ptr, te_row, te_pos, mu, ph, hb, s, nx, ny,
-                 wi, wj, rough, amb);
+  double W5[2][4];
+  adj_edge_front(e, Ef, sten, nrm, w5, Ua, hbar, ph, fx, hb, s, nx, ny, wi, wj, W5, rough, amb);
   double* ge = Ge + (size_t)e * 72;
   const double g1 = ph.g1;
-  double W5[2][4];
-  adj_edge_w5(e, Ef, s, w5, Ua, W5);
   for (int i = 0; i < 72; ++i) ge[i] = 0.0;
   adj::RoeState rs;
   double L[4][4];
@@ -317,8 +302,8 @@ __global__ void __launch_bounds__(128) k_adj_edge_full(
     right_apply_d(rs.u, rs.v, rs.H, rs.c, nx, ny, C[side], wside[side]);
   }
   bool fb[2];
-  fb[0] = !(wside[0][0] > 0.0) || !(press(wside[0], g1) > 0.0);
-  fb[1] = !(wside[1][0] > 0.0) || !(press(wside[1], g1) > 0.0);
+  fb[0] = !admissible_d(wside[0]);
+  fb[1] = !admissible_d(wside[1]);
   if (fb[0]) for (int r = 0; r < 4; ++r) wside[0][r] = wi[r];
   if (fb[1]) for (int r = 0; r < 4; ++r) wside[1][r] = wj[r];
   // ---- reverse
@@ -416,58 +401,143 @@ __global__ void __launch_bounds__(128) k_adj_edge_full(
   }
 }
 
-// One thread per vertex: vertex-flux part of (dR/dU)^T mu, the edge sensitivities of the
+// The transposed gathers read mu with its 12 rows side by side (96 bytes: three sectors of a row, where
+// the 12 x V layout takes 12) and the divergence coefficients in the order of the transposed lists.
+// Before, the edge kernel gathered both from the forward layout and summed the 5-node values in FP64:
+// 230 us for 76,800 edges, now 5 (this copy) + 36 (k_adj_hbar) + 128 us; the vertex kernel 100 us for
+// 25,600 vertices, now 73.  The FP64 pipe bounds all three (177, 400 and 800 FP64 instructions an edge
+// or vertex), so more lanes cost more in reductions than they hide: 1, 2 and 4 lanes measured 36, 42 and
+// 54 us for the edges, 89, 72 and 89 us for the vertices.
+__global__ void __launch_bounds__(256) k_adj_aos(int V, const double* __restrict__ mu, double* __restrict__ mua) {
+  const int v = blockIdx.x * blockDim.x + threadIdx.x;
+  if (v >= V) return;
+  double2* o = reinterpret_cast<double2*>(mua + (size_t)v * 12);
+#pragma unroll
+  for (int i = 0; i < 6; ++i) o[i] = make_double2(mu[(size_t)(2 * i) * V + v], mu[(size_t)(2 * i + 1) * V + v]);
+}
+
+// Coefficients in transposed order: entry t of a list names row trow[t] and its entry tpos[t]; out
+// holds the row's `rows` coefficients of that entry side by side.
+__global__ void k_adj_gather_coef(int n, int rows, const int32_t* __restrict__ trow,
+                                  const int32_t* __restrict__ tpos, const int32_t* __restrict__ ptr,
+                                  const double* __restrict__ coef, double* __restrict__ out) {
+  const int t = blockIdx.x * blockDim.x + threadIdx.x;
+  if (t >= n) return;
+  const int r = trow[t], p0 = ptr[r], N = ptr[r + 1] - p0;
+  for (int k = 0; k < rows; ++k) out[(size_t)t * rows + k] = coef[(size_t)rows * p0 + (size_t)k * N + tpos[t]];
+}
+
+constexpr int kAdjLanes = 2, kAdjEdgeLanes = 1;
+
+// Sum of x over the G lanes of a group, in a fixed order.
+template <int G>
+__device__ __forceinline__ double group_sum(double x) {
+#pragma unroll
+  for (int o = 1; o < G; o <<= 1) x += __shfl_xor_sync(0xffffffffu, x, o, G);
+  return x;
+}
+
+// hbar = -(D^T mu) at every flux edge: kAdjEdgeLanes lanes take the rows that read it in turn.
+__global__ void __launch_bounds__(128) k_adj_hbar(int Ef, const int32_t* __restrict__ te_ptr,
+                                                  const int32_t* __restrict__ te_row,
+                                                  const double* __restrict__ te_coef,
+                                                  const double* __restrict__ mua, double* __restrict__ hbar) {
+  constexpr int G = kAdjEdgeLanes;
+  const int gt = blockIdx.x * blockDim.x + threadIdx.x, e = gt / G, lane = gt % G;
+  const bool live = e < Ef;
+  double h[4] = {0.0, 0.0, 0.0, 0.0};
+  const int t1 = live ? te_ptr[e + 1] : 0;
+  for (int t = live ? te_ptr[e] + lane : 0; t < t1; t += G) {
+    const double2* m = reinterpret_cast<const double2*>(mua + (size_t)te_row[t] * 12);
+    const double* c = te_coef + (size_t)3 * t;
+    const double d0 = c[0], dx = c[1], dy = c[2];
+    const double2 a = m[0], b = m[1], ax = m[2], bx = m[3], ay = m[4], by = m[5];
+    h[0] = fma(-d0, a.x, fma(-dx, ax.x, fma(-dy, ay.x, h[0])));
+    h[1] = fma(-d0, a.y, fma(-dx, ax.y, fma(-dy, ay.y, h[1])));
+    h[2] = fma(-d0, b.x, fma(-dx, bx.x, fma(-dy, by.x, h[2])));
+    h[3] = fma(-d0, b.y, fma(-dx, bx.y, fma(-dy, by.y, h[3])));
+  }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) h[q] = group_sum<G>(h[q]);
+  if (live && lane == 0) {
+    reinterpret_cast<double2*>(hbar + (size_t)e * 4)[0] = make_double2(h[0], h[1]);
+    reinterpret_cast<double2*>(hbar + (size_t)e * 4)[1] = make_double2(h[2], h[3]);
+  }
+}
+
+// kAdjLanes lanes per vertex: vertex-flux part of (dR/dU)^T mu, the edge sensitivities of the
 // stencils this vertex belongs to, then out = cx X + cy Y + cz Z + cg g.
+template <bool VISC>
 __global__ void __launch_bounds__(128) k_adj_vertex(
-    int V, const double* __restrict__ Us, const int32_t* __restrict__ vptr,
-    const double* __restrict__ cv, const double* __restrict__ cvis,
-    const int32_t* __restrict__ tv_ptr,
-    const int32_t* __restrict__ tv_row, const int32_t* __restrict__ tv_pos,
-    const int32_t* __restrict__ ts_ptr, const int32_t* __restrict__ ts_ent,
-    const double* __restrict__ mu, const double* __restrict__ Ge, double* out, double cx,
-    const double* X, double cy, const double* Y, double cz, const double* Z, double cg,
-    Phys ph) {
-  int u = blockIdx.x * blockDim.x + threadIdx.x;
-  if (u >= V) return;
+    int V, const double* __restrict__ Us, const int32_t* __restrict__ tv_ptr,
+    const int32_t* __restrict__ tv_row, const double* __restrict__ tv_coef,
+    const double* __restrict__ tv_visc, const int32_t* __restrict__ ts_ptr,
+    const int32_t* __restrict__ ts_ent, const double* __restrict__ mua, const double* __restrict__ Ge,
+    double* out, double cx, const double* X, double cy, const double* Y, double cz, const double* Z,
+    double cg, Phys ph) {
+  constexpr int G = kAdjLanes;
+  const int gt = blockIdx.x * blockDim.x + threadIdx.x, u = gt / G, lane = gt % G;
+  const bool live = u < V;
   // R = -D [F, G, h] + Dv [Fv, Gv]: the Euler fluxes take -D^T mu, the viscous ones +Dv^T mu
   double Fb[4] = {0, 0, 0, 0}, Gb[4] = {0, 0, 0, 0};
   double Fvb[4] = {0, 0, 0, 0}, Gvb[4] = {0, 0, 0, 0};
-  for (int t = tv_ptr[u]; t < tv_ptr[u + 1]; ++t) {
-    int r = tv_row[t], j = tv_pos[t];
-    int n0 = vptr[r], N = vptr[r + 1] - n0;
-    const double* c = cv + 6 * (size_t)n0;
-    double d0f = c[j], d0g = c[N + j], dxf = c[2 * N + j], dxg = c[3 * N + j];
-    double dyf = c[4 * N + j], dyg = c[5 * N + j];
+  const int t1 = live ? tv_ptr[u + 1] : 0;
+  for (int t = live ? tv_ptr[u] + lane : 0; t < t1; t += G) {
+    const double2* m = reinterpret_cast<const double2*>(mua + (size_t)tv_row[t] * 12);
+    const double2* c = reinterpret_cast<const double2*>(tv_coef + (size_t)6 * t);
+    const double2 c0 = c[0], c1 = c[1], c2 = c[2];
+    const double2 a = m[0], b = m[1], ax = m[2], bx = m[3], ay = m[4], by = m[5];
+    const double m0[4] = {a.x, a.y, b.x, b.y}, mx[4] = {ax.x, ax.y, bx.x, bx.y}, my[4] = {ay.x, ay.y, by.x, by.y};
+#pragma unroll
     for (int q = 0; q < 4; ++q) {
-      double m0 = mu[(size_t)q * V + r], mx = mu[(size_t)(4 + q) * V + r];
-      double my = mu[(size_t)(8 + q) * V + r];
-      Fb[q] -= d0f * m0 + dxf * mx + dyf * my;
-      Gb[q] -= d0g * m0 + dxg * mx + dyg * my;
+      Fb[q] = fma(-c0.x, m0[q], fma(-c1.x, mx[q], fma(-c2.x, my[q], Fb[q])));
+      Gb[q] = fma(-c0.y, m0[q], fma(-c1.y, mx[q], fma(-c2.y, my[q], Gb[q])));
     }
-    if (cvis) {
-      const double* z = cvis + 6 * (size_t)n0;
-      double e0f = z[j], e0g = z[N + j], exf = z[2 * N + j], exg = z[3 * N + j];
-      double eyf = z[4 * N + j], eyg = z[5 * N + j];
+    if (VISC) {
+      const double2* z = reinterpret_cast<const double2*>(tv_visc + (size_t)6 * t);
+      const double2 z0 = z[0], z1 = z[1], z2 = z[2];
+#pragma unroll
       for (int q = 0; q < 4; ++q) {
-        double m0 = mu[(size_t)q * V + r], mx = mu[(size_t)(4 + q) * V + r];
-        double my = mu[(size_t)(8 + q) * V + r];
-        Fvb[q] += e0f * m0 + exf * mx + eyf * my;
-        Gvb[q] += e0g * m0 + exg * mx + eyg * my;
+        Fvb[q] = fma(z0.x, m0[q], fma(z1.x, mx[q], fma(z2.x, my[q], Fvb[q])));
+        Gvb[q] = fma(z0.y, m0[q], fma(z1.y, mx[q], fma(z2.y, my[q], Gvb[q])));
       }
     }
   }
-  double w[12], g[12];
-  for (int r = 0; r < 12; ++r) w[r] = Us[(size_t)r * V + u];
+  double g[12];
+#pragma unroll
   for (int r = 0; r < 12; ++r) g[r] = 0.0;
-  adj::euler_flux_vjp(w, ph.gamma - 1.0, Fb, Gb, g);
-  if (cvis) adj::viscous_flux_vjp(w, ph.gamma - 1.0, ph.mu, ph.kappa, ph.R_gas, Fvb, Gvb, g);
-  for (int t = ts_ptr[u]; t < ts_ptr[u + 1]; ++t) {
-    int ent = ts_ent[t];
-    const double* ge = Ge + (size_t)(ent / 6) * 72 + 12 * (ent % 6);
-    for (int r = 0; r < 12; ++r) g[r] += ge[r];
+  const int s1 = live ? ts_ptr[u + 1] : 0;
+  for (int t = live ? ts_ptr[u] + lane : 0; t < s1; t += G) {
+    const int ent = ts_ent[t];
+    const double2* ge = reinterpret_cast<const double2*>(Ge + (size_t)(ent / 6) * 72 + 12 * (ent % 6));
+#pragma unroll
+    for (int i = 0; i < 6; ++i) {
+      const double2 x = ge[i];
+      g[2 * i] += x.x;
+      g[2 * i + 1] += x.y;
+    }
   }
+#pragma unroll
+  for (int q = 0; q < 4; ++q) {
+    Fb[q] = group_sum<G>(Fb[q]);
+    Gb[q] = group_sum<G>(Gb[q]);
+    if (VISC) {
+      Fvb[q] = group_sum<G>(Fvb[q]);
+      Gvb[q] = group_sum<G>(Gvb[q]);
+    }
+  }
+#pragma unroll
+  for (int r = 0; r < 12; ++r) g[r] = group_sum<G>(g[r]);
+  if (!live) return;
+  double w[12];
+#pragma unroll
+  for (int r = 0; r < 12; ++r) w[r] = (VISC || r < 4) ? Us[(size_t)r * V + u] : 0.0;
+  adj::euler_flux_vjp(w, ph.gamma - 1.0, Fb, Gb, g);
+  if (VISC) adj::viscous_flux_vjp(w, ph.gamma - 1.0, ph.mu, ph.kappa, ph.R_gas, Fvb, Gvb, g);
+#pragma unroll
   for (int r = 0; r < 12; ++r) {
-    size_t i = (size_t)r * V + u;
+    if (r % G != lane) continue;
+    const size_t i = (size_t)r * V + u;
     double o = cg * g[r];
     if (X) o += cx * X[i];
     if (Y) o += cy * Y[i];
@@ -578,8 +648,28 @@ hfd_status build_transposes(hfd_mesh* m) {
   if ((st = upload_vec(m, &m->adj_te_pos, teq)) != HFD_OK) return st;
   if ((st = upload_vec(m, &m->adj_ts_ptr, tsp)) != HFD_OK) return st;
   if ((st = upload_vec(m, &m->adj_ts_ent, tse)) != HFD_OK) return st;
+  auto coefs = [&](int n, int rows, const int32_t* row, const int32_t* pos, const int32_t* ptr, const void* coef,
+                   double** dst) {
+    void* p = nullptr;
+    ACK(mesh_malloc(m, &p, std::max<size_t>((size_t)n * rows * sizeof(double), 16)));
+    *dst = static_cast<double*>(p);
+    if (n > 0)
+      hfd::k_adj_gather_coef<<<(n + 255) / 256, 256>>>(n, rows, row, pos, ptr, (const double*)coef, *dst);
+    ACK(cudaGetLastError());
+    return HFD_OK;
+  };
+  if ((st = coefs(eptr[A], 3, m->adj_te_row, m->adj_te_pos, d.eptr, d.ce, &m->adj_te_coef)) != HFD_OK) return st;
+  if ((st = coefs(vptr[A], 6, m->adj_tv_row, m->adj_tv_pos, d.vptr, d.cv, &m->adj_tv_coef)) != HFD_OK) return st;
+  if (d.viscous &&
+      (st = coefs(vptr[A], 6, m->adj_tv_row, m->adj_tv_pos, d.vptr, d.cvis, &m->adj_tv_visc)) != HFD_OK)
+    return st;
+  ACK(cudaDeviceSynchronize());
   std::vector<double> zeros;
-  zeros.resize((size_t)72 * Ef);
+  zeros.resize((size_t)4 * Ef);
+  if ((st = upload_vec(m, &m->adj_hbar, zeros)) != HFD_OK) return st;
+  zeros.assign((size_t)12 * V, 0.0);
+  if ((st = upload_vec(m, &m->adj_mua, zeros)) != HFD_OK) return st;
+  zeros.assign((size_t)72 * Ef, 0.0);
   if ((st = upload_vec(m, &m->adj_Ge, zeros)) != HFD_OK) return st;
   zeros.assign((size_t)12 * V, 0.0);
   if ((st = upload_vec(m, &m->adj_B1, zeros)) != HFD_OK) return st;
@@ -633,22 +723,37 @@ hfd_status residual_vjp(hfd_mesh* m, const double* Us, const double* mu, double*
                         double cg, cudaStream_t s) {
   const hfd::DevMesh& d = m->dm;
   ACK(hfd::launch_vertex(d, Us, m->ph, s));          // AoS copy of the stage state
+  hfd::k_adj_aos<<<(d.V + 255) / 256, 256, 0, s>>>(d.V, mu, m->adj_mua);
+  ACK(cudaGetLastError());
+  hfd::k_adj_hbar<<<(unsigned)(((size_t)d.Ef * hfd::kAdjEdgeLanes + 127) / 128), 128, 0, s>>>(
+      d.Ef, m->adj_te_ptr, m->adj_te_row, m->adj_te_coef, m->adj_mua, m->adj_hbar);
+  ACK(cudaGetLastError());
+  hfd::EdgeFx fx;                     // the pairs and codes launch_vertex wrote for the edge kernel
+  if (d.div_fx && !d.div_df) {
+    fx.uf = d.fx.uf;
+    fx.uc = d.fx.uc;
+    fx.w5f = d.fx.w5f;
+    fx.w5e = d.fx.w5e;
+  }
   // edges with both sides on the 5-node branch, then the listed remainder
   ACK(cudaMemsetAsync(m->adj_count, 0, sizeof(int32_t), s));
   hfd::k_adj_edge<<<(d.Ef + 127) / 128, 128, 0, s>>>(
-      d.Ef, d.V, d.sten, (const double*)d.nrm, (const double*)d.w5, (const double*)d.w3,
-      (const double*)d.Ua, d.eptr, (const double*)d.ce, m->adj_te_ptr, m->adj_te_row,
-      m->adj_te_pos, mu, m->adj_Ge, m->ph, m->adj_list, m->adj_count);
+      d.Ef, d.sten, (const double*)d.nrm, (const double*)d.w5, (const double*)d.w3,
+      (const double*)d.Ua, m->adj_hbar, m->adj_Ge, m->ph, fx, m->adj_list, m->adj_count);
   ACK(cudaGetLastError());
   hfd::k_adj_edge_full<<<(d.Ef + 127) / 128, 128, 0, s>>>(
-      d.Ef, d.V, d.sten, (const double*)d.nrm, (const double*)d.w5, (const double*)d.w3,
-      (const double*)d.Ua, d.eptr, (const double*)d.ce, m->adj_te_ptr, m->adj_te_row,
-      m->adj_te_pos, mu, m->adj_Ge, m->ph, m->adj_list, m->adj_count);
+      d.Ef, d.sten, (const double*)d.nrm, (const double*)d.w5, (const double*)d.w3,
+      (const double*)d.Ua, m->adj_hbar, m->adj_Ge, m->ph, fx, m->adj_list, m->adj_count);
   ACK(cudaGetLastError());
-  hfd::k_adj_vertex<<<(d.V + 127) / 128, 128, 0, s>>>(
-      d.V, Us, d.vptr, (const double*)d.cv, d.viscous ? (const double*)d.cvis : nullptr,
-      m->adj_tv_ptr, m->adj_tv_row, m->adj_tv_pos,
-      m->adj_ts_ptr, m->adj_ts_ent, mu, m->adj_Ge, out, cx, X, cy, Y, cz, Z, cg, m->ph);
+  const unsigned nb = (unsigned)(((size_t)d.V * hfd::kAdjLanes + 127) / 128);
+  if (d.viscous)
+    hfd::k_adj_vertex<true><<<nb, 128, 0, s>>>(
+        d.V, Us, m->adj_tv_ptr, m->adj_tv_row, m->adj_tv_coef, m->adj_tv_visc, m->adj_ts_ptr, m->adj_ts_ent,
+        m->adj_mua, m->adj_Ge, out, cx, X, cy, Y, cz, Z, cg, m->ph);
+  else
+    hfd::k_adj_vertex<false><<<nb, 128, 0, s>>>(
+        d.V, Us, m->adj_tv_ptr, m->adj_tv_row, m->adj_tv_coef, nullptr, m->adj_ts_ptr, m->adj_ts_ent,
+        m->adj_mua, m->adj_Ge, out, cx, X, cy, Y, cz, Z, cg, m->ph);
   ACK(cudaGetLastError());
   // X, Y, Z are transposed already (zero transmissive ghost columns), so T(out) = cx X + cy Y +
   // cz Z + cg T((dR/dU)^T mu)

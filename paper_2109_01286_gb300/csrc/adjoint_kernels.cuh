@@ -3,6 +3,7 @@
 // same arithmetic as the forward functions in kernels.cu (branch decisions held fixed).
 #pragma once
 
+#include "fp64_roots.cuh"
 #include "kernels.hpp"
 
 namespace hfd {
@@ -11,25 +12,30 @@ namespace adj {
 // Roe-averaged state (u, v, H, c) of two conservative states (the weights sqrt(rho) form).
 struct RoeState {
   double irl, irr, ul, vl, ur, vr, pl, pr, Hl, Hr, rl, rr, fl, fr, u, v, H, c;
+  double isum, ic;      // 1 / (sqrt(rho_l) + sqrt(rho_r)), 1 / c
 };
 
 __device__ __forceinline__ void roe_state(const double* wl, const double* wr, double g1, RoeState& s) {
-  s.irl = 1.0 / wl[0];
-  s.irr = 1.0 / wr[0];
+  const double sl = rsqrt64(wl[0]), sr = rsqrt64(wr[0]);
+  s.irl = sl * sl;
+  s.irr = sr * sr;
   s.ul = wl[1] * s.irl; s.vl = wl[2] * s.irl;
   s.ur = wr[1] * s.irr; s.vr = wr[2] * s.irr;
   s.pl = g1 * (wl[3] - 0.5 * (wl[1] * s.ul + wl[2] * s.vl));
   s.pr = g1 * (wr[3] - 0.5 * (wr[1] * s.ur + wr[2] * s.vr));
   s.Hl = (wl[3] + s.pl) * s.irl;
   s.Hr = (wr[3] + s.pr) * s.irr;
-  s.rl = sqrt(wl[0]);
-  s.rr = sqrt(wr[0]);
-  s.fl = s.rl / (s.rl + s.rr);
+  s.rl = wl[0] * sl;
+  s.rr = wr[0] * sr;
+  s.isum = rcp64(s.rl + s.rr);
+  s.fl = s.rl * s.isum;
   s.fr = 1.0 - s.fl;
   s.u = s.fl * s.ul + s.fr * s.ur;
   s.v = s.fl * s.vl + s.fr * s.vr;
   s.H = s.fl * s.Hl + s.fr * s.Hr;
-  s.c = sqrt(g1 * (s.H - 0.5 * (s.u * s.u + s.v * s.v)));
+  const double c2 = g1 * (s.H - 0.5 * (s.u * s.u + s.v * s.v));
+  s.ic = rsqrt64(c2);
+  s.c = c2 * s.ic;
 }
 
 // adjoint of the primitive quantities of one state: given bars of (u_k, v_k, p_k, H_k) and of
@@ -61,7 +67,7 @@ __device__ __forceinline__ void roe_state_vjp(const double* wl, const double* wr
                                               const RoeState& s, double ub, double vb, double Hb,
                                               double cb, double* wlb, double* wrb) {
   // c = sqrt(g1 (H - (u^2 + v^2)/2))
-  double c2b = cb / (2.0 * s.c);
+  double c2b = 0.5 * cb * s.ic;
   Hb += g1 * c2b;
   ub -= g1 * s.u * c2b;
   vb -= g1 * s.v * c2b;
@@ -71,10 +77,9 @@ __device__ __forceinline__ void roe_state_vjp(const double* wl, const double* wr
   double ulb = s.fl * ub, urb = s.fr * ub, vlb = s.fl * vb, vrb = s.fr * vb;
   double Hlb = s.fl * Hb, Hrb = s.fr * Hb;
   flb -= frb;                                   // fr = 1 - fl
-  double den = s.rl + s.rr;
-  double rlb = flb * s.rr / (den * den), rrb = -flb * s.rl / (den * den);
-  wlb[0] += rlb / (2.0 * s.rl);
-  wrb[0] += rrb / (2.0 * s.rr);
+  const double t = 0.5 * flb * (s.isum * s.isum);     // 1 / sqrt(rho) = sqrt(rho) / rho
+  wlb[0] += t * s.rr * (s.rl * s.irl);
+  wrb[0] -= t * s.rl * (s.rr * s.irr);
   prim_vjp(wl, s.irl, s.ul, s.vl, s.pl, ulb, vlb, 0.0, Hlb, 0.0, g1, wlb);
   prim_vjp(wr, s.irr, s.ur, s.vr, s.pr, urb, vrb, 0.0, Hrb, 0.0, g1, wrb);
 }
@@ -83,7 +88,7 @@ __device__ __forceinline__ void roe_state_vjp(const double* wl, const double* wr
 __device__ __forceinline__ void left_ev_vjp(double u, double v, double c, double nx, double ny,
                                             double g1, const double (*Lb)[4], double& ub,
                                             double& vb, double& cb) {
-  double ic = 1.0 / c;
+  double ic = rcp64(c);
   double b1 = g1 * ic * ic;
   double qn = u * nx + v * ny;
   double b1b = 0, b2b = 0, qnb = 0, qtb = 0, icb = 0;
@@ -132,7 +137,7 @@ __device__ void roe_flux_vjp(const double* wl, const double* wr, double nx, doub
   RoeState s;
   roe_state(wl, wr, g1, s);
   const double u = s.u, v = s.v, H = s.H, c = s.c;
-  double ic = 1.0 / c, b1 = g1 * ic * ic, b2 = 0.5 * b1 * (u * u + v * v);
+  double ic = s.ic, b1 = g1 * ic * ic, b2 = 0.5 * b1 * (u * u + v * v);
   double qn = u * nx + v * ny, qt = -u * ny + v * nx;
   double L[4][4] = {
       {0.5 * (b2 + qn * ic), -0.5 * (b1 * u + nx * ic), -0.5 * (b1 * v + ny * ic), 0.5 * b1},

@@ -56,6 +56,10 @@ struct hfd_mesh {
   int32_t *adj_te_ptr = nullptr, *adj_te_row = nullptr, *adj_te_pos = nullptr;
   int32_t *adj_ts_ptr = nullptr, *adj_ts_ent = nullptr;
   double *adj_Ge = nullptr, *adj_B1 = nullptr, *adj_B2 = nullptr;
+  // the divergence's coefficients in the order of the transposed lists (3 per edge entry, 6 per vertex
+  // entry), mu with its 12 rows side by side, and -(D^T mu) per flux edge
+  double *adj_te_coef = nullptr, *adj_tv_coef = nullptr, *adj_tv_visc = nullptr;
+  double *adj_mua = nullptr, *adj_hbar = nullptr;
   int32_t *adj_list = nullptr, *adj_count = nullptr;
   // transpose of the transmissive ghost refresh (meshes with ghosts): unique donors, the CSR of
   // each donor's ghosts in ascending order with their flags; scratch for the step input with
