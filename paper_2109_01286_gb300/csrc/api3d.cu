@@ -16,6 +16,7 @@ struct hfd3_mesh {
   hfd::Phys3 ph;
   hfd3_options opts;
   std::vector<void*> allocs;
+  int* fx_flag = nullptr;       // device word of the packing kernel (null: rows not packed)
 };
 
 namespace {
@@ -78,6 +79,38 @@ hfd_status upload_edges(hfd3_mesh* m) {
   return HFD_OK;
 }
 
+// The fixed-point divergence: allocates m->d.fx on the first call and packs the coefficients.  Left off
+// (the FP64 gather runs) if an index is out of range or a coefficient does not fit.
+hfd_status pack_fx(hfd3_mesh* m) {
+  hfd::DevMesh3& d = m->d;
+  const hfd::Prep3& P = m->P;
+  d.fx_ok = false;
+  if (d.V == 0 || 3 * (int64_t)d.V + d.E > INT32_MAX) return HFD_OK;
+  if (!m->fx_flag) {
+    std::vector<int32_t> ptr(d.V + 1, 0);
+    for (int v = 0; v < d.V; ++v)
+      ptr[v + 1] = ptr[v] + (3 * (P.vptr[v + 1] - P.vptr[v]) + P.eptr[v + 1] - P.eptr[v] + 15) / 16;
+    for (int32_t u : P.vidx)
+      if (u < 0 || u >= d.V) return HFD_OK;
+    for (int32_t e : P.eidx)
+      if (e < 0 || e >= d.E) return HFD_OK;
+    const size_t n = (size_t)ptr[d.V];
+    TRY3(dalloc(m, (void**)&d.fx.ptr, ptr.size() * sizeof(int32_t)));
+    TRY3(dalloc(m, (void**)&d.fx.id, 4 * n * sizeof(int4)));
+    TRY3(dalloc(m, (void**)&d.fx.c, 32 * n * sizeof(int4)));
+    TRY3(dalloc(m, (void**)&d.fx.cexp, (size_t)d.V * sizeof(int2)));
+    TRY3(dalloc(m, (void**)&d.fx.rec, 3 * (3 * (size_t)d.V + d.E) * sizeof(int4)));
+    TRY3(put(ptr, d.fx.ptr));
+    TRY3(dalloc(m, (void**)&m->fx_flag, sizeof(int)));
+  }
+  int flag = 0;
+  CK3(cudaMemset(m->fx_flag, 0, sizeof(int)));
+  CK3(hfd::launch3_pack(d, m->fx_flag, nullptr));
+  CK3(cudaMemcpy(&flag, m->fx_flag, sizeof flag, cudaMemcpyDeviceToHost));
+  d.fx_ok = flag == 0;
+  return HFD_OK;
+}
+
 hfd_status create(const hfd3_mesh_desc* desc, const hfd3_options* o, hfd3_mesh* m) {
   TRY3(hfd::build_prep3(desc, o, &m->P));
   const hfd::Prep3& P = m->P;
@@ -110,6 +143,7 @@ hfd_status create(const hfd3_mesh_desc* desc, const hfd3_options* o, hfd3_mesh* 
   TRY3(put(P.eidx, d.eidx));
   TRY3(put(P.cv, d.cv));
   TRY3(put(P.ce, d.ce));
+  TRY3(pack_fx(m));
   m->ph.gamma = o->gamma;
   m->ph.g1 = o->gamma - 1.0;
   m->ph.eps = o->weno_eps;
@@ -270,8 +304,10 @@ hfd_status hfd3_prep_set(hfd3_mesh* m, const char* name, const void* src, int64_
   std::memcpy(a.p, src, (size_t)a.n * a.elt);
   if (!m->d.err) return HFD_OK;               // host-only mesh: no device copy to refresh
   const std::string s(name);
-  if (s == "cv") return put(m->P.cv, m->d.cv);
-  if (s == "ce") return put(m->P.ce, m->d.ce);
+  if (s == "cv" || s == "ce") {
+    TRY3(s == "cv" ? put(m->P.cv, m->d.cv) : put(m->P.ce, m->d.ce));
+    return pack_fx(m);
+  }
   return upload_edges(m);
 }
 

@@ -332,13 +332,6 @@ __global__ void __launch_bounds__(128, 4) k_div_fx(DivFx m, StageArgs sa, const 
 }
 
 // ------------------------------------------------------------------ coefficients to fixed point
-// Exponent e with |x| < 2^e (0 for x = 0), from a double's field.
-__device__ __forceinline__ int exp_above(double x) { return x == 0.0 ? -10000 : ilogb(x) + 1; }
-
-__device__ __forceinline__ int2 coef_limbs(double c, int e, int L) {
-  return fx_split(llrint(scalbn(c, 2 * L - 1 - e)), L);
-}
-
 // One thread per row: packs the row's FP64 coefficients (cv, ce, cvis: structure of arrays over the
 // row's entries) into chunks.  Flags a row whose exponents leave 10 bits or one of whose vertices
 // is on none of its edges (its exponent word would not cover that vertex).

@@ -38,6 +38,13 @@ __device__ __forceinline__ int2 fx_split(long long v, int L) {
   return make_int2((int)h, (int)(v - (h << L)));
 }
 
+// Exponent e with |x| < 2^e (0 for x = 0), from a double's field.
+__device__ __forceinline__ int exp_above(double x) { return x == 0.0 ? -10000 : ilogb(x) + 1; }
+
+__device__ __forceinline__ int2 coef_limbs(double c, int e, int L) {
+  return fx_split(llrint(scalbn(c, 2 * L - 1 - e)), L);
+}
+
 // x at the scale of code E, as stored: the 64-bit integer x 2^(1022 - E + L - 1 + 32), truncated
 // toward zero; the upper word is the high limb, the lower one the low limb and 32 - L more bits.
 __device__ __forceinline__ int2 fx_encode(double x, int E, int L) {

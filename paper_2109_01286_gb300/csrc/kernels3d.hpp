@@ -14,4 +14,9 @@ cudaError_t launch3_edge(const DevMesh3& m, const Phys3& ph, cudaStream_t s);
 cudaError_t launch3_div(const DevMesh3& m, const double* Us, const double* Un, double* out,
                         int mode, double a, double b, double dt, cudaStream_t s);
 
+// Packs m.cv and m.ce into m.fx; *flag (device) is set if a coefficient does not fit.
+cudaError_t launch3_pack(const DevMesh3& m, int* flag, cudaStream_t s);
+// The lanes of the next launches: 0 the fixed-point divergence, else the FP64 one.
+inline int div3_lanes(const DevMesh3& m) { return m.lanes ? m.lanes : m.fx_ok ? 0 : 4; }
+
 }  // namespace hfd

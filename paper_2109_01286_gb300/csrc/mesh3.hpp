@@ -5,6 +5,9 @@
 
 #include "hfd3d.h"
 
+struct int2;   // CUDA's vector types
+struct int4;
+
 namespace hfd {
 
 // Everything geometry-only of a periodic tetrahedral mesh (host, FP64).  Edge arrays are
@@ -31,10 +34,23 @@ struct Prep3 {
 // Builds the preprocessing; HFD_OK or an error status with hfd_last_error set.
 hfd_status build_prep3(const hfd3_mesh_desc* d, const hfd3_options* o, Prep3* P);
 
+// The divergence rows in fixed point (k3_div_fx): a row is a list of products of a 5-vector record --
+// an edge's flux, or F, G or K of a vertex -- with one coefficient of each of d_0 .. d_z, in chunks
+// of 16 products.
+struct Div3Fx {
+  int32_t* ptr = nullptr;       // V + 1: chunks
+  int4* id = nullptr;           // 4 per chunk: records of stream s = 0..3, 4 each
+  int4* c = nullptr;            // 32 per chunk: [product of the stream][stream][d_0 d_x | d_y d_z] limb pairs
+  int2* cexp = nullptr;         // V: exponents of the rows d_0 .. d_z, 16 bits each
+  int4* rec = nullptr;          // 3 V + E records of 3: five pairs and a code word
+};
+
 // Device arrays of a 3D mesh.
 struct DevMesh3 {
   int V = 0, E = 0;
-  int lanes = 4;                // threads per vertex in the divergence gather (1, 2, 4)
+  int lanes = 0;                // threads per vertex in the FP64 gather (1, 2, 4); 0: fixed point if fx
+  bool fx_ok = false;           // the rows fit fixed point
+  Div3Fx fx;
   int32_t* sten = nullptr;      // 6 x E (SoA)
   double* frame = nullptr;      // 9 x E (SoA)
   double* w5 = nullptr;         // 40 x E (SoA)
