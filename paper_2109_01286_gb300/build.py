@@ -30,7 +30,7 @@ def _nvcc():
 
 def _sources():
     return [os.path.join(CSRC, f) for f in ("prep.cpp", "kernels.cu", "div_fixed.cu", "api.cu", "noalloc.cu",
-                                            "adjoint.cu", "peaks.cu", "prep3.cpp", "kernels3d.cu",
+                                            "adjoint.cu", "peaks.cu", "prep3.cpp", "kernels3d.cu", "edge3d.cu",
                                             "api3d.cu")]
 
 
@@ -39,7 +39,7 @@ def _deps():
                                                          "adjoint_kernels.cuh", "linalg.hpp",
                                                          "mesh3.hpp", "kernels3d.hpp", "fp_convert.cuh",
                                                          "fixed_point.cuh", "div_common.cuh", "mbar.cuh",
-                                                         "fp64_roots.cuh", "edge64.cuh")] + \
+                                                         "fp64_roots.cuh", "edge64.cuh", "record3.cuh")] + \
         [os.path.join(INCLUDE, "hfd.h"), os.path.join(INCLUDE, "hfd3d.h"), os.path.abspath(__file__)]
 
 

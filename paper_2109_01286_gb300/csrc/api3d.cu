@@ -16,7 +16,7 @@ struct hfd3_mesh {
   hfd::Phys3 ph;
   hfd3_options opts;
   std::vector<void*> allocs;
-  int* fx_flag = nullptr;       // device word of the packing kernel (null: rows not packed)
+  int* fx_flag = nullptr;       // device word of the packing kernels
 };
 
 namespace {
@@ -70,13 +70,25 @@ hfd_status put(const std::vector<T>& h, T* dptr) {
     if (s_ != HFD_OK) return s_;         \
   } while (0)
 
+// The edges' weights in fixed point; left off (the sums run in FP64) where a weight does not fit.
+hfd_status pack_edges(hfd3_mesh* m) {
+  hfd::DevMesh3& d = m->d;
+  int flag = 0;
+  d.ex_ok = false;
+  CK3(cudaMemset(m->fx_flag, 0, sizeof(int)));
+  CK3(hfd::launch3_pack_w5(d, m->fx_flag, nullptr));
+  CK3(cudaMemcpy(&flag, m->fx_flag, sizeof flag, cudaMemcpyDeviceToHost));
+  d.ex_ok = flag == 0;
+  return HFD_OK;
+}
+
 hfd_status upload_edges(hfd3_mesh* m) {
   const int E = m->P.E;
   TRY3(put(to_soa(m->P.sten, E, 6), m->d.sten));
   TRY3(put(to_soa(m->P.frame, E, 9), m->d.frame));
   TRY3(put(to_soa(m->P.w5, E, 40), m->d.w5));
   TRY3(put(to_soa(m->P.w3, E, 18), m->d.w3));
-  return HFD_OK;
+  return pack_edges(m);
 }
 
 // The fixed-point divergence: allocates m->d.fx on the first call and packs the coefficients.  Left off
@@ -86,7 +98,7 @@ hfd_status pack_fx(hfd3_mesh* m) {
   const hfd::Prep3& P = m->P;
   d.fx_ok = false;
   if (d.V == 0 || 3 * (int64_t)d.V + d.E > INT32_MAX) return HFD_OK;
-  if (!m->fx_flag) {
+  if (!d.fx.ptr) {
     std::vector<int32_t> ptr(d.V + 1, 0);
     for (int v = 0; v < d.V; ++v)
       ptr[v + 1] = ptr[v] + (3 * (P.vptr[v + 1] - P.vptr[v]) + P.eptr[v + 1] - P.eptr[v] + 15) / 16;
@@ -95,13 +107,12 @@ hfd_status pack_fx(hfd3_mesh* m) {
     for (int32_t e : P.eidx)
       if (e < 0 || e >= d.E) return HFD_OK;
     const size_t n = (size_t)ptr[d.V];
-    TRY3(dalloc(m, (void**)&d.fx.ptr, ptr.size() * sizeof(int32_t)));
     TRY3(dalloc(m, (void**)&d.fx.id, 4 * n * sizeof(int4)));
     TRY3(dalloc(m, (void**)&d.fx.c, 32 * n * sizeof(int4)));
     TRY3(dalloc(m, (void**)&d.fx.cexp, (size_t)d.V * sizeof(int2)));
     TRY3(dalloc(m, (void**)&d.fx.rec, 3 * (3 * (size_t)d.V + d.E) * sizeof(int4)));
+    TRY3(dalloc(m, (void**)&d.fx.ptr, ptr.size() * sizeof(int32_t)));
     TRY3(put(ptr, d.fx.ptr));
-    TRY3(dalloc(m, (void**)&m->fx_flag, sizeof(int)));
   }
   int flag = 0;
   CK3(cudaMemset(m->fx_flag, 0, sizeof(int)));
@@ -136,6 +147,16 @@ hfd_status create(const hfd3_mesh_desc* desc, const hfd3_options* o, hfd3_mesh* 
   TRY3(dalloc(m, (void**)&d.U2, 20 * V * sizeof(double)));
   TRY3(dalloc(m, (void**)&d.err, sizeof(unsigned)));
   CK3(cudaMemset(d.err, 0, sizeof(unsigned)));
+  TRY3(dalloc(m, (void**)&m->fx_flag, sizeof(int)));
+  TRY3(dalloc(m, (void**)&d.ex.uf, 10 * V * sizeof(int4)));
+  TRY3(dalloc(m, (void**)&d.ex.uc, 2 * V * sizeof(uint4)));
+  TRY3(dalloc(m, (void**)&d.ex.w5f, 40 * E * sizeof(int2)));
+  TRY3(dalloc(m, (void**)&d.ex.w5e, E * sizeof(int2)));
+  TRY3(dalloc(m, (void**)&d.ex.framef, 9 * E * sizeof(float)));
+  TRY3(dalloc(m, (void**)&d.ex.list, E * sizeof(int2)));
+  TRY3(dalloc(m, (void**)&d.ex.listw, 12 * E * sizeof(double)));
+  TRY3(dalloc(m, (void**)&d.ex.count, sizeof(int)));
+  CK3(cudaMemset(d.ex.count, 0, sizeof(int)));
   TRY3(upload_edges(m));
   TRY3(put(P.vptr, d.vptr));
   TRY3(put(P.eptr, d.eptr));
@@ -151,6 +172,7 @@ hfd_status create(const hfd3_mesh_desc* desc, const hfd3_options* o, hfd3_mesh* 
   m->ph.sens_hi = o->sens_hi;
   m->ph.harten = o->harten;
   m->ph.half_inv_harten = 0.5 / o->harten;
+  m->ph.g1f = (float)(o->gamma - 1.0);
   m->ph.epsf = (float)o->weno_eps;
   m->ph.sens_lof = (float)o->sens_lo;
   m->ph.sens_hif = (float)o->sens_hi;

@@ -2,24 +2,18 @@
 // SSP-RK3 step; FP64 state, fluxes and sums.  Per Runge-Kutta stage:
 //   k3_vertex  one thread per vertex: the vertex-major copy of the 20 unknowns and the analytic
 //              flux vectors F, G, K (Sec. 2.3, vertex fluxes, in 3D);
-//   k3_edge    one thread per edge: Alg. 1 in 3D (Roe average of the edge ends, five-wave
-//              characteristic projection along the edge, uniform WENO5 weights as the sensor --
-//              taken in FP32 and again in FP64 inside a band around each threshold -- 5-node
-//              Hermite value or weighted 3-node value per component and side,
-//              back-projection, positivity fallback) and Roe's flux with Harten's fix;
+//   k3_edge    edge fluxes (edge3d.cu);
 //   k3_div_fx  8 lanes per vertex: the CSR gather of the least-squares divergence rows
 //              d_0, d_x, d_y, d_z over the vertex fluxes and edge fluxes (Eq.
 //              (flux_polynomials) in 3D) in fixed point, fused with the SSP-RK3 stage update;
 //   k3_div     the same gather in FP64, 1, 2 or 4 lanes per vertex (chosen lanes, long rows).
-// The characteristic projection uses the closed forms of the left and right eigenvectors of
-// the flux Jacobian along n with the frame (n, t1, t2): waves q_n - c, entropy, shear along
-// t1, shear along t2, q_n + c.
 #include <cuda_runtime.h>
 
 #include "fixed_point.cuh"
-#include "fp_convert.cuh"
+#include "fp64_roots.cuh"
 #include "kernels3d.hpp"
 #include "mbar.cuh"
+#include "record3.cuh"
 
 namespace hfd {
 namespace {
@@ -28,173 +22,13 @@ constexpr unsigned kErrNonfinite = 1u, kErrPositivity = 2u, kErrIndex = 4u;
 
 __device__ __forceinline__ bool finite3(double x) { return isfinite(x); }
 
-// The eigen-structure of one Roe state along the frame (n, t1, t2), and the two states'
-// reciprocal densities and pressures (shared with the normal fluxes).
-struct Eig {
-  double u[3], H, c, qn, q1, q2, K, b1, b2, ic;
-  double n[3], t1[3], t2[3];
-  double irl, irr, pl, pr;
-};
-
-// One reciprocal square root per state gives sqrt(rho) and 1/rho, one more gives c and 1/c
-// (the CUDA math library's rsqrt); one division forms the Roe weights.
-__device__ __forceinline__ void roe_state(const double* wl, const double* wr, double g1, Eig& s) {
-  const double sl = rsqrt(wl[0]), sr = rsqrt(wr[0]);
-  s.irl = sl * sl;
-  s.irr = sr * sr;
-  s.pl = g1 * (wl[4] - 0.5 * (wl[1] * wl[1] + wl[2] * wl[2] + wl[3] * wl[3]) * s.irl);
-  s.pr = g1 * (wr[4] - 0.5 * (wr[1] * wr[1] + wr[2] * wr[2] + wr[3] * wr[3]) * s.irr);
-  const double is = 1.0 / (wl[0] * sl + wr[0] * sr);
-#pragma unroll
-  for (int k = 0; k < 3; ++k) s.u[k] = (wl[k + 1] * sl + wr[k + 1] * sr) * is;
-  s.H = ((wl[4] + s.pl) * sl + (wr[4] + s.pr) * sr) * is;
-  s.K = s.u[0] * s.u[0] + s.u[1] * s.u[1] + s.u[2] * s.u[2];
-  const double c2 = g1 * (s.H - 0.5 * s.K);
-  s.ic = rsqrt(c2);
-  s.c = c2 * s.ic;
-  s.qn = s.u[0] * s.n[0] + s.u[1] * s.n[1] + s.u[2] * s.n[2];
-  s.q1 = s.u[0] * s.t1[0] + s.u[1] * s.t1[1] + s.u[2] * s.t1[2];
-  s.q2 = s.u[0] * s.t2[0] + s.u[1] * s.t2[1] + s.u[2] * s.t2[2];
-  s.b1 = g1 * s.ic * s.ic;
-  s.b2 = 0.5 * s.b1 * s.K;
-}
-
-// c = L a for the five conserved components a.
-__device__ __forceinline__ void to_char(const Eig& s, const double* a, double* c) {
-  const double um = s.u[0] * a[1] + s.u[1] * a[2] + s.u[2] * a[3];
-  const double nm = (s.n[0] * a[1] + s.n[1] * a[2] + s.n[2] * a[3]) * s.ic;
-  const double t1m = s.t1[0] * a[1] + s.t1[1] * a[2] + s.t1[2] * a[3];
-  const double t2m = s.t2[0] * a[1] + s.t2[1] * a[2] + s.t2[2] * a[3];
-  const double qc = s.qn * s.ic;
-  c[0] = 0.5 * ((s.b2 + qc) * a[0] - s.b1 * um - nm + s.b1 * a[4]);
-  c[1] = (1.0 - s.b2) * a[0] + s.b1 * um - s.b1 * a[4];
-  c[2] = t1m - s.q1 * a[0];
-  c[3] = t2m - s.q2 * a[0];
-  c[4] = 0.5 * ((s.b2 - qc) * a[0] - s.b1 * um + nm + s.b1 * a[4]);
-}
-
-// w = R c.
-__device__ __forceinline__ void from_char(const Eig& s, const double* c, double* w) {
-  w[0] = c[0] + c[1] + c[4];
-#pragma unroll
-  for (int k = 0; k < 3; ++k)
-    w[k + 1] = (c[0] + c[1] + c[4]) * s.u[k] + (c[4] - c[0]) * s.c * s.n[k] + c[2] * s.t1[k] +
-               c[3] * s.t2[k];
-  w[4] = (c[0] + c[4]) * s.H + (c[4] - c[0]) * s.c * s.qn + c[1] * (0.5 * s.K) + c[2] * s.q1 +
-         c[3] * s.q2;
-}
-
-// The FP32 copy of an eigen-structure for the sensor, rounded by integer operations.
-struct EigF {
-  float u[3], n[3], t1[3], t2[3], ic, qn, q1, q2, b1, b2;
-};
-
-__device__ __forceinline__ void to_f32(const Eig& s, EigF& f) {
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    f.u[k] = d2f_rn(s.u[k]);
-    f.n[k] = d2f_rn(s.n[k]);
-    f.t1[k] = d2f_rn(s.t1[k]);
-    f.t2[k] = d2f_rn(s.t2[k]);
-  }
-  f.ic = d2f_rn(s.ic);
-  f.qn = d2f_rn(s.qn);
-  f.q1 = d2f_rn(s.q1);
-  f.q2 = d2f_rn(s.q2);
-  f.b1 = d2f_rn(s.b1);
-  f.b2 = d2f_rn(s.b2);
-}
-
-// c = L a in FP32 (the formulas of to_char).
-__device__ __forceinline__ void to_char_f(const EigF& s, const float* a, float* c) {
-  const float um = s.u[0] * a[1] + s.u[1] * a[2] + s.u[2] * a[3];
-  const float nm = (s.n[0] * a[1] + s.n[1] * a[2] + s.n[2] * a[3]) * s.ic;
-  const float t1m = s.t1[0] * a[1] + s.t1[1] * a[2] + s.t1[2] * a[3];
-  const float t2m = s.t2[0] * a[1] + s.t2[1] * a[2] + s.t2[2] * a[3];
-  const float qc = s.qn * s.ic;
-  c[0] = 0.5f * ((s.b2 + qc) * a[0] - s.b1 * um - nm + s.b1 * a[4]);
-  c[1] = (1.0f - s.b2) * a[0] + s.b1 * um - s.b1 * a[4];
-  c[2] = t1m - s.q1 * a[0];
-  c[3] = t2m - s.q2 * a[0];
-  c[4] = 0.5f * ((s.b2 - qc) * a[0] - s.b1 * um + nm + s.b1 * a[4]);
-}
-
-// rho > 0 and p > 0 (R16): p has the sign of E rho - |m|^2 / 2 when rho > 0.
-__device__ __forceinline__ bool admissible3(const double* w) {
-  return w[0] > 0.0 && w[4] * w[0] - 0.5 * (w[1] * w[1] + w[2] * w[2] + w[3] * w[3]) > 0.0;
-}
-
-// Uniform WENO5 on the five values u0..u4 (Jiang-Shu indicators, linear weights 1/16, 10/16,
-// 5/16) with every weight multiplied by (eps+b1)^2 (eps+b2)^2 (eps+b3)^2, so that the sensor
-// needs no division: t[i] is weight i times that product and S their sum; omega_i = t[i] / S.
-__device__ __forceinline__ void weno3(double u0, double u1, double u2, double u3, double u4,
-                                      double eps, double* t, double& S) {
-  const double e1 = u0 - 2.0 * u1 + u2, f1 = u0 - 4.0 * u1 + 3.0 * u2;
-  const double e2 = u1 - 2.0 * u2 + u3, f2 = u1 - u3;
-  const double e3 = u2 - 2.0 * u3 + u4, f3 = 3.0 * u2 - 4.0 * u3 + u4;
-  const double b1 = 13.0 / 12.0 * (e1 * e1) + 0.25 * (f1 * f1);
-  const double b2 = 13.0 / 12.0 * (e2 * e2) + 0.25 * (f2 * f2);
-  const double b3 = 13.0 / 12.0 * (e3 * e3) + 0.25 * (f3 * f3);
-  double s1 = eps + b1, s2 = eps + b2, s3 = eps + b3;
-  s1 *= s1;
-  s2 *= s2;
-  s3 *= s3;
-  t[0] = (1.0 / 16.0) * (s2 * s3);
-  t[1] = (10.0 / 16.0) * (s1 * s3);
-  t[2] = (5.0 / 16.0) * (s1 * s2);
-  S = t[0] + t[1] + t[2];
-}
-
-// weno3 in FP32, for the sensor's first pass.
-__device__ __forceinline__ void weno3f(float u0, float u1, float u2, float u3, float u4, float eps,
-                                       float& t0, float& S) {
-  const float e1 = u0 - 2.0f * u1 + u2, f1 = u0 - 4.0f * u1 + 3.0f * u2;
-  const float e2 = u1 - 2.0f * u2 + u3, f2 = u1 - u3;
-  const float e3 = u2 - 2.0f * u3 + u4, f3 = 3.0f * u2 - 4.0f * u3 + u4;
-  float s1 = eps + (13.0f / 12.0f * (e1 * e1) + 0.25f * (f1 * f1));
-  float s2 = eps + (13.0f / 12.0f * (e2 * e2) + 0.25f * (f2 * f2));
-  float s3 = eps + (13.0f / 12.0f * (e3 * e3) + 0.25f * (f3 * f3));
-  s1 *= s1;
-  s2 *= s2;
-  s3 *= s3;
-  t0 = 0.0625f * (s2 * s3);
-  S = t0 + 0.625f * (s1 * s3) + 0.3125f * (s1 * s2);
-}
-
-// Relative width of the band around each sensor threshold inside which the FP32 decision is
-// taken again in FP64.
-constexpr float kGuard3 = 1e-3f;
-
-// F_n(w) from the state, its reciprocal density and its pressure.
-__device__ __forceinline__ void normal_flux3(const double* w, double ir, double p, const double* n,
-                                             double* f) {
-  const double un = (w[1] * n[0] + w[2] * n[1] + w[3] * n[2]) * ir;
-  f[0] = w[0] * un;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) f[k + 1] = w[k + 1] * un + p * n[k];
-  f[4] = (w[4] + p) * un;
-}
-
 // ------------------------------------------------------------------ k3_vertex
-// A 5-vector's record in fixed point: its pairs and the codes of mass, momentum (one for the three: each row
-// reads fluxes in all directions, so every momentum sum has pressure-sized terms) and energy.
-constexpr int kBits3 = 29;
-__device__ __forceinline__ void st_record3(int4* rec, size_t i, const double* f) {
-  const int E0 = fx_code(f[0]), E1 = max(fx_code(f[1]), max(fx_code(f[2]), fx_code(f[3]))), E2 = fx_code(f[4]);
-  const int2 p0 = fx_encode(f[0], E0, kBits3), p1 = fx_encode(f[1], E1, kBits3), p2 = fx_encode(f[2], E1, kBits3);
-  const int2 p3 = fx_encode(f[3], E1, kBits3), p4 = fx_encode(f[4], E2, kBits3);
-  int4* o = rec + 3 * i;
-  o[0] = make_int4(p0.x, p0.y, p1.x, p1.y);
-  o[1] = make_int4(p2.x, p2.y, p3.x, p3.y);
-  o[2] = make_int4(p4.x, p4.y, (int)((unsigned)E0 | ((unsigned)E1 << 16)), E2);
-}
-
 // Ua: 20 values per vertex (160 B); FGK: F, G, K per vertex at a stride of 16 (128 B); FX: records 3 v,
 // 3 v + 1, 3 v + 2 instead.
 template <bool FX>
 __global__ void __launch_bounds__(256) k3_vertex(int V, const double* __restrict__ U,
                                                  double* __restrict__ Ua, double* __restrict__ FGK,
-                                                 int4* __restrict__ rec, double g1) {
+                                                 int4* __restrict__ rec, Edge3Fx ex, double g1) {
   const int v = blockIdx.x * blockDim.x + threadIdx.x;
   if (v >= V) return;
   double w[20];
@@ -203,7 +37,36 @@ __global__ void __launch_bounds__(256) k3_vertex(int V, const double* __restrict
   double2* ua = reinterpret_cast<double2*>(Ua + (size_t)20 * v);
 #pragma unroll
   for (int i = 0; i < 10; ++i) ua[i] = make_double2(w[2 * i], w[2 * i + 1]);
-  const double ir = 1.0 / w[0];
+  if (v == 0) *ex.count = 0;                     // the edge kernel's list starts empty
+  if (ex.uf) {                                   // pairs and codes for the edge kernel
+    int Ev[5], Ed[5];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) {
+      Ev[q] = fx_code(w[q]);
+      Ed[q] = max(fx_code(w[5 + q]), max(fx_code(w[10 + q]), fx_code(w[15 + q])));
+    }
+    int4* o = ex.uf + (size_t)10 * v;
+#pragma unroll
+    for (int g = 0; g < 4; ++g) {
+      const int* E = g ? Ed : Ev;
+      const double* a = w + 5 * g;
+#pragma unroll
+      for (int i = 0; i < 2; ++i) {
+        const int2 s = fx_encode(a[2 * i], E[2 * i], kBits3), t = fx_encode(a[2 * i + 1], E[2 * i + 1], kBits3);
+        o[2 * g + i] = make_int4(s.x, s.y, t.x, t.y);
+      }
+    }
+    const int2 e0 = fx_encode(w[4], Ev[4], kBits3), e1 = fx_encode(w[9], Ed[4], kBits3);
+    const int2 e2 = fx_encode(w[14], Ed[4], kBits3), e3 = fx_encode(w[19], Ed[4], kBits3);
+    o[8] = make_int4(e0.x, e0.y, e1.x, e1.y);
+    o[9] = make_int4(e2.x, e2.y, e3.x, e3.y);
+    unsigned c[5];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) c[q] = (unsigned)Ev[q] | ((unsigned)Ed[q] << 16);
+    ex.uc[2 * (size_t)v] = make_uint4(c[0], c[1], c[2], c[3]);
+    ex.uc[2 * (size_t)v + 1] = make_uint4(c[4], 0u, 0u, 0u);
+  }
+  const double ir = rcp64(w[0]);
   const double u = w[1] * ir, vv = w[2] * ir, ww = w[3] * ir;
   const double p = g1 * (w[4] - 0.5 * (w[1] * u + w[2] * vv + w[3] * ww));
   const double f[16] = {w[1], w[1] * u + p, w[2] * u, w[3] * u, (w[4] + p) * u,
@@ -217,181 +80,6 @@ __global__ void __launch_bounds__(256) k3_vertex(int V, const double* __restrict
 #pragma unroll
     for (int i = 0; i < 8; ++i) o[i] = make_double2(f[2 * i], f[2 * i + 1]);
   }
-}
-
-// ------------------------------------------------------------------ k3_edge
-// One thread per edge.  Stencil ids (6 x E), frame (9 x E), w5 (40 x E) and w3 (18 x E) are
-// structure-of-arrays streams; node data are gathered from Ua.  h: 8 doubles per edge (5 used); FX:
-// record 3 V + e instead.
-template <bool FX>
-__global__ void __launch_bounds__(128) k3_edge(int E, int V, const int32_t* __restrict__ sten,
-                                               const double* __restrict__ frame,
-                                               const double* __restrict__ w5,
-                                               const double* __restrict__ w3,
-                                               const double* __restrict__ Ua,
-                                               double* __restrict__ h, int4* __restrict__ rec,
-                                               Phys3 ph, unsigned* __restrict__ err) {
-  const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e >= E) return;
-  int s[6];
-  bool bad = false;
-#pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    s[k] = __ldg(sten + (size_t)k * E + e);
-    bad |= (unsigned)s[k] >= (unsigned)V;
-  }
-  if (bad) {
-    atomicOr(err, kErrIndex);
-    return;
-  }
-  const double g1 = ph.g1;
-  Eig st;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    st.n[k] = __ldg(frame + (size_t)k * E + e);
-    st.t1[k] = __ldg(frame + (size_t)(3 + k) * E + e);
-    st.t2[k] = __ldg(frame + (size_t)(6 + k) * E + e);
-  }
-  double wi[5], wj[5];
-#pragma unroll
-  for (int q = 0; q < 5; ++q) {
-    wi[q] = __ldg(Ua + (size_t)20 * s[2] + q);
-    wj[q] = __ldg(Ua + (size_t)20 * s[3] + q);
-  }
-  roe_state(wi, wj, g1, st);
-  // FP32 sensor: characteristic values of the six nodes' differences from the tail state (the
-  // WENO indicators see differences only), each difference formed in FP64 and rounded once;
-  // and the 5-node sums of both sides in conservative variables, in FP64
-  EigF sf;
-  to_f32(st, sf);
-  float cf[6][5];
-  double W[2][5];
-#pragma unroll
-  for (int q = 0; q < 5; ++q) W[0][q] = W[1][q] = 0.0;
-#pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    double a[20];
-    const double2* src = reinterpret_cast<const double2*>(Ua + (size_t)20 * s[k]);
-#pragma unroll
-    for (int i = 0; i < 10; ++i) {
-      const double2 t = __ldg(src + i);
-      a[2 * i] = t.x;
-      a[2 * i + 1] = t.y;
-    }
-    float d[5];
-#pragma unroll
-    for (int q = 0; q < 5; ++q) d[q] = d2f_rn(a[q] - wi[q]);
-    to_char_f(sf, d, cf[k]);
-#pragma unroll
-    for (int side = 0; side < 2; ++side) {
-      const int j = k - side;                 // node index within this side's five
-      if (j < 0 || j > 4) continue;
-#pragma unroll
-      for (int dd = 0; dd < 4; ++dd) {
-        const double wt = __ldg(w5 + (size_t)(20 * side + 4 * j + dd) * E + e);
-#pragma unroll
-        for (int q = 0; q < 5; ++q) W[side][q] = fma(wt, a[5 * dd + q], W[side][q]);
-      }
-    }
-  }
-  // per side and characteristic component: FP32 decision, taken again in FP64 (on the node
-  // values' characteristic values, as the 3-node candidates need) inside the guard band or on a
-  // non-finite FP32 sum; weighted 3-node values where the decision is rough
-#pragma unroll
-  for (int side = 0; side < 2; ++side) {
-    unsigned flag = 0;                        // rough in FP32, or undecided
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      if (ph.force_branch == 1) break;
-      if (ph.force_branch == 2) {
-        flag |= 1u << q;
-        continue;
-      }
-      float t0, S;
-      if (side == 0) weno3f(cf[0][q], cf[1][q], cf[2][q], cf[3][q], cf[4][q], ph.epsf, t0, S);
-      else           weno3f(cf[5][q], cf[4][q], cf[3][q], cf[2][q], cf[1][q], ph.epsf, t0, S);
-      const float mlo = t0 - ph.sens_lof * S, mhi = ph.sens_hif * S - t0;
-      const bool smooth = mlo > 0.f && mhi > 0.f;
-      const bool clear = isfinite(S) && fabsf(mlo) > kGuard3 * S && fabsf(mhi) > kGuard3 * S;
-      if (!smooth || !clear) flag |= 1u << q;
-    }
-    if (!flag) continue;
-    double C[5];
-    to_char(st, W[side], C);
-    bool any = false;
-    const double* w = w3 + (size_t)(9 * side) * E + e;
-#pragma unroll
-    for (int q = 0; q < 5; ++q) {
-      if (!((flag >> q) & 1u)) continue;
-      double cq[5];
-#pragma unroll
-      for (int j = 0; j < 5; ++j) {
-        const int k = side == 0 ? j : 5 - j;
-        double a[5], c[5];
-#pragma unroll
-        for (int r = 0; r < 5; ++r) a[r] = __ldg(Ua + (size_t)20 * s[k] + r);
-        to_char(st, a, c);
-        cq[j] = c[q];
-      }
-      double o[3], S;
-      weno3(cq[0], cq[1], cq[2], cq[3], cq[4], ph.eps, o, S);
-      const bool smooth = o[0] > ph.sens_lo * S && o[0] < ph.sens_hi * S;
-      if (ph.force_branch != 2 && smooth) continue;
-      const double iS = 1.0 / S;
-      double wt[9];
-#pragma unroll
-      for (int i = 0; i < 9; ++i) wt[i] = __ldg(w + (size_t)i * E);
-      const double c1 = wt[0] * cq[0] + wt[1] * cq[1] + wt[2] * cq[2];
-      const double c2 = wt[3] * cq[1] + wt[4] * cq[2] + wt[5] * cq[3];
-      const double c3 = wt[6] * cq[2] + wt[7] * cq[3] + wt[8] * cq[4];
-      C[q] = (o[0] * iS) * c1 + (o[1] * iS) * c2 + (o[2] * iS) * c3;
-      any = true;
-    }
-    if (any) from_char(st, C, W[side]);
-  }
-  // positivity (R16): fall back to the end state of that side
-  if (!admissible3(W[0]))
-#pragma unroll
-    for (int q = 0; q < 5; ++q) W[0][q] = wi[q];
-  if (!admissible3(W[1]))
-#pragma unroll
-    for (int q = 0; q < 5; ++q) W[1][q] = wj[q];
-  // Roe's flux along n with Harten's fix on all five waves
-  Eig r;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) {
-    r.n[k] = st.n[k];
-    r.t1[k] = st.t1[k];
-    r.t2[k] = st.t2[k];
-  }
-  roe_state(W[0], W[1], g1, r);
-  double dw[5], al[5];
-#pragma unroll
-  for (int q = 0; q < 5; ++q) dw[q] = W[1][q] - W[0][q];
-  to_char(r, dw, al);
-  const double lam[5] = {r.qn - r.c, r.qn, r.qn, r.qn, r.qn + r.c};
-  const double del = ph.harten * r.c, i2del = ph.half_inv_harten * r.ic;
-#pragma unroll
-  for (int i = 0; i < 5; ++i) {
-    double a = fabs(lam[i]);
-    if (a < del) a = (lam[i] * lam[i] + del * del) * i2del;
-    al[i] *= a;
-  }
-  double diss[5], fl[5], fr[5];
-  from_char(r, al, diss);
-  normal_flux3(W[0], r.irl, r.pl, r.n, fl);
-  normal_flux3(W[1], r.irr, r.pr, r.n, fr);
-  double hq[5];
-#pragma unroll
-  for (int q = 0; q < 5; ++q) hq[q] = 0.5 * (fl[q] + fr[q]) - 0.5 * diss[q];
-  if (FX) {
-    st_record3(rec, (size_t)3 * V + e, hq);
-    return;
-  }
-  double* o = h + (size_t)8 * e;
-  reinterpret_cast<double2*>(o)[0] = make_double2(hq[0], hq[1]);
-  reinterpret_cast<double2*>(o)[1] = make_double2(hq[2], hq[3]);
-  o[4] = hq[4];
 }
 
 // ------------------------------------------------------------------ k3_div
@@ -755,20 +443,8 @@ cudaError_t launch3_pack(const DevMesh3& m, int* flag, cudaStream_t s) {
 cudaError_t launch3_vertex(const DevMesh3& m, const double* U, const Phys3& ph, cudaStream_t s) {
   if (m.V == 0) return cudaSuccess;
   const unsigned nb = (unsigned)((m.V + 255) / 256);
-  if (div3_lanes(m) == 0) k3_vertex<true><<<nb, 256, 0, s>>>(m.V, U, m.Ua, m.FGK, m.fx.rec, ph.g1);
-  else                    k3_vertex<false><<<nb, 256, 0, s>>>(m.V, U, m.Ua, m.FGK, m.fx.rec, ph.g1);
-  return cudaGetLastError();
-}
-
-cudaError_t launch3_edge(const DevMesh3& m, const Phys3& ph, cudaStream_t s) {
-  if (m.E == 0) return cudaSuccess;
-  const unsigned nb = (unsigned)((m.E + 127) / 128);
-  if (div3_lanes(m) == 0)
-    k3_edge<true><<<nb, 128, 0, s>>>(m.E, m.V, m.sten, m.frame, m.w5, m.w3, m.Ua, m.h, m.fx.rec, ph,
-                                     m.err);
-  else
-    k3_edge<false><<<nb, 128, 0, s>>>(m.E, m.V, m.sten, m.frame, m.w5, m.w3, m.Ua, m.h, m.fx.rec, ph,
-                                     m.err);
+  if (div3_lanes(m) == 0) k3_vertex<true><<<nb, 256, 0, s>>>(m.V, U, m.Ua, m.FGK, m.fx.rec, edge3_fx(m), ph.g1);
+  else                    k3_vertex<false><<<nb, 256, 0, s>>>(m.V, U, m.Ua, m.FGK, m.fx.rec, edge3_fx(m), ph.g1);
   return cudaGetLastError();
 }
 

@@ -16,6 +16,14 @@ cudaError_t launch3_div(const DevMesh3& m, const double* Us, const double* Un, d
 
 // Packs m.cv and m.ce into m.fx; *flag (device) is set if a coefficient does not fit.
 cudaError_t launch3_pack(const DevMesh3& m, int* flag, cudaStream_t s);
+// Packs m.w5 into m.ex (and the frame in FP32); *flag (device) is set if a weight does not fit.
+cudaError_t launch3_pack_w5(const DevMesh3& m, int* flag, cudaStream_t s);
+// The edges' fixed-point arrays, without nodes and weights (the sums in FP64) where these do not fit.
+inline Edge3Fx edge3_fx(const DevMesh3& m) {
+  Edge3Fx x = m.ex;
+  if (!m.ex_ok) x.uf = nullptr;
+  return x;
+}
 // The lanes of the next launches: 0 the fixed-point divergence, else the FP64 one.
 inline int div3_lanes(const DevMesh3& m) { return m.lanes ? m.lanes : m.fx_ok ? 0 : 4; }
 

@@ -7,6 +7,7 @@
 
 struct int2;   // CUDA's vector types
 struct int4;
+struct uint4;
 
 namespace hfd {
 
@@ -45,12 +46,26 @@ struct Div3Fx {
   int4* rec = nullptr;          // 3 V + E records of 3: five pairs and a code word
 };
 
+// What the edge kernels read and write in fixed point.
+struct Edge3Fx {
+  int4* uf = nullptr;           // V x 10: a node's 20 pairs, by value and derivatives components 0..3, then 4
+  uint4* uc = nullptr;          // V x 2: code word per component (values | derivatives << 16)
+  int4* w5f = nullptr;          // 20 x E: limb pairs of two weights, order of w5
+  int2* w5e = nullptr;          // E: exponents (see k3_pack_w5)
+  float* framef = nullptr;      // 9 x E: the frame in FP32
+  int2* list = nullptr;         // edges left to k3_edge_weno: {edge, components}
+  double* listw = nullptr;      // their 5-node sums: 6 doubles per side, 5 used
+  int* count = nullptr;
+};
+
 // Device arrays of a 3D mesh.
 struct DevMesh3 {
   int V = 0, E = 0;
   int lanes = 0;                // threads per vertex in the FP64 gather (1, 2, 4); 0: fixed point if fx
   bool fx_ok = false;           // the rows fit fixed point
   Div3Fx fx;
+  bool ex_ok = false;           // the edges' weights fit fixed point
+  Edge3Fx ex;
   int32_t* sten = nullptr;      // 6 x E (SoA)
   double* frame = nullptr;      // 9 x E (SoA)
   double* w5 = nullptr;         // 40 x E (SoA)
@@ -68,7 +83,7 @@ struct DevMesh3 {
 
 struct Phys3 {
   double gamma, g1, eps, sens_lo, sens_hi, harten, half_inv_harten;
-  float epsf, sens_lof, sens_hif;   // the sensor's constants rounded once to FP32 (host)
+  float g1f, epsf, sens_lof, sens_hif;   // the sensor's constants rounded once to FP32 (host)
   int force_branch;
 };
 

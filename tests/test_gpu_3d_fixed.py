@@ -84,3 +84,28 @@ def test_rows_with_non_finite_fluxes_match_fp64():
     U[4, 100] = U[4, 101]
     U[0, 300] = U[0, 301]
     assert (np.abs(R.numpy() - P.numpy())[ok] <= _bound(M, U)[ok]).all()
+
+
+@pytest.mark.parametrize("shape", [(7, 7, 7), (12, 7, 10)])
+@pytest.mark.parametrize("force", [0, 1, 2])
+def test_edge_sums_in_fixed_point_match_fp64(shape, force):
+    """A weight that is not finite turns the edges' fixed-point sums off for the whole mesh; rows that do
+    not read that edge agree.  A sum of 20 products is off by 20 units of 2^-53 of sum |w| |v| < 4 |v| either
+    way, a flux by at most 10 times its states: within 2 * 800 units of the row's sum |c| |f|."""
+    from paper_2109_01286_gb300 import hfd3d
+    nx, ny, nz = shape
+    m = T.periodic_tet_box(nx, ny, nz, 10.0, 10.0 * ny / nx, 10.0 * nz / nx, seed=3)
+    M = hfd3d.Mesh3(m, force_branch=force)
+    U = T.vortex_tube(m)
+    Ud = torch.from_numpy(U).cuda()
+    R = M.residual(Ud).cpu().numpy()
+    M.check()
+    w5 = M.prep_get("w5").copy()
+    w5.reshape(-1, 40)[5, 7] = np.nan
+    M.prep_set("w5", w5)
+    P = M.residual(Ud).cpu().numpy()
+    torch.cuda.synchronize()
+    ep, ei = M.prep_get("eptr"), M.prep_get("eidx")
+    far = np.array([5 not in ei[ep[v]:ep[v + 1]] for v in range(U.shape[1])])
+    assert far.any() and np.isfinite(P[:, far]).all()
+    assert (np.abs(R - P)[:, far] <= 2 * _bound(M, U)[:, far]).all()
