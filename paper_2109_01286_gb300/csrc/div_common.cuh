@@ -87,40 +87,51 @@ struct RowShare {
   static __device__ __forceinline__ int count(int lane) { return G >= 8 && (lane & 1) ? 1 : kMax; }
 };
 
-// Writes R, or the Runge-Kutta stage combination a*Un + b*(Us + dt*R), for `count` rows row[i] of
-// vertex r; flags non-finite values and non-positive densities in the error word.
-template <int N>
-__device__ __forceinline__ void finish_rows(int r, int lane, int count, const int* row, const double* R,
-                                            int V, const StageArgs& sa,
+// Writes R, or the Runge-Kutta stage combination a*Un + b*(Us + dt*R), for the rows of vertex r that
+// this lane of G holds, value(i) being R of its i-th; flags non-finite values and non-positive
+// densities in the error word.
+template <int G, typename F>
+__device__ __forceinline__ void finish_rows(int r, int lane, F value, int V, const StageArgs& sa,
                                             const int32_t* __restrict__ vmem,
                                             const unsigned long long* dtbits, double cfl,
                                             double* dt_last, unsigned* err) {
   const double* __restrict__ Us = sa.Us;
   const double* __restrict__ Un = sa.Un;
+  double* out = sa.out;
+  const int mode = sa.mode;
+  const double a = sa.a, b = sa.b, dt_fixed = sa.dt_fixed;
   // time step of this vertex's mesh (a batch holds several meshes, each with its own CFL step)
   const int mem = vmem ? __ldg(vmem + r) : 0;
-  const double dt = sa.dt_fixed > 0.0 ? sa.dt_fixed
-                    : sa.dt_member ? __ldg(sa.dt_member + mem)
-                                   : cfl * __longlong_as_double((long long)dtbits[mem]);
-  if (sa.mode == DIV_STAGE && lane == 0 && dt_last && (r == 0 || (vmem && __ldg(vmem + r - 1) != mem)))
+  double dt = dt_fixed > 0.0 ? dt_fixed
+               : sa.dt_member ? __ldg(sa.dt_member + mem)
+                              : cfl * __longlong_as_double((long long)dtbits[mem]);
+  if (mode == DIV_STAGE && lane == 0 && dt_last && (r == 0 || (vmem && __ldg(vmem + r - 1) != mem)))
     dt_last[mem] = dt;
+  // rows held by this lane after the reduce-scatter: base .. base + per - 1
+  int per = G == 1 ? 12 : G == 2 ? 6 : 3;
+  int base = (G >= 2 && (lane & (G / 2)) ? 6 : 0) + (G >= 4 && (lane & (G / 4)) ? 3 : 0);
+  if (G >= 8) {
+    if (lane & 1) { base += 2; per = 1; } else { per = 2; }
+  }
   unsigned bad = 0;
 #pragma unroll
-  for (int i = 0; i < N; ++i) {
-    if (i >= count) break;
-    const size_t idx = (size_t)row[i] * V + r;
+  for (int i = 0; i < 12 / (G >= 8 ? 4 : G); ++i) {
+    if (i >= per) break;
+    int k = base + i;
+    double R = value(i);
+    size_t idx = (size_t)k * V + r;
     double o;
-    if (sa.mode == DIV_RESIDUAL) {
-      o = R[i];
+    if (mode == DIV_RESIDUAL) {
+      o = R;
     } else {
       // explicit roundings, so that every kernel holding this code (four-launch, fixed-point,
       // persistent) gives the same bits: one FMA, one multiply, one FMA
-      o = __dmul_rn(sa.b, __fma_rn(dt, R[i], Us[idx]));
-      if (sa.a != 0.0) o = __fma_rn(sa.a, Un[idx], o);   // the first stage does not read the base state
+      o = __dmul_rn(b, __fma_rn(dt, R, Us[idx]));
+      if (a != 0.0) o = __fma_rn(a, Un[idx], o);   // the first stage does not read the base state
     }
-    sa.out[idx] = o;
+    out[idx] = o;
     if (!finite_bits(o)) bad |= ERRBIT_NONFINITE;
-    if (sa.mode == DIV_STAGE && row[i] == 0 && !(o > 0.0)) bad |= ERRBIT_POSITIVITY;
+    if (mode == DIV_STAGE && k == 0 && !(o > 0.0)) bad |= ERRBIT_POSITIVITY;
   }
   if (bad) atomicOr(err, bad);
 }

@@ -321,14 +321,10 @@ __global__ void __launch_bounds__(128, 4) k_div_fx(DivFx m, StageArgs sa, const 
     }
   }
   if (!live) return;
-  int row[RowShare<G>::kMax];
 #pragma unroll
-  for (int i = 0; i < RowShare<G>::kMax; ++i) {
-    row[i] = base + i;
-    if (odd && i < RowShare<G>::count(lane)) R[i] = fallback_sum(m, r, row[i] >> 2, row[i] & 3, VISC);
-  }
-  finish_rows<RowShare<G>::kMax>(r, lane, RowShare<G>::count(lane), row, R, m.V, sa, vmem, dtbits, cfl,
-                                 dt_last, err);
+  for (int i = 0; i < RowShare<G>::kMax; ++i)
+    if (odd && i < RowShare<G>::count(lane)) R[i] = fallback_sum(m, r, (base + i) >> 2, (base + i) & 3, VISC);
+  finish_rows<G>(r, lane, [&](int i) { return R[i]; }, m.V, sa, vmem, dtbits, cfl, dt_last, err);
 }
 
 // ------------------------------------------------------------------ coefficients to fixed point

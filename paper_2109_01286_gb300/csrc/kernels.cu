@@ -1281,14 +1281,7 @@ __device__ __forceinline__ void div_finish(int r, int lane, bool live, T* acc, i
                                            double* dt_last, unsigned* err) {
   reduce_scatter12<G>(acc, lane);
   if (!live) return;
-  double R[RowShare<G>::kMax];
-#pragma unroll
-  for (int i = 0; i < RowShare<G>::kMax; ++i) R[i] = -(double)acc[i];
-  int row[RowShare<G>::kMax];
-#pragma unroll
-  for (int i = 0; i < RowShare<G>::kMax; ++i) row[i] = RowShare<G>::first(lane) + i;
-  finish_rows<RowShare<G>::kMax>(r, lane, RowShare<G>::count(lane), row, R, V, sa, vmem, dtbits, cfl,
-                                 dt_last, err);
+  finish_rows<G>(r, lane, [&](int i) { return -(double)acc[i]; }, V, sa, vmem, dtbits, cfl, dt_last, err);
 }
 
 template <typename T, int G, bool VISC>
