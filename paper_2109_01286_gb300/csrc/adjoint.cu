@@ -115,7 +115,7 @@ __device__ __forceinline__ void adj_edge_front(
   for (int r = 0; r < 4; ++r) { wi[r] = Ua[(size_t)s[2] * 12 + r]; wj[r] = Ua[(size_t)s[3] * 12 + r]; }
   // ---- forward: the 5-node sums and the FP32 sensor exactly as the edge kernel takes them
   float cf6[6][4];
-  if (fx.uf && edge_fixed64(e, Ef, s, fx, (float)nx, (float)ny, ph, W5, cf6)) {
+  if (fx.uf && edge_fixed64<false>(e, Ef, s, fx, (float)nx, (float)ny, ph, W5, cf6)) {
     sensor32(cf6, ph, rough, amb);
     return;
   }

@@ -124,8 +124,20 @@ __device__ __forceinline__ void sensor32(const float (*cf)[4], const Phys& ph, u
 // scale top_q = max(value code, derivative code + d).  Also the sensor's characteristic values of
 // the differences from the tail state: the integer differences, rounded to FP32.  False: some value
 // is not finite, and nothing is written.
+// SHARED: the thread's weights are in shared memory (stage_w5), at ws.
+constexpr int kEdgeBlock = 128;                    // threads of a block that stages them, at most
+__device__ __forceinline__ void stage_w5(int2* ws, const EdgeFx& fx, int Ef, int e) {
+#pragma unroll
+  for (int i = 0; i < 30; ++i)
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(
+                     (unsigned)__cvta_generic_to_shared(ws + kEdgeBlock * i)),
+                 "l"(fx.w5f + (size_t)i * Ef + e)
+                 : "memory");
+}
+template <bool SHARED>
 __device__ __forceinline__ bool edge_fixed64(int e, int Ef, const int* s, const EdgeFx& fx, float nx, float ny,
-                                             const Phys& ph, double (*W)[4], float (*cf)[4]) {
+                                             const Phys& ph, double (*W)[4], float (*cf)[4],
+                                             const int2* ws = nullptr) {
   constexpr int L = 29;
   uint4 E = __ldg(fx.uc + s[0]);
 #pragma unroll
@@ -192,6 +204,7 @@ __device__ __forceinline__ bool edge_fixed64(int e, int Ef, const int* s, const 
     roe_avg(fi, fj, ph.g1f, u, v, H, cs);
     left_ev(u, v, cs, nx, ny, ph.g1f, Lf);
   }
+  if (SHARED) asm volatile("cp.async.wait_all;" ::: "memory");
   long long hh[2][4], x[2][4];
 #pragma unroll
   for (int i = 0; i < 2; ++i)
@@ -217,7 +230,8 @@ __device__ __forceinline__ bool edge_fixed64(int e, int Ef, const int* s, const 
 #pragma unroll
       for (int side = 0; side < 2; ++side) {
         if (k < side || k > 4 + side) continue;
-        const int2 w = __ldg(fx.w5f + (size_t)(15 * side + 3 * (k - side) + g) * Ef + e);
+        const int i = 15 * side + 3 * (k - side) + g;
+        const int2 w = SHARED ? ws[kEdgeBlock * i] : __ldg(fx.w5f + (size_t)i * Ef + e);
 #pragma unroll
         for (int q = 0; q < 4; ++q) fx_fma(hh[side][q], x[side][q], w.x, w.y, bh[q], bl[q]);
       }

@@ -737,7 +737,8 @@ __device__ __forceinline__ void edge_body64(int e, int Ef, int V, const int32_t*
                                             const double* __restrict__ nrm, const double* __restrict__ w5,
                                             const double* __restrict__ w3, const double* __restrict__ Ua,
                                             double* __restrict__ h, const Phys& ph, unsigned* err,
-                                            uint8_t* __restrict__ dbg, const EdgeFx& fx) {
+                                            uint8_t* __restrict__ dbg, const EdgeFx& fx,
+                                            const int2* ws = nullptr) {
   const double g1 = ph.g1;
   int s[6];
 #pragma unroll
@@ -748,7 +749,7 @@ __device__ __forceinline__ void edge_body64(int e, int Ef, int V, const int32_t*
   ld4(Ua + (size_t)s[3] * 12, wj);
   double W[2][4];
   float cf[6][4];
-  if (!fx.uf || !edge_fixed64(e, Ef, s, fx, d2f_rn(nx), d2f_rn(ny), ph, W, cf)) {
+  if (!fx.uf || !edge_fixed64<LIST>(e, Ef, s, fx, d2f_rn(nx), d2f_rn(ny), ph, W, cf, ws)) {
 #pragma unroll
     for (int r = 0; r < 4; ++r) W[0][r] = W[1][r] = 0.0;
     // FP32 left eigenvectors at the Roe state of the edge ends (sensor only)
@@ -1002,7 +1003,7 @@ __global__ void __launch_bounds__(128, 5) k_edge(int Ef, int V, const int32_t* _
 
 // FP64 edges whose two sides take the 5-node branch; the others are listed.
 // 128 registers (some spilled): 4 blocks of 128 an SM; 3 or 5 measured 4 and 2 percent slower.
-__global__ void __launch_bounds__(128, 4) k_edge64(int Ef, int V, const int32_t* __restrict__ sten,
+__global__ void __launch_bounds__(kEdgeBlock, 4) k_edge64(int Ef, int V, const int32_t* __restrict__ sten,
                                                    const double* __restrict__ nrm,
                                                    const double* __restrict__ w5,
                                                    const double* __restrict__ w3,
@@ -1010,7 +1011,10 @@ __global__ void __launch_bounds__(128, 4) k_edge64(int Ef, int V, const int32_t*
                                                    Phys ph, unsigned* err, uint8_t* __restrict__ dbg,
                                                    EdgeFx fx) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < Ef) edge_body64<true>(e, Ef, V, sten, nrm, w5, w3, Ua, h, ph, err, dbg, fx);
+  __shared__ int2 ws[30 * kEdgeBlock];
+  if (e >= Ef) return;
+  if (fx.uf) stage_w5(ws + threadIdx.x, fx, Ef, e);
+  edge_body64<true>(e, Ef, V, sten, nrm, w5, w3, Ua, h, ph, err, dbg, fx, ws + threadIdx.x);
 }
 
 // edge_fixed64's 5-node sum of one side's component q (the same integers, so the same bits).
