@@ -568,6 +568,7 @@ hfd_status upload(const hfd::Prep& P, int precision, hfd_mesh* m) {
   m->ph.mu = o.mu;
   m->ph.R_gas = o.R_gas;
   m->ph.kappa = o.mu * (o.gamma * o.R_gas / (o.gamma - 1.0)) / o.prandtl;
+  m->ph.kappa_R = m->ph.kappa / o.R_gas;
   m->ph.flux = o.flux;
   m->ph.force_branch = o.force_branch;
   m->ph.finish();

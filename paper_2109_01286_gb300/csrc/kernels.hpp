@@ -10,6 +10,7 @@ namespace hfd {
 struct Phys {
   double gamma, eps, sens_lo, sens_hi, harten, cfl;
   double mu, kappa, R_gas;      // viscous model (Sec. 2.3; constant mu, kappa = mu c_p / Pr)
+  double kappa_R;               // kappa / R_gas
   int flux;                     // 0 Roe (Harten's fix), 1 Rusanov
   int force_branch;             // 0 sensor, 1 every side 5-node, 2 every side 3-node WENO
   double g1;                    // gamma - 1
