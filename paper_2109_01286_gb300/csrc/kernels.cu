@@ -1871,29 +1871,31 @@ __global__ void __launch_bounds__(kStageThreads) k_div_staged(
 // Ghost refresh of state U (R14): a transmissive ghost copies its donor in U and zeroes the
 // derivative normal to its boundary; a fixed ghost (donor -1, wall bands holding given values)
 // takes its values from the step's base state `base` (nothing to do when U is the base).
-__device__ __forceinline__ void ghost_body(int g, int Gn, int V, const int32_t* gid,
+// The rows r0 .. r0 + N - 1 are read before any is written: alternating, each read waits for the
+// one before (the compiler must assume that a write to U changes it).
+template <int N>
+__device__ __forceinline__ void ghost_body(int g, int r0, int Gn, int V, const int32_t* gid,
                                            const int32_t* gdonor, const int32_t* gflags, double* U,
                                            const double* base, unsigned* err) {
   if (g >= Gn) return;
   int t = chk_idx(gid[g], V, err), d = gdonor[g], f = gflags[g];
   if (d >= 0) d = chk_idx(d, V, err);
-  if (d < 0) {
-    if (base != U)
+  if (d < 0 && base == U) return;
+  const double* src = d < 0 ? base + t : U + d;
+  double val[N];
 #pragma unroll
-      for (int r = 0; r < 12; ++r) U[(size_t)r * V + t] = base[(size_t)r * V + t];
-    return;
-  }
+  for (int i = 0; i < N; ++i) val[i] = src[(size_t)(r0 + i) * V];
 #pragma unroll
-  for (int r = 0; r < 12; ++r) {
-    double val = U[(size_t)r * V + d];
-    if ((r >= 4 && r < 8 && (f & 1)) || (r >= 8 && (f & 2))) val = 0.0;
-    U[(size_t)r * V + t] = val;
+  for (int i = 0; i < N; ++i) {
+    const int r = r0 + i;
+    if (d >= 0 && ((r >= 4 && r < 8 && (f & 1)) || (r >= 8 && (f & 2)))) val[i] = 0.0;
+    U[(size_t)r * V + t] = val[i];
   }
 }
 
 __global__ void k_ghost(int Gn, int V, const int32_t* gid, const int32_t* gdonor,
                         const int32_t* gflags, double* U, const double* base, unsigned* err) {
-  ghost_body(blockIdx.x * blockDim.x + threadIdx.x, Gn, V, gid, gdonor, gflags, U, base, err);
+  ghost_body<4>(blockIdx.x * blockDim.x + threadIdx.x, 4 * blockIdx.y, Gn, V, gid, gdonor, gflags, U, base, err);
 }
 
 // min over the active vertices of each mesh of l_min / (|u| + c) (R12), in two passes without
@@ -2037,7 +2039,7 @@ __global__ void __launch_bounds__(128) k_stage(KernelArgs ka, StageArgs sa, Phys
   double* U = const_cast<double*>(sa.Us);
   if (do_ghost) {
     for (int g = tid; g < ka.G; g += stride)
-      ghost_body(g, ka.G, ka.V, ka.gid, ka.gdonor, ka.gflags, U, sa.Un, ka.err);
+      ghost_body<12>(g, 0, ka.G, ka.V, ka.gid, ka.gdonor, ka.gflags, U, sa.Un, ka.err);
     if (!grid_barrier(ka.bar, nb, ka.err, ka.spins)) return;
   }
   __shared__ float s0f[4];
@@ -2089,7 +2091,7 @@ KernelArgs kernel_args(const DevMesh& m) {
 
 cudaError_t launch_ghost(const DevMesh& m, double* U, const double* base, cudaStream_t s) {
   if (m.G == 0) return cudaSuccess;
-  k_ghost<<<blocks(m.G, 256), 256, 0, s>>>(m.G, m.V, m.gid, m.gdonor, m.gflags, U, base, m.err);
+  k_ghost<<<dim3(blocks(m.G, 64), 3), 64, 0, s>>>(m.G, m.V, m.gid, m.gdonor, m.gflags, U, base, m.err);
   return cudaGetLastError();
 }
 
