@@ -2133,6 +2133,10 @@ cudaError_t launch_vertex(const DevMesh& m, const double* U, const Phys& ph, cud
 constexpr int kEdge8Max = 8000;
 static int edge_threads(int Ef) { return Ef <= 152 * 64 ? 32 : Ef <= 152 * 128 ? 64 : 128; }
 
+int edge_launches(const DevMesh& m) {
+  return m.Ef == 0 ? 0 : m.precision == 0 && m.Ef > kEdge8Max ? 2 : 1;
+}
+
 cudaError_t launch_edge(const DevMesh& m, const Phys& ph, cudaStream_t s) {
   if (m.Ef == 0) return cudaSuccess;
   EdgeFx fx;
