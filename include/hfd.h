@@ -343,8 +343,8 @@ hfd_status hfd_check_conversions(int64_t n, const double* x, float* f_int, float
  * four-quadrant problem and the circular Sod mesh; on low-Mach flows the energy flux's nearly
  * divergence-free part still cancels (at Mach 0.1, about 250x), and the 48-bit products leave
  * ~1e-11 relative there, against ~1e-12 for the plain form.  Speed on the four-quadrant
- * 1024x1024 mesh (GB300): the divergence 1.66 ms against 2.23 ms, the edge kernel 0.11 ms
- * slower (it forms dh), the step 11.05 ms against 12.45 ms.  The viscous rows stay FP64.
+ * 1024x1024 mesh (GB300): the divergence 1.66 ms against 2.23 ms for FP64 sums and 0.96 ms for
+ * folded = 0.  The viscous rows stay FP64.
  * folded = 0: fixed point.  Each row's coefficients and the fluxes it reads are 57-bit integers
  * relative to their largest, multiplied and summed exactly on the integer pipe (three 32x32+64-bit
  * multiply-adds per product), so that only the factors are rounded: the sums are closer to the exact

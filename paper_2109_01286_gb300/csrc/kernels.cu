@@ -2128,7 +2128,8 @@ cudaError_t launch_vertex(const DevMesh& m, const double* U, const Phys& ph, cud
 // listed for k_edge_weno), 8 lanes each in meshes of few edges, whose time is the chain of one warp:
 // 1728 edges 15 us with 8 lanes and 43 us in one pass of one thread each, 7800 edges 28 and 30 us, 12300
 // edges 36 and 30 us.  Before (one kernel, sums in FP64, 341 FP64 instructions a smooth edge): 45 us for
-// 1728 edges, 125 us for 196,600 (now 97 us, 128 FP64 instructions), 330 us for 512,000 (246 us).
+// 1728 edges, 125 us for 196,600 (now 87 us, 128 FP64 instructions), 330 us for 512,000 (237 us, its listed edges included; 248 us
+// with the weights loaded where they are used instead of copied to shared memory at the start).
 // Threads per block: an SM partition has its own FP64 unit, so blocks of 32 spread a small mesh best.
 constexpr int kEdge8Max = 8000;
 static int edge_threads(int Ef) { return Ef <= 152 * 64 ? 32 : Ef <= 152 * 128 ? 64 : 128; }

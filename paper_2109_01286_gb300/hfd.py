@@ -419,8 +419,8 @@ class Mesh:
         return out
 
     def set_fp64_div(self, folded):
-        """hfd_mesh_set_fp64_div: the folded double-float FP64 divergence (1) or the plain FP64
-        one (0)."""
+        """hfd_mesh_set_fp64_div: the folded double-float FP64 divergence (1) or the
+        fixed-point one (0)."""
         _ok(_lib.hfd_mesh_set_fp64_div(self._h, int(folded)), "hfd_mesh_set_fp64_div")
 
     def set_div_staged(self, staged):
