@@ -299,12 +299,15 @@ hfd_status hfd_mesh_set_launch(hfd_mesh* mesh, int32_t persistent, int32_t grid)
  * HFD_ERR_TIMEOUT in the error word and returns instead of waiting.  Drops captured graphs. */
 hfd_status hfd_mesh_set_barrier_limit(hfd_mesh* mesh, uint32_t polls);
 
-/* Lanes (threads) per vertex in the divergence gather: 1, 2, 4 or 8.  The default is 4 (coalesced
- * groups), and 8 for FP64 meshes of fewer than 20,000 rows, which fill the GPU better so.  Each lane
- * sums a strided share of the entries and the shares are combined by a fixed reduce-scatter, so a
- * lane count gives deterministic results that agree with the other counts to rounding; the
- * fixed-point FP64 divergence (hfd_mesh_set_fp64_div) has 4 and 8 lanes, runs 1 and 2 as 4, and
- * gives the same bits with both.  The persistent form (hfd_mesh_set_launch) has kernels for 1, 2 and 4 lanes and runs 8 as 4.  Drops
+/* Lanes (threads) per vertex in the divergence gather: 1, 2, 4 or 8.  Each lane sums a strided share
+ * of the entries and the shares are combined by a fixed reduce-scatter, so a lane count gives
+ * deterministic results that agree with the other counts to rounding.  FP64 meshes: 1 and 2 run
+ * the sums of the divergence and of the edges in FP64; 4 and 8 run them in fixed point
+ * (hfd_mesh_set_fp64_div), with the same bits for both, or in FP64 where the mesh has no fixed-point
+ * form.  The default is 4 for FP32 meshes (coalesced groups) and for FP64 ones in fixed point, 8
+ * for those of fewer than 20,000 rows, which fill the GPU better so, and 1 for FP64 meshes without
+ * that form (bound by the FP64 pipe: no cross-lane reduction).  The persistent form
+ * (hfd_mesh_set_launch) has FP64 sums for 1, 2 and 4 lanes and runs 8 as 4.  Drops
  * captured graphs.  Errors: HFD_ERR_ARG (another count, or a persistent grid set by
  * hfd_mesh_set_launch that the new count's kernel cannot hold co-resident). */
 hfd_status hfd_mesh_set_lanes(hfd_mesh* mesh, int32_t lanes);
@@ -351,8 +354,8 @@ hfd_status hfd_check_conversions(int64_t n, const double* x, float* f_int, float
  * ones than those of FP64 multiply-adds (rms error 0.15 to 0.35 of theirs) and do not depend on
  * the order of the entries or the lane count.  Rows that read a flux that is not finite are
  * evaluated in FP64.  Meshes with a row of more than 400 products (2 per vertex, 1 per edge) take
- * the plain FP64 form, as does the persistent launch: 24 FP64 multiply-adds per stencil vertex
- * and 12 per stencil edge with the lane count of hfd_mesh_set_lanes.  Drops captured graphs.
+ * the plain FP64 form, as do meshes with 1 or 2 lanes (hfd_mesh_set_lanes) and the persistent launch: 24
+ * FP64 multiply-adds per stencil vertex and 12 per stencil edge.  Drops captured graphs.
  * Errors: HFD_ERR_ARG (folded not 0 or 1), HFD_ERR_UNSUPPORTED (folded = 1 on an FP32 mesh). */
 hfd_status hfd_mesh_set_fp64_div(hfd_mesh* mesh, int32_t folded);
 

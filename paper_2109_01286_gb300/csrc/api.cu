@@ -450,6 +450,14 @@ hfd_status upload_streams(hfd_mesh* m, const hfd::Prep& P, const std::vector<int
   return HFD_OK;
 }
 
+// The lanes of the next launches: 1 and 2 run an FP64 mesh's sums in FP64, 4 and 8 in fixed point where
+// the mesh has that form.
+bool lanes_fixed(const hfd_mesh* m, int lanes) { return m->fixed_point && lanes >= 4; }
+void use_lanes(hfd_mesh* m, int lanes) {
+  m->lanes = lanes;
+  m->dm.div_fx = lanes_fixed(m, lanes) ? 1 : 0;
+}
+
 hfd_status upload(const hfd::Prep& P, int precision, hfd_mesh* m) {
   CK(cudaGetDevice(&m->device));
   m->opts = P.opts;
@@ -552,12 +560,16 @@ hfd_status upload(const hfd::Prep& P, int precision, hfd_mesh* m) {
   CK(cudaStreamCreateWithFlags(&m->cap, cudaStreamNonBlocking));
   // lanes per vertex in the divergence: the fixed-point FP64 kernel and the FP32 one take coalesced
   // groups of 4 (8 where the mesh is too small to fill the GPU, see div_fixed.cu); the plain FP64
-  // kernel is bound by the FP64 pipe and runs best without a cross-lane reduction (1)
-  m->lanes = m->opts.precision != 0 ? 4 : !d.div_fx ? 1 : d.fx.rows == 8 ? 8 : 4;
+  // kernel is bound by the FP64 pipe and runs best without a cross-lane reduction (1).  The persistent
+  // form takes the same count with FP64 sums: a step with 4 lanes and with 1 measured 238 and 517 us at
+  // 60x60, 242 and 522 at 100x100, 557 and 634 at 191x191, 2067 and 2069 at 400x400
+  m->fixed_point = d.div_fx != 0;
+  int lanes = m->opts.precision != 0 ? 4 : !d.div_fx ? 1 : d.fx.rows == 8 ? 8 : 4;
   if (const char* env = getenv("HFD_DIV_LANES")) {   // tuning override: 1, 2, 4 or 8
     int l = atoi(env);
-    if (l == 1 || l == 2 || l == 4 || l == 8) m->lanes = l;
+    if (l == 1 || l == 2 || l == 4 || l == 8) lanes = l;
   }
+  use_lanes(m, lanes);
   const hfd_options& o = P.opts;
   m->ph.gamma = o.gamma;
   m->ph.eps = o.weno_eps;
@@ -869,7 +881,7 @@ hfd_status hfd_mesh_set_lanes(hfd_mesh* m, int32_t lanes) {
       return HFD_ERR_ARG;
     }
   }
-  m->lanes = lanes;
+  use_lanes(m, lanes);
   drop_graphs(m);
   return HFD_OK;
 }
@@ -982,7 +994,7 @@ hfd_status hfd_mesh_autotune(hfd_mesh* m, const double* U, void* stream, int32_t
   CK(cudaEventCreate(&e1));
   float best = 1e30f;
   Cand pick = cands[0];
-  DevMesh dd = d;                              // the trial's divergence kernel choice
+  DevMesh dd = d;                              // the trial's choice of kernels
   const double dt = 1e-12;   // any fixed step: the work does not depend on it
   for (const Cand& c : cands) {
     float tot = 0;
@@ -994,9 +1006,10 @@ hfd_status hfd_mesh_autotune(hfd_mesh* m, const double* U, void* stream, int32_t
                                         m->ph, c.lanes, c.grid, true, s));
       } else {
         dd.div_staged = c.staged;
-        if (d.G) CK(hfd::launch_ghost(d, m->U1, m->U1, s));
-        CK(hfd::launch_vertex(d, m->U1, m->ph, s));
-        CK(hfd::launch_edge(d, m->ph, s));
+        dd.div_fx = lanes_fixed(m, c.lanes) ? 1 : 0;
+        if (d.G) CK(hfd::launch_ghost(dd, m->U1, m->U1, s));
+        CK(hfd::launch_vertex(dd, m->U1, m->ph, s));
+        CK(hfd::launch_edge(dd, m->ph, s));
         CK(hfd::launch_div(dd, m->U1, m->U1, m->U2, hfd::DIV_STAGE, 0.0, 1.0, dt, m->ph, c.lanes, s));
       }
       CK(cudaEventRecord(e1, s));
@@ -1015,7 +1028,7 @@ hfd_status hfd_mesh_autotune(hfd_mesh* m, const double* U, void* stream, int32_t
   CK(cudaMemsetAsync(d.err, 0, sizeof(unsigned), s));
   m->persistent = pick.persistent;
   m->grid = pick.grid;
-  m->lanes = pick.lanes;
+  use_lanes(m, pick.lanes);
   m->dm.div_staged = pick.staged;
   drop_graphs(m);
   if (choice) {

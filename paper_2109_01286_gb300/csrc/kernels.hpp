@@ -143,7 +143,8 @@ struct DevMesh {
   void* cvdf = nullptr;
   void* cedf = nullptr;
   double* sig = nullptr;
-  // FP64 meshes: the divergence in fixed point (div_fx = 1, unless div_df is set); k_vertex and
+  // FP64 meshes: the divergence in fixed point (div_fx = 1, unless div_df is set; 0 with chosen lanes 1
+  // and 2); k_vertex and
   // k_edge then write FG, FGv and h in its stored form
   int div_fx = 0;
   DivFx fx;

@@ -32,6 +32,7 @@ struct hfd_mesh {
   hfd::DevMesh dm;
   hfd::Phys ph{};
   int lanes = 4;                        // lanes per vertex in the divergence kernel (1, 2, 4, 8)
+  bool fixed_point = false;             // FP64: the divergence has a fixed-point form (4 and 8 lanes)
   int persistent = 0;                   // 1: one cooperative launch per RK stage
   int grid = 0;                         // blocks of the persistent launch (0: all resident)
   std::vector<int32_t> perm;            // internal -> input

@@ -400,7 +400,8 @@ class Mesh:
         _ok(_lib.hfd_mesh_set_barrier_limit(self._h, int(polls)), "hfd_mesh_set_barrier_limit")
 
     def set_lanes(self, lanes):
-        """Lanes per vertex in the divergence gather (1, 2, 4 or 8)."""
+        """Lanes per vertex in the divergence gather (1, 2, 4 or 8); on FP64 meshes 1 and 2 take FP64
+        sums, 4 and 8 fixed-point ones."""
         _ok(_lib.hfd_mesh_set_lanes(self._h, int(lanes)), "hfd_mesh_set_lanes")
 
     def autotune(self, U, stream=None):
