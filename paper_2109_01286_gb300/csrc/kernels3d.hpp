@@ -24,7 +24,8 @@ inline Edge3Fx edge3_fx(const DevMesh3& m) {
   if (!m.ex_ok) x.uf = nullptr;
   return x;
 }
-// The lanes of the next launches: 0 the fixed-point divergence, else the FP64 one.
-inline int div3_lanes(const DevMesh3& m) { return m.lanes ? m.lanes : m.fx_ok ? 0 : 4; }
+// The lanes of the next launches: 0 the fixed-point divergence, which 4 lanes (the default) stand for where the
+// rows have that form, else the FP64 one.
+inline int div3_lanes(const DevMesh3& m) { return m.lanes == 4 && m.fx_ok ? 0 : m.lanes; }
 
 }  // namespace hfd

@@ -61,7 +61,7 @@ struct Edge3Fx {
 // Device arrays of a 3D mesh.
 struct DevMesh3 {
   int V = 0, E = 0;
-  int lanes = 0;                // threads per vertex in the FP64 gather (1, 2, 4); 0: fixed point if fx
+  int lanes = 4;                // chosen lanes (1, 2: the FP64 gather; 4: fixed point if fx_ok)
   bool fx_ok = false;           // the rows fit fixed point
   Div3Fx fx;
   bool ex_ok = false;           // the edges' weights fit fixed point
