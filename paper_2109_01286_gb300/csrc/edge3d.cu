@@ -268,7 +268,7 @@ __device__ __forceinline__ bool sums_fixed(int e, int E, const int* s, const Edg
 #pragma unroll
   for (int q = 0; q < 5; ++q) {
     top[q] = max((int)(M.c[q] & 0xffffu), (int)(M.c[q] >> 16) + we.y);
-    unit[q] = __int_as_float((min(max(top[q] - 1022, -98), 127) - (L - 1) + 127) << 23);
+    unit[q] = exp2_f32(top[q] - 1022 - (L - 1));
   }
   // a pair's limbs at its component's scale (far: some shift of the node is 32 or more)
   auto limbs = [&](int hi, int lo, int d, bool far, int& bh, int& bl) {

@@ -2,6 +2,7 @@
 // (adjoint.cu): states, sensor, and the 5-node sums in fixed point.
 #pragma once
 #include "fixed_point.cuh"
+#include "fp_convert.cuh"
 #include "kernels.hpp"
 
 namespace hfd {
@@ -155,7 +156,7 @@ __device__ __forceinline__ bool edge_fixed64(int e, int Ef, const int* s, const 
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
     top[q] = max(Ew[q], Ed[q] + we.y);
-    unit[q] = __int_as_float((min(max(top[q] - 1022, -98), 127) - (L - 1) + 127) << 23);
+    unit[q] = exp2_f32(top[q] - 1022 - (L - 1));
   }
   // a node's codes, read again where they are used (L1) rather than held for all six nodes; its shifts;
   // and the limbs of its four values (g = 0), x derivatives (1) or y derivatives (2)

@@ -30,4 +30,10 @@ __device__ __forceinline__ float d2f_rn(double x) {
   const unsigned bits = e >= -126 ? ((unsigned)(e + 126) << 23) + qr : qr;
   return __uint_as_float(sign | bits);
 }
+
+// 2^e as a float: infinity above its range, subnormal or zero below, so that integers times it leave FP32's range
+// where the value's own conversion would.
+__device__ __forceinline__ float exp2_f32(int e) {
+  return __int_as_float(e >= -126 ? (min(e, 128) + 127) << 23 : e >= -149 ? 1 << (e + 149) : 0);
+}
 }  // namespace hfd
