@@ -243,6 +243,12 @@ __device__ __forceinline__ Codes3 ld_codes3(const uint4* uc, int v) {
   const uint4 a = __ldg(uc + (size_t)2 * v);
   return {{a.x, a.y, a.z, a.w, __ldg(reinterpret_cast<const unsigned*>(uc + (size_t)2 * v + 1))}};
 }
+__device__ __forceinline__ Codes3 max_codes3(const Codes3& a, const Codes3& b) {
+  Codes3 m;
+#pragma unroll
+  for (int q = 0; q < 5; ++q) m.c[q] = __vmaxu2(a.c[q], b.c[q]);
+  return m;
+}
 __device__ __forceinline__ bool any_raw3(const Codes3& E) {
   const unsigned m = __vmaxu2(__vmaxu2(__vmaxu2(E.c[0], E.c[1]), __vmaxu2(E.c[2], E.c[3])), E.c[4]);
   return (m & 0xffffu) == kFxRaw || (m >> 16) == kFxRaw;
@@ -250,26 +256,36 @@ __device__ __forceinline__ bool any_raw3(const Codes3& E) {
 
 // The same in fixed point.  Weights: one exponent per side for the values (we.x: 16 bits each) and d = we.y
 // above it for the derivatives of both; all products of component q share the scale
-// top_q = max(value code, derivative code + d).  False: some value is not finite.
+// top_q = max(value code, derivative code + d).  False: some value is not finite, or a side lies too far below
+// the scale, which covers the far node of the other side.
 __device__ __forceinline__ bool sums_fixed(int e, int E, const int* s, const Edge3Fx& fx, const int4* w5, float g1,
                                            double (*W)[5], float (*cf)[5]) {
   constexpr int L = kBits3;
-  Codes3 M = ld_codes3(fx.uc, s[0]);
+  Codes3 M = ld_codes3(fx.uc, s[1]);               // of the four nodes that both sides read
 #pragma unroll
-  for (int k = 1; k < 6; ++k) {
-    const Codes3 c = ld_codes3(fx.uc, s[k]);
-#pragma unroll
-    for (int q = 0; q < 5; ++q) M.c[q] = __vmaxu2(M.c[q], c.c[q]);
-  }
-  if (any_raw3(M)) return false;
+  for (int k = 2; k < 5; ++k) M = max_codes3(M, ld_codes3(fx.uc, s[k]));
+  const Codes3 M0 = max_codes3(M, ld_codes3(fx.uc, s[0])), M1 = max_codes3(M, ld_codes3(fx.uc, s[5]));
+  if (any_raw3(max_codes3(M0, M1))) return false;
   const int2 we = __ldg(fx.w5e + e);
-  int top[5];
+  // a component may lie one code below the scale, a momentum as far as sqrt(rho E) of its side reaches (as in 2D,
+  // edge64.cuh: FP64 sums are the more accurate ones below that)
+  int top[5], t0[5], t1[5];
   float unit[5];                                   // FP32 value of 2^-(L-1) of the scale
 #pragma unroll
   for (int q = 0; q < 5; ++q) {
-    top[q] = max((int)(M.c[q] & 0xffffu), (int)(M.c[q] >> 16) + we.y);
+    t0[q] = max((int)(M0.c[q] & 0xffffu), (int)(M0.c[q] >> 16) + we.y);
+    t1[q] = max((int)(M1.c[q] & 0xffffu), (int)(M1.c[q] >> 16) + we.y);
+    top[q] = max(t0[q], t1[q]);
     unit[q] = exp2_f32(top[q] - 1022 - (L - 1));
   }
+  const int m0 = (t0[0] + t0[4]) >> 1, m1 = (t1[0] + t1[4]) >> 1;
+  bool apart = false;
+#pragma unroll
+  for (int q = 0; q < 5; ++q) {
+    const bool mom = q >= 1 && q < 4;
+    apart |= top[q] - min(mom ? max(t0[q], m0) : t0[q], mom ? max(t1[q], m1) : t1[q]) > 1;
+  }
+  if (apart) return false;
   // a pair's limbs at its component's scale (far: some shift of the node is 32 or more)
   auto limbs = [&](int hi, int lo, int d, bool far, int& bh, int& bl) {
     if (far) fx_far(hi, lo, d);

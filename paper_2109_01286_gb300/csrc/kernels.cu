@@ -737,8 +737,10 @@ __device__ __forceinline__ void flux64(double* wl, double* wr, Prim64 pl, Prim64
     roe_flux64(wl, wr, pl, pr, nx, ny, ph.g1, ph.harten, ph.half_inv_harten, hq);
 }
 
-// LIST: edges with a 3-node (or re-decided) component are only listed, for k_edge_weno.
-template <bool LIST>
+// LIST: edges with a 3-node (or re-decided) component are only listed, for k_edge_weno.  FX: 5-node sums in
+// fixed point; edges that these do not hold (LIST: listed too) take FP64 sums.  A kernel with both kinds of sums
+// in one thread spills more: 1.5% on a step of the four-quadrant 512x512 mesh.
+template <bool LIST, bool FX>
 __device__ __forceinline__ void edge_body64(int e, int Ef, int V, const int32_t* __restrict__ sten,
                                             const double* __restrict__ nrm, const double* __restrict__ w5,
                                             const double* __restrict__ w3, const double* __restrict__ Ua,
@@ -755,7 +757,12 @@ __device__ __forceinline__ void edge_body64(int e, int Ef, int V, const int32_t*
   ld4(Ua + (size_t)s[3] * 12, wj);
   double W[2][4];
   float cf[6][4];
-  if (!fx.uf || !edge_fixed64<LIST>(e, Ef, s, fx, d2f_rn(nx), d2f_rn(ny), ph, W, cf, ws)) {
+  if (!FX || !edge_fixed64<LIST>(e, Ef, s, fx, d2f_rn(nx), d2f_rn(ny), ph, W, cf, ws)) {
+    if (LIST && FX) {             // FP64 sums with 8 lanes; every component is decided again
+      asm volatile("cp.async.wait_all;" ::: "memory");
+      fx.list[atomicAdd(fx.count, 1)] = make_int2(e, ph.force_branch == 1 ? 0 : 0xff);
+      return;
+    }
 #pragma unroll
     for (int r = 0; r < 4; ++r) W[0][r] = W[1][r] = 0.0;
     // FP32 left eigenvectors at the Roe state of the edge ends (sensor only)
@@ -822,7 +829,7 @@ __device__ __forceinline__ void edge_body(int e, int Ef, int V, const int32_t* _
                                           const EdgeFx& fx) {
   if (e >= Ef) return;
   if constexpr (std::is_same<T, double>::value) {
-    edge_body64<false>(e, Ef, V, sten, nrm, w5, w3, Ua, h, ph, err, dbg, fx);
+    edge_body64<false, false>(e, Ef, V, sten, nrm, w5, w3, Ua, h, ph, err, dbg, fx);
     return;
   }
   const T g1 = phys_g1<T>(ph);
@@ -1009,6 +1016,7 @@ __global__ void __launch_bounds__(128, 5) k_edge(int Ef, int V, const int32_t* _
 
 // FP64 edges whose two sides take the 5-node branch; the others are listed.
 // 128 registers (some spilled): 4 blocks of 128 an SM; 3 or 5 measured 4 and 2 percent slower.
+template <bool FX>
 __global__ void __launch_bounds__(kEdgeBlock, 4) k_edge64(int Ef, int V, const int32_t* __restrict__ sten,
                                                    const double* __restrict__ nrm,
                                                    const double* __restrict__ w5,
@@ -1017,30 +1025,28 @@ __global__ void __launch_bounds__(kEdgeBlock, 4) k_edge64(int Ef, int V, const i
                                                    Phys ph, unsigned* err, uint8_t* __restrict__ dbg,
                                                    EdgeFx fx) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  __shared__ int2 ws[30 * kEdgeBlock];
+  __shared__ int2 ws[FX ? 30 * kEdgeBlock : 1];
   if (e >= Ef) return;
-  if (fx.uf) stage_w5(ws + threadIdx.x, fx, Ef, e);
-  edge_body64<true>(e, Ef, V, sten, nrm, w5, w3, Ua, h, ph, err, dbg, fx, ws + threadIdx.x);
+  if (FX) stage_w5(ws + threadIdx.x, fx, Ef, e);
+  edge_body64<true, FX>(e, Ef, V, sten, nrm, w5, w3, Ua, h, ph, err, dbg, fx, ws + threadIdx.x);
 }
 
 // edge_fixed64's 5-node sum of one side's component q (the same integers, so the same bits).
 __device__ __forceinline__ bool lane_fixed64(int e, int Ef, const int* s, int side, int q, const EdgeFx& fx,
                                              double& W5) {
   constexpr int L = 29;
-  uint4 c[6], E = make_uint4(0, 0, 0, 0);
+  uint4 c[6];
 #pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    c[k] = __ldg(fx.uc + s[k]);
-    E = make_uint4(__vmaxu2(E.x, c[k].x), __vmaxu2(E.y, c[k].y), __vmaxu2(E.z, c[k].z), __vmaxu2(E.w, c[k].w));
-  }
-  const unsigned all = __vmaxu2(__vmaxu2(E.x, E.y), __vmaxu2(E.z, E.w));
-  if ((all & 0xffffu) == kFxRaw || (all >> 16) == kFxRaw) return false;
+  for (int k = 0; k < 6; ++k) c[k] = __ldg(fx.uc + s[k]);
+  const uint4 E = max_codes8(max_codes8(c[1], c[2]), max_codes8(c[3], c[4]));
+  const int2 we = __ldg(fx.w5e + e);
+  uint2 tops;
+  if (any_raw8(max_codes8(E, max_codes8(c[0], c[5]))) || !sides_in_range(E, c[0], c[5], we.y, tops)) return false;
   auto code = [&](const uint4& v, bool deriv) {
     const unsigned w = deriv ? (q & 2 ? v.w : v.z) : (q & 2 ? v.y : v.x);
     return (int)(w >> (16 * (q & 1))) & 0xffff;
   };
-  const int2 we = __ldg(fx.w5e + e);
-  const int top = max(code(E, false), code(E, true) + we.y);
+  const int top = (int)((q & 2 ? tops.y : tops.x) >> (16 * (q & 1))) & 0xffff;
   long long hh = 0, x = 0;
 #pragma unroll
   for (int j = 0; j < 5; ++j) {
@@ -2162,9 +2168,10 @@ cudaError_t launch_edge(const DevMesh& m, const Phys& ph, cudaStream_t s) {
       return cudaGetLastError();
     }
     const int nt = edge_threads(m.Ef);
-    k_edge64<<<blocks(m.Ef, nt), nt, 0, s>>>(m.Ef, m.V, m.sten, (const double*)m.nrm, (const double*)m.w5,
-                                             (const double*)m.w3, (const double*)m.Ua, (double*)m.h, ph,
-                                             m.err, m.dbg_branch, fx);
+    auto* k = fx.uf ? k_edge64<true> : k_edge64<false>;
+    k<<<blocks(m.Ef, nt), nt, 0, s>>>(m.Ef, m.V, m.sten, (const double*)m.nrm, (const double*)m.w5,
+                                      (const double*)m.w3, (const double*)m.Ua, (double*)m.h, ph, m.err,
+                                      m.dbg_branch, fx);
     // the list's length is known on the device only: enough blocks for a full GPU, or the whole mesh
     const int nb = std::min(blocks((long long)m.Ef * 8, nt), 152 * 4 * (128 / nt));
     k_edge_weno<false><<<nb, nt, 0, s>>>(m.Ef, m.V, m.sten, (const double*)m.nrm, (const double*)m.w5,
