@@ -349,13 +349,16 @@ hfd_status hfd_check_conversions(int64_t n, const double* x, float* f_int, float
  * 1024x1024 mesh (GB300): the divergence 1.66 ms against 2.23 ms for FP64 sums and 0.96 ms for
  * folded = 0.  The viscous rows stay FP64.
  * folded = 0: fixed point.  Each row's coefficients and the fluxes it reads are 57-bit integers
- * relative to their largest, multiplied and summed exactly on the integer pipe (three 32x32+64-bit
- * multiply-adds per product), so that only the factors are rounded: the sums are closer to the exact
- * ones than those of FP64 multiply-adds (rms error 0.15 to 0.35 of theirs) and do not depend on
- * the order of the entries or the lane count.  Rows that read a flux that is not finite are
- * evaluated in FP64.  Meshes with a row of more than 400 products (2 per vertex, 1 per edge) take
- * the plain FP64 form, as do meshes with 1 or 2 lanes (hfd_mesh_set_lanes) and the persistent launch: 24
- * FP64 multiply-adds per stencil vertex and 12 per stencil edge.  Drops captured graphs.
+ * relative to their row's scale, multiplied and summed on the integer pipe in two limbs each: three
+ * of the four limb products (32x32+64-bit multiply-adds) are summed exactly, and the fourth, of the two low
+ * limbs, at most 2^-57 of the scale, is left out.  Over rows of one magnitude the sums are closer to
+ * the exact ones than those of FP64 multiply-adds (rms error 0.15 to 0.35 of theirs); they do not depend
+ * on the order of the entries or the lane count, nor on the other rows of the mesh or batch.  Rows
+ * that read a flux that is not finite are evaluated in FP64.  Meshes with a coefficient that is not
+ * finite or outside 2^+-500, or with a tile of rows too large for shared memory (128 KB: a valence of several
+ * hundred), take the plain FP64 form, as do meshes with 1 or 2 lanes (hfd_mesh_set_lanes) and the
+ * persistent launch: 24 FP64 multiply-adds per stencil vertex and 12 per stencil edge.  Drops
+ * captured graphs.
  * Errors: HFD_ERR_ARG (folded not 0 or 1), HFD_ERR_UNSUPPORTED (folded = 1 on an FP32 mesh). */
 hfd_status hfd_mesh_set_fp64_div(hfd_mesh* mesh, int32_t folded);
 

@@ -110,8 +110,8 @@ hfd_status dev_alloc(hfd_mesh* m, void** dst, size_t bytes) {
 
 // The fixed-point form of an FP64 mesh's divergence (d.fx, d.div_fx): chunk pointers and tile
 // records here, the coefficients packed on the device from the uploaded rows.  Meshes whose rows
-// have no such form (a row of more than kFxRowMax28 products, coefficients outside the exponent
-// field, a tile too large for shared memory) keep the plain FP64 kernel.
+// have no such form (coefficients that are not finite or outside the exponent field, a tile too large
+// for shared memory) keep the plain FP64 kernel.
 hfd_status build_div_fx(hfd_mesh* m, const std::vector<int32_t>& vptr, const std::vector<int32_t>& vidx,
                         const std::vector<int32_t>& eptr, const std::vector<int32_t>& eidx) {
   DevMesh& d = m->dm;
@@ -122,10 +122,11 @@ hfd_status build_div_fx(hfd_mesh* m, const std::vector<int32_t>& vptr, const std
   std::vector<int32_t> cv(A + 1, 0), ce(A + 1, 0);
   for (int r = 0; r < A; ++r) {
     const int N = vptr[r + 1] - vptr[r], M = eptr[r + 1] - eptr[r];
-    if (N == 0 || M == 0 || 2 * N + M > hfd::kFxRowMax28) return HFD_OK;
-    if (2 * N + M > hfd::kFxRowMax29) f.L = 28;
-    cv[r + 1] = cv[r] + (N + C - 1) / C;
-    ce[r + 1] = ce[r] + (M + C - 1) / C;
+    if (N == 0 || M == 0) return HFD_OK;
+    const int nc = (N + C - 1) / C, mc = (M + C - 1) / C;
+    if (2 * nc + mc > hfd::kFxCarry) f.carry = true;      // products of a lane of four
+    cv[r + 1] = cv[r] + nc;
+    ce[r + 1] = ce[r] + mc;
   }
   // tiles
   f.rows = A < hfd::kFxSmallRows ? 8 : 16;

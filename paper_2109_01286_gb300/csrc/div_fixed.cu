@@ -63,6 +63,10 @@ struct FxAcc {
 #pragma unroll
     for (int i = 0; i < 12; ++i) { hh[i] = 0; x[i] = 0; }
   }
+  __device__ __forceinline__ void carry() {
+#pragma unroll
+    for (int i = 0; i < 12; ++i) x[i] = fx_carry(hh[i], x[i], kFxBits);
+  }
   // the four components of a flux vector (limbs a: components 0, 1; b: 2, 3) times the
   // coefficients (ch, cl) of row d_k
   __device__ __forceinline__ void row(int k, int4 a, int4 b, int ch, int cl) {
@@ -84,8 +88,8 @@ __device__ __forceinline__ bool shifts(uint2 E, uint2 e, int* d) {
 }
 
 // Four components' stored pairs to limbs at the row's scale.
-template <int L>
 __device__ __forceinline__ void limbs4(int4& a, int4& b, const int* d) {
+  constexpr int L = kFxBits;
   fx_limbs(a.x, a.y, d[0], L);
   fx_limbs(a.z, a.w, d[1], L);
   fx_limbs(b.x, b.y, d[2], L);
@@ -99,14 +103,14 @@ __device__ __forceinline__ void far4(int4& a, int4& b, int* d) {
 }
 
 // The vertex entries of one row (Euler fluxes with cv, or viscous fluxes with cvis): lane `lane` of
-// G takes the entries lane, lane + G, ...  id: the entries' positions in the tile's staged
+// G takes the entries first + lane, first + lane + G, ... (first: a multiple of G).  id: the entries' positions in the tile's staged
 // vertices (four planes of 16-byte pieces F01, F23, G01, G23, n pieces each; sx: code words), cc:
 // the row's coefficient chunks, E: the row's codes.
-template <int G, int L>
-__device__ __forceinline__ void vertex_entries(FxAcc& A, int entries, int lane, uint2 E, const uint16_t* id,
+template <int G>
+__device__ __forceinline__ void vertex_entries(FxAcc& A, int first, int entries, int lane, uint2 E, const uint16_t* id,
                                                const int4* cc, const int4* planes, int n, const uint2* sx) {
-  cc += 12 * (lane >> 2) + (lane & 3);
-  for (int j = lane; j < entries; j += G, cc += 3 * G) {
+  cc += 12 * (lane >> 2) + (lane & 3) + 3 * first;
+  for (int j = first + lane; j < entries; j += G, cc += 3 * G) {
     const int u = id[j];
     const int4* f = planes + u;
     int4 f0 = f[0], f1 = f[n], g0 = f[2 * n], g1 = f[3 * n];
@@ -117,43 +121,63 @@ __device__ __forceinline__ void vertex_entries(FxAcc& A, int entries, int lane, 
       far4(f0, f1, df);
       far4(g0, g1, d);
     }
-    limbs4<L>(f0, f1, d);
+    limbs4(f0, f1, d);
     A.row(0, f0, f1, k0.x, k0.y);
     A.row(1, f0, f1, k1.x, k1.y);
     A.row(2, f0, f1, k2.x, k2.y);
-    limbs4<L>(g0, g1, d);
+    limbs4(g0, g1, d);
     A.row(0, g0, g1, k0.z, k0.w);
     A.row(1, g0, g1, k1.z, k1.w);
     A.row(2, g0, g1, k2.z, k2.w);
   }
 }
 
-template <int G, int L>
-__device__ __forceinline__ void edge_entries(FxAcc& A, int entries, int lane, uint2 E, const uint16_t* id,
+template <int G>
+__device__ __forceinline__ void edge_entries(FxAcc& A, int first, int entries, int lane, uint2 E, const uint16_t* id,
                                              const unsigned char* cc, const int4* planes, int n,
                                              const uint2* sx) {
-  const unsigned char* c01 = cc + 96 * (lane >> 2) + 16 * (lane & 3);
-  const unsigned char* c2 = cc + 96 * (lane >> 2) + 64 + 8 * (lane & 3);
-  for (int j = lane; j < entries; j += G, c01 += 24 * G, c2 += 24 * G) {
+  const unsigned char* c01 = cc + 96 * (lane >> 2) + 16 * (lane & 3) + 24 * first;
+  const unsigned char* c2 = cc + 96 * (lane >> 2) + 64 + 8 * (lane & 3) + 24 * first;
+  for (int j = first + lane; j < entries; j += G, c01 += 24 * G, c2 += 24 * G) {
     const int u = id[j];
     int4 h0 = planes[u], h1 = planes[n + u];
     const int4 k01 = __ldg(reinterpret_cast<const int4*>(c01));
     const int2 k2 = __ldg(reinterpret_cast<const int2*>(c2));
     int d[4];
     if (shifts(E, sx[u], d)) far4(h0, h1, d);
-    limbs4<L>(h0, h1, d);
+    limbs4(h0, h1, d);
     A.row(0, h0, h1, k01.x, k01.y);
     A.row(1, h0, h1, k01.z, k01.w);
     A.row(2, h0, h1, k2.x, k2.y);
   }
 }
 
+// Calls f(first, end) for all entries of a row: at once, or (CARRY) in spans of at most kFxCarry products of
+// a lane, `per` an entry, after each of which the cross sums are carried over (the same sums, so the same
+// bits).  One row of more than about 150 products sends its mesh or batch to the kernel with CARRY: 160,000
+// rows and a mesh whose largest row has 282 products 400 us a residual (386 us with 28-bit limbs for every
+// row, which need no carry but hold 55-bit factors), 582 products 455 us (986 us in FP64); 372 us
+// beside rows of ordinary length.  Most of that is the shared memory of the largest tile.
+template <int G, bool CARRY, typename F>
+__device__ __forceinline__ void in_spans(FxAcc& A, int entries, int per, F f) {
+  if (!CARRY) {
+    f(0, entries);
+    return;
+  }
+  const int span = G * (kFxCarry / per);
+#pragma unroll 1
+  for (int first = 0; first < entries; first += span) {
+    f(first, min(entries, first + span));
+    A.carry();
+  }
+}
+
 // Adds the lanes' sums (exactly) and leaves each lane its share of the 12 rows (RowShare): value i
 // is (hh[i] 2^L + lo[i]) in units of the row's scale.
-template <int G, int L>
+template <int G>
 __device__ __forceinline__ void reduce_rows(FxAcc& A, unsigned* lo, int lane) {
 #pragma unroll
-  for (int i = 0; i < 12; ++i) lo[i] = fx_carry(A.hh[i], A.x[i], L);
+  for (int i = 0; i < 12; ++i) lo[i] = fx_carry(A.hh[i], A.x[i], kFxBits);
   reduce_scatter12<G>(A.hh, lane);
   reduce_scatter12<G>(lo, lane);
 }
@@ -170,11 +194,11 @@ __device__ __noinline__ double fallback_sum(const DivFx& m, int r, int k, int q,
   const unsigned* mee = reinterpret_cast<const unsigned*>(m.ee);
   auto code = [&](unsigned e) { return (int)(e >> (16 * (q & 1))) & 0xffff; };
   auto coef = [&](int hi, int lo, int ke) {
-    return scalbn((double)((long long)hi * (1ll << m.L) + lo), coef_exp(ke, k) - (2 * m.L - 1));
+    return scalbn((double)((long long)hi * (1ll << kFxBits) + lo), coef_exp(ke, k) - (2 * kFxBits - 1));
   };
   auto flux = [&](const int4* base, size_t piece, unsigned e) {
     const int4 p = base[piece + half];
-    return fx_decode(q & 1 ? make_int2(p.z, p.w) : make_int2(p.x, p.y), code(e), m.L);
+    return fx_decode(q & 1 ? make_int2(p.z, p.w) : make_int2(p.x, p.y), code(e), kFxBits);
   };
   auto vertices = [&](const int4* cv, const int4* FG, const unsigned* ex, int ke, double sign) {
     const int n0 = m.nvptr[r], N = m.nvptr[r + 1] - n0;
@@ -215,10 +239,11 @@ __device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;
 // (the ids of the vertices and edges its rows read, each once, and the entries' positions in them)
 // and its coefficients by bulk copies, contiguous in their arrays; the listed fluxes, all at once; the
 // state.  Everything else reads shared memory.
-template <int G, int L, bool VISC>
+template <int G, bool CARRY, bool VISC>
 __global__ void __launch_bounds__(128, 4) k_div_fx(DivFx m, StageArgs sa, const int32_t* __restrict__ vmem,
                                                 const unsigned long long* dtbits, double cfl,
                                                 double* dt_last, unsigned* err) {
+  constexpr int L = kFxBits;
   extern __shared__ __align__(128) unsigned char smem[];
   __shared__ __align__(8) unsigned long long bar;
   const int tid = threadIdx.x, nt = blockDim.x;
@@ -298,10 +323,14 @@ __global__ void __launch_bounds__(128, 4) k_div_fx(DivFx m, StageArgs sa, const 
   A.clear();
   if (!ok && tid == 0) atomicOr(err, ERRBIT_TIMEOUT);
   if (live && !odd && ok) {
-    edge_entries<G, L>(A, 4 * mc, lane, E, eid, m.ce + 96 * (size_t)(mb + m0), sH, ne, sxe);
-    vertex_entries<G, L>(A, 4 * nc, lane, E, vid, m.cv + 12 * (size_t)(cb + c0), sF, nv, sx);
+    in_spans<G, CARRY>(A, 4 * mc, 1, [&](int first, int end) {
+      edge_entries<G>(A, first, end, lane, E, eid, m.ce + 96 * (size_t)(mb + m0), sH, ne, sxe);
+    });
+    in_spans<G, CARRY>(A, 4 * nc, 2, [&](int first, int end) {
+      vertex_entries<G>(A, first, end, lane, E, vid, m.cv + 12 * (size_t)(cb + c0), sF, nv, sx);
+    });
   }
-  reduce_rows<G, L>(A, lo, lane);
+  reduce_rows<G>(A, lo, lane);
   // a flux is b 2^(code - 1022 - (2L - 1)) and a coefficient a 2^(e - (2L - 1)); lo counts 2^L of a b
   constexpr int unit = L - 1022 - 2 * (2 * L - 1);
 #pragma unroll
@@ -312,8 +341,10 @@ __global__ void __launch_bounds__(128, 4) k_div_fx(DivFx m, StageArgs sa, const 
   if (VISC) {
     A.clear();
     if (live && !odd && ok)
-      vertex_entries<G, L>(A, 4 * nc, lane, Ev, vid, m.cvis + 12 * (size_t)(cb + c0), sFv, nv, sxv);
-    reduce_rows<G, L>(A, lo, lane);
+      in_spans<G, CARRY>(A, 4 * nc, 2, [&](int first, int end) {
+        vertex_entries<G>(A, first, end, lane, Ev, vid, m.cvis + 12 * (size_t)(cb + c0), sFv, nv, sxv);
+      });
+    reduce_rows<G>(A, lo, lane);
 #pragma unroll
     for (int i = 0; i < RowShare<G>::kMax; ++i) {
       const int k = (base + i) >> 2, q = (base + i) & 3;
@@ -336,7 +367,8 @@ __global__ void k_pack_fx(int A, int Ef, const int32_t* __restrict__ vp, const i
                           const double* __restrict__ cv, const double* __restrict__ ce,
                           const double* __restrict__ cvis, const int32_t* __restrict__ sten,
                           const int32_t* __restrict__ cvp, const int32_t* __restrict__ cep, int4* ocv, unsigned char* oce, int4* ocvis, int2* cexp,
-                          int L, int* flag) {
+                          int* flag) {
+  constexpr int L = kFxBits;
   const int r = blockIdx.x * blockDim.x + threadIdx.x;
   if (r >= A) return;
   const int n0 = vp[r], N = vp[r + 1] - n0, m0 = ep[r], M = ep[r + 1] - m0;
@@ -347,19 +379,27 @@ __global__ void k_pack_fx(int A, int Ef, const int32_t* __restrict__ vp, const i
   bool bad = false;
   for (int k = 0; k < 3; ++k) {
     int t = -10000, tz = -10000;
+    double sum = 0.0, sumz = 0.0;
     for (int j = 0; j < N; ++j) {
       t = max(t, max(exp_above(c[(2 * k) * N + j]), exp_above(c[(2 * k + 1) * N + j])));
       if (z) tz = max(tz, max(exp_above(z[(2 * k) * N + j]), exp_above(z[(2 * k + 1) * N + j])));
       bad |= !isfinite(c[(2 * k) * N + j]) || !isfinite(c[(2 * k + 1) * N + j]);
       if (z) bad |= !isfinite(z[(2 * k) * N + j]) || !isfinite(z[(2 * k + 1) * N + j]);
+      sum += fabs(c[(2 * k) * N + j]) + fabs(c[(2 * k + 1) * N + j]);
+      if (z) sumz += fabs(z[(2 * k) * N + j]) + fabs(z[(2 * k + 1) * N + j]);
     }
     for (int j = 0; j < M; ++j) {
       t = max(t, exp_above(d[k * M + j]));
       bad |= !isfinite(d[k * M + j]);
+      sum += fabs(d[k * M + j]);
     }
     e[k] = t == -10000 ? 0 : t;
     ez[k] = tz == -10000 ? 0 : tz;
     bad |= abs(e[k]) > 500 || abs(ez[k]) > 500;
+    if (bad) break;
+    while (sum > scalbn((double)kFxCoefSum, e[k])) ++e[k];
+    while (sumz > scalbn((double)kFxCoefSum, ez[k])) ++ez[k];
+    bad |= e[k] > 500 || ez[k] > 500;
   }
   if (bad) {
     *flag = 1;
@@ -407,14 +447,14 @@ cudaError_t pack_div_fx(const DevMesh& m, int* flag, cudaStream_t s) {
   k_pack_fx<<<(m.A + 63) / 64, 64, 0, s>>>(
       m.A, m.Ef, m.vptr, m.vidx, m.eptr, m.eidx, (const double*)m.cv, (const double*)m.ce,
       m.viscous ? (const double*)m.cvis : nullptr, m.sten, f.vptr, f.eptr, f.cv, f.ce,
-      f.cvis, f.cexp, f.L, flag);
+      f.cvis, f.cexp, flag);
   return cudaGetLastError();
 }
 
 // One thread per flux edge: the 30 weights of its sides (side * 15 + node * 3 + {value, x, y}) as limbs.
 // Exponents: one per side for the values, and one offset for the derivatives of both sides.
 __global__ void k_pack_w5(int Ef, const double* __restrict__ w5, int2* w5f, int2* w5e, int* flag) {
-  constexpr int L = 29;
+  constexpr int L = kFxBits;
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= Ef) return;
   int ev[2] = {-10000, -10000}, off = -10000;
@@ -449,15 +489,15 @@ cudaError_t pack_w5_fx(const DevMesh& m, int* flag, cudaStream_t s) {
   return cudaGetLastError();
 }
 
-template <int G, int L>
+template <int G, bool CARRY>
 static const void* fx_kernel(bool visc) {
-  return visc ? (const void*)&k_div_fx<G, L, true> : (const void*)&k_div_fx<G, L, false>;
+  return visc ? (const void*)&k_div_fx<G, CARRY, true> : (const void*)&k_div_fx<G, CARRY, false>;
 }
 
 static const void* fx_kernel(const DevMesh& m, int lanes) {
   const bool visc = m.viscous != 0;
-  if (m.fx.L == 29) return lanes == 8 ? fx_kernel<8, 29>(visc) : fx_kernel<4, 29>(visc);
-  return lanes == 8 ? fx_kernel<8, 28>(visc) : fx_kernel<4, 28>(visc);
+  if (m.fx.carry) return lanes == 8 ? fx_kernel<8, true>(visc) : fx_kernel<4, true>(visc);
+  return lanes == 8 ? fx_kernel<8, false>(visc) : fx_kernel<4, false>(visc);
 }
 
 cudaError_t prepare_div_fx(const DevMesh& m) {

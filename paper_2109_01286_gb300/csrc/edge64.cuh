@@ -76,7 +76,6 @@ struct EdgeFx {
   const uint4* uc = nullptr;       // [V] 8 codes of 16 bits: w (4), w_x and w_y together (4)
   const int2* w5f = nullptr;       // [30][Ef] limb pairs, order of w5
   const int2* w5e = nullptr;       // [Ef] exponents (see pack_w5)
-  int L = 0;
   int2* list = nullptr;            // edges left to k_edge_weno: {edge, components}
   int* count = nullptr;
 };
@@ -172,7 +171,7 @@ template <bool SHARED>
 __device__ __forceinline__ bool edge_fixed64(int e, int Ef, const int* s, const EdgeFx& fx, float nx, float ny,
                                              const Phys& ph, double (*W)[4], float (*cf)[4],
                                              const int2* ws = nullptr) {
-  constexpr int L = 29;
+  constexpr int L = kFxBits;
   uint4 E = __ldg(fx.uc + s[1]);
 #pragma unroll
   for (int k = 2; k < 5; ++k) E = max_codes8(E, __ldg(fx.uc + s[k]));

@@ -4,7 +4,7 @@
 // multiply-adds at 64 (measured; FP32 at 128).  A divergence row is a sum of products with one
 // magnitude: its coefficients share a scale and so do the fluxes its stencil reads, so the sum
 // needs no floating point.  Both factors are integers of up to 2 L - 1 bits and a sign relative to
-// a power of two, split in limbs of L bits (L = 29, or 28 for rows of more than 127 products),
+// a power of two, split in limbs of L = 29 bits,
 // a = ah 2^L + al with |ah|, |al| <= 2^(L-1), b = bh 2^L + bl with |bh| <= 2^(L-1), 0 <= bl < 2^L:
 //   sum a b = 2^(2 L) sum ah bh + 2^L sum (ah bl + al bh)     (+ sum al bl, left out: below
 //                                                              2^(1-2L) of the scale per product)
@@ -14,15 +14,18 @@
 // of 2^-53 of the running sum per product in FP64: over random rows of 60 to 110 products the rms
 // error is 0.15 to 0.35 of the FP64 sum's.
 //
-// Bounds: a product of high limbs is at most 2^(2L-2), so a row of K products stays below 2^63 for
-// K <= 127 (L = 29) or 400 (L = 28); a lane's cross sum takes at most 3 2^(2L-2) per product, which
-// is below 2^63 for 42 (L = 29) or 170 products in one lane.
+// Bounds: a row's coefficients take a scale of which they add up to kFxCoefSum = 127 at most, which for rows
+// of up to 127 products is the largest one's; with |bh| <= 2^(L-1) the high products then add up to
+// 127 2^(2L-2) and K 2^(L-1) for the roundings of K coefficients, below 2^63 = 128 2^(2L-2) for K up to
+// 2^27.  A lane's cross sum takes at most 3 2^(2L-2) per product, which is below 2^63 for 42 products: a
+// lane carries it over after kFxCarry.
 #pragma once
 #include <cuda_runtime.h>
 
 namespace hfd {
 
-constexpr int kFxRowMax29 = 127, kFxRowMax28 = 400;   // products in one row by L
+constexpr int kFxBits = 29;        // L
+constexpr int kFxCoefSum = 127, kFxCarry = 40;
 constexpr int kFxRaw = 0x7ff;      // code of a group stored as raw FP64 values
 
 // A group of values with one scale has a code E: the FP64 exponent field of the largest (at least

@@ -424,13 +424,12 @@ __device__ __forceinline__ bool admissible(const T* w) {
 // ------------------------------------------------------------------ k_vertex
 // A vertex's two flux vectors: 8 values of T, or (FP64 with an array of exponent codes) the
 // fixed-point divergence's stored pairs and the vertex's exponent word.
-__device__ __forceinline__ void st_fluxes(float* FG, int v, const float* F, const float* G, uint2*,
-                                          int) {
+__device__ __forceinline__ void st_fluxes(float* FG, int v, const float* F, const float* G, uint2*) {
   st4(FG + (size_t)v * 8, F);
   st4(FG + (size_t)v * 8 + 4, G);
 }
 __device__ __forceinline__ void st_fluxes(double* FG, int v, const double* F, const double* G,
-                                          uint2* ex, int L) {
+                                          uint2* ex) {
   if (!ex) {
     st4(FG + (size_t)v * 8, F);
     st4(FG + (size_t)v * 8 + 4, G);
@@ -442,8 +441,8 @@ __device__ __forceinline__ void st_fluxes(double* FG, int v, const double* F, co
   int4* o = reinterpret_cast<int4*>(FG + (size_t)v * 8);
 #pragma unroll
   for (int i = 0; i < 2; ++i) {
-    const int2 a = fx_encode(F[2 * i], E[2 * i], L), b = fx_encode(F[2 * i + 1], E[2 * i + 1], L);
-    const int2 c = fx_encode(G[2 * i], E[2 * i], L), d = fx_encode(G[2 * i + 1], E[2 * i + 1], L);
+    const int2 a = fx_encode(F[2 * i], E[2 * i], kFxBits), b = fx_encode(F[2 * i + 1], E[2 * i + 1], kFxBits);
+    const int2 c = fx_encode(G[2 * i], E[2 * i], kFxBits), d = fx_encode(G[2 * i + 1], E[2 * i + 1], kFxBits);
     o[i] = make_int4(a.x, a.y, b.x, b.y);
     o[2 + i] = make_int4(c.x, c.y, d.x, d.y);
   }
@@ -456,13 +455,12 @@ struct VertexFx {
   uint2 *ex = nullptr, *exv = nullptr;
   int4* uf = nullptr;
   uint4* uc = nullptr;
-  int L = 0;
   int* count = nullptr;            // zeroed: the edge kernel's list starts empty
 };
 
 __device__ __forceinline__ void st_nodes(int v, const double* w, const VertexFx& fx) {
   if (!fx.uf) return;
-  constexpr int L = 29;
+  constexpr int L = kFxBits;
   int E[8];
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
@@ -526,7 +524,7 @@ __device__ __forceinline__ void vertex_body(int v, int V, const double* __restri
     T p = g1 * fma(T(-0.5), fma(q[1], u, q[2] * vv), q[3]);
     T F[4] = {q[1], q[1] * u + p, q[2] * u, (q[3] + p) * u};
     T Gf[4] = {q[2], q[1] * vv, q[2] * vv + p, (q[3] + p) * vv};
-    st_fluxes(FG, v, F, Gf, fx.ex, fx.L);
+    st_fluxes(FG, v, F, Gf, fx.ex);
     st_nodes(v, w, fx);
   }
   if (VISC) {   // viscous flux from w, w_x, w_y (Sec. 2.3; chain rule for the primitives)
@@ -552,7 +550,7 @@ __device__ __forceinline__ void vertex_body(int v, int V, const double* __restri
     };
     T Fv[4] = {T(0), to_T(txx), to_T(txy), to_T(fma(uu, txx, fma(vw, txy, qx)))};
     T Gv[4] = {T(0), to_T(txy), to_T(tyy), to_T(fma(uu, txy, fma(vw, tyy, qy)))};
-    st_fluxes(FGv, v, Fv, Gv, fx.exv, fx.L);
+    st_fluxes(FGv, v, Fv, Gv, fx.exv);
   }
 }
 
@@ -707,8 +705,8 @@ __device__ __forceinline__ void store_flux64(int e, int i, int j, const double* 
     const uint2 m = make_uint2(__vmaxu2(a.x, b.x), __vmaxu2(a.y, b.y));
     const int E[4] = {max((int)(m.x & 0xffff), fx_code(hq[0])), max((int)(m.x >> 16), fx_code(hq[1])),
                       max((int)(m.y & 0xffff), fx_code(hq[2])), max((int)(m.y >> 16), fx_code(hq[3]))};
-    const int2 p0 = fx_encode(hq[0], E[0], fx.L), p1 = fx_encode(hq[1], E[1], fx.L);
-    const int2 p2 = fx_encode(hq[2], E[2], fx.L), p3 = fx_encode(hq[3], E[3], fx.L);
+    const int2 p0 = fx_encode(hq[0], E[0], kFxBits), p1 = fx_encode(hq[1], E[1], kFxBits);
+    const int2 p2 = fx_encode(hq[2], E[2], kFxBits), p3 = fx_encode(hq[3], E[3], kFxBits);
     int4* o = reinterpret_cast<int4*>(h + (size_t)e * 4);
     o[0] = make_int4(p0.x, p0.y, p1.x, p1.y);
     o[1] = make_int4(p2.x, p2.y, p3.x, p3.y);
@@ -1034,7 +1032,7 @@ __global__ void __launch_bounds__(kEdgeBlock, 4) k_edge64(int Ef, int V, const i
 // edge_fixed64's 5-node sum of one side's component q (the same integers, so the same bits).
 __device__ __forceinline__ bool lane_fixed64(int e, int Ef, const int* s, int side, int q, const EdgeFx& fx,
                                              double& W5) {
-  constexpr int L = 29;
+  constexpr int L = kFxBits;
   uint4 c[6];
 #pragma unroll
   for (int k = 0; k < 6; ++k) c[k] = __ldg(fx.uc + s[k]);
@@ -2111,7 +2109,6 @@ cudaError_t launch_vertex(const DevMesh& m, const double* U, const Phys& ph, cud
       fx.exv = m.fx.exv;
       fx.uf = m.fx.uf;
       fx.uc = m.fx.uc;
-      fx.L = m.fx.L;
     }
     if (m.viscous)
       k_vertex<double, true><<<nb, 256, 0, s>>>(m.V, U, (double*)m.Ua, (double*)m.FG, (double*)m.FGv,
@@ -2153,7 +2150,6 @@ cudaError_t launch_edge(const DevMesh& m, const Phys& ph, cudaStream_t s) {
     } else if (m.div_fx) {
       fx.ex = m.fx.ex;
       fx.ee = m.fx.ee;
-      fx.L = m.fx.L;
       fx.uf = m.fx.uf;
       fx.uc = m.fx.uc;
       fx.w5f = m.fx.w5f;

@@ -62,7 +62,7 @@ constexpr int kStagePtrSlot = 160;     // 36 row pointers of a tile (pb .. r1, w
 // entry of its chunks, vertices first, the position in that list as 16 bits.
 struct DivFx {
   int A = 0, V = 0, Ef = 0;
-  int L = 29;                 // bits of a limb
+  bool carry = false;         // some lane takes more than kFxCarry products
   int rows = 16;              // rows per tile: 8 or 16
   int smem = 0;               // bytes of the tile that stages the most
   int32_t *vptr = nullptr, *eptr = nullptr;

@@ -6,7 +6,7 @@ namespace hfd {
 
 // A 5-vector's record in fixed point: its pairs and the codes of mass, momentum (one for the three: each row
 // reads fluxes in all directions, so every momentum sum has pressure-sized terms) and energy.
-constexpr int kBits3 = 29;
+constexpr int kBits3 = kFxBits;
 __device__ __forceinline__ void st_record3(int4* rec, size_t i, const double* f) {
   const int E0 = fx_code(f[0]), E1 = max(fx_code(f[1]), max(fx_code(f[2]), fx_code(f[3]))), E2 = fx_code(f[4]);
   const int2 p0 = fx_encode(f[0], E0, kBits3), p1 = fx_encode(f[1], E1, kBits3), p2 = fx_encode(f[2], E1, kBits3);
