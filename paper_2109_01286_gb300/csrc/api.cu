@@ -644,7 +644,7 @@ hfd_status step_impl(hfd_mesh* m, double* U, double dt, cudaStream_t s, Timer* t
       cudaEventRecord(b, s);
       tm->ev.push_back({kind, {a, b}});
       // the CFL minimum is two kernels (two-pass reduction), and so are the FP64 edges but for small meshes
-      tm->launches += kind == 4 ? 2 : kind == 2 ? hfd::edge_launches(d) : 1;
+      tm->launches += kind == 4 ? 2 : kind == 2 ? hfd::edge_launches(d, m->ph) : 1;
     }
     return e;
   };

@@ -160,16 +160,18 @@ __device__ __forceinline__ void roe_flux(const T* wl, const T* wr, T nx, T ny, T
 struct Prim64 {       // of a state w: 1/rho, sqrt(rho), velocity, pressure, E + p, enthalpy
   double ir, r, u, v, p, Ep, H;
 };
+// Products are rounded by themselves: where a kernel shuffles them to another lane the compiler cannot merge them
+// with the sums that read them, and elsewhere it must not, for the same bits.
 __device__ __forceinline__ Prim64 prim64(const double* w, double g1) {
   Prim64 q;
   const double s = rsqrt64(w[0]);
-  q.ir = s * s;
-  q.r = w[0] * s;
-  q.u = w[1] * q.ir;
-  q.v = w[2] * q.ir;
-  q.p = g1 * fma(-0.5, fma(w[1], q.u, w[2] * q.v), w[3]);
-  q.Ep = w[3] + q.p;
-  q.H = q.Ep * q.ir;
+  q.ir = __dmul_rn(s, s);
+  q.r = __dmul_rn(w[0], s);
+  q.u = __dmul_rn(w[1], q.ir);
+  q.v = __dmul_rn(w[2], q.ir);
+  q.p = __dmul_rn(g1, fma(-0.5, fma(w[1], q.u, w[2] * q.v), w[3]));
+  q.Ep = __dadd_rn(w[3], q.p);
+  q.H = __dmul_rn(q.Ep, q.ir);
   return q;
 }
 // Roe-averaged u, v, K = u^2 + v^2, H, c, 1/c of two states (the right state's weight from one
@@ -612,30 +614,54 @@ __device__ __forceinline__ void sensor64(T u0, T u1, T u2, T u3, T u4, const Phy
   S = t[0] + t[1] + t[2];
 }
 
-// Characteristic values of the conservative values a: rows q_n - c, entropy, shear, q_n + c of the
-// left eigenvectors (left_ev), with the shared parts formed once (13 FP64 instructions).
+// One component of one side: the weighted 3-node value of the side's characteristic values u (k3: its 3-node
+// weights), and whether the sensor finds them smooth.  Every rounding is written out, so that the kernels agree.
+__device__ __forceinline__ double weno64(const double* u, const double* k3, const Phys& ph, bool& smooth) {
+  double s[3];
+  auto square = [&](int i, double a, double e) {     // (eps + 13/12 a^2 + e^2/4)^2
+    const double x = __dadd_rn(ph.eps, __fma_rn(__dmul_rn(13.0 / 12.0, a), a, __dmul_rn(__dmul_rn(0.25, e), e)));
+    s[i] = __dmul_rn(x, x);
+  };
+  square(0, __dadd_rn(__fma_rn(-2.0, u[1], u[0]), u[2]), __fma_rn(3.0, u[2], __fma_rn(-4.0, u[1], u[0])));
+  square(1, __dadd_rn(__fma_rn(-2.0, u[2], u[1]), u[3]), __dadd_rn(u[1], -u[3]));
+  square(2, __dadd_rn(__fma_rn(-2.0, u[3], u[2]), u[4]), __dadd_rn(__fma_rn(3.0, u[2], __dmul_rn(-4.0, u[3])), u[4]));
+  const double t0 = __dmul_rn(__dmul_rn(1.0 / 16.0, s[1]), s[2]), t1 = __dmul_rn(__dmul_rn(10.0 / 16.0, s[0]), s[2]);
+  const double t2 = __dmul_rn(__dmul_rn(5.0 / 16.0, s[0]), s[1]), S = __dadd_rn(__dadd_rn(t0, t1), t2);
+  smooth = t0 > __dmul_rn(ph.sens_lo, S) && t0 < __dmul_rn(ph.sens_hi, S);
+  double c[3];
+#pragma unroll
+  for (int i = 0; i < 3; ++i)
+    c[i] = __fma_rn(k3[3 * i + 2], u[i + 2], __fma_rn(k3[3 * i + 1], u[i + 1], __dmul_rn(k3[3 * i], u[i])));
+  return __dmul_rn(__fma_rn(t2, c[2], __fma_rn(t1, c[1], __dmul_rn(t0, c[0]))), rcp64(S));
+}
+
+// Characteristic values of the conservative values v: rows q_n - c, entropy, shear, q_n + c of the
+// left eigenvectors (left_ev), each row's product by itself in the order in which a lane of k_edge_weno forms it, so
+// that an edge's bits do not depend on the kernel (15 FP64 instructions; 13 with the acoustic rows' shared parts).
 struct Left64 {
-  double h0, hu, hv, h3;           // halves of b2, b1 u, b1 v, b1
-  double n0, n1, n2;               // halves of q_n / c, n_x / c, n_y / c
+  double l0[3], lu[3], lv[3], h3;  // rows q_n - c, entropy, q_n + c; the energy's column is h3 (1, -2, 1)
   double qt, nx, ny;
   __device__ __forceinline__ Left64(const Roe64& a, double nx_, double ny_, double g1) : nx(nx_), ny(ny_) {
     h3 = 0.5 * g1 * (a.ic * a.ic);
-    hu = h3 * a.u;
-    hv = h3 * a.v;
-    h0 = 0.5 * h3 * a.K;
-    const double hic = 0.5 * a.ic;
-    n1 = nx * hic;
-    n2 = ny * hic;
-    n0 = fma(a.u, n1, a.v * n2);
+    const double hic = 0.5 * a.ic, n1 = nx * hic, n2 = ny * hic, n0 = fma(a.u, n1, a.v * n2);
+    const double hK = __dmul_rn(h3, 0.5 * a.K), hu = __dmul_rn(h3, a.u), hv = __dmul_rn(h3, a.v);
+    l0[0] = __dadd_rn(n0, hK);
+    l0[1] = fma(-2.0 * h3, 0.5 * a.K, 1.0);
+    l0[2] = __dadd_rn(-n0, hK);
+    lu[0] = -__dadd_rn(n1, hu);
+    lu[1] = 2.0 * hu;
+    lu[2] = __dadd_rn(n1, -hu);
+    lv[0] = -__dadd_rn(n2, hv);
+    lv[1] = 2.0 * hv;
+    lv[2] = __dadd_rn(n2, -hv);
     qt = fma(a.v, nx, -a.u * ny);
   }
-  __device__ __forceinline__ void apply(const double* a, double* C) const {
-    const double A = fma(h0, a[0], fma(-hu, a[1], fma(-hv, a[2], h3 * a[3])));
-    const double N = fma(n0, a[0], fma(-n1, a[1], -n2 * a[2]));
-    C[0] = A + N;
-    C[1] = fma(-2.0, A, a[0]);
-    C[2] = fma(nx, a[2], fma(-ny, a[1], -qt * a[0]));
-    C[3] = A - N;
+  __device__ __forceinline__ void apply(const double* v, double* C) const {
+    const double e = __dmul_rn(h3, v[3]);
+    C[0] = fma(l0[0], v[0], fma(lu[0], v[1], fma(lv[0], v[2], e)));
+    C[1] = fma(l0[1], v[0], fma(lu[1], v[1], fma(lv[1], v[2], -2.0 * e)));
+    C[2] = fma(-qt, v[0], fma(-ny, v[1], __dmul_rn(nx, v[2])));
+    C[3] = fma(l0[2], v[0], fma(lu[2], v[1], fma(lv[2], v[2], e)));
   }
 };
 
@@ -661,13 +687,9 @@ __device__ __forceinline__ unsigned weno_side64(const Left64& L, const Roe64& a,
   unsigned taken = 0;
 #pragma unroll
   for (int q = 0; q < 4; ++q) {
-    double t[3], S;
-    sensor64(c[0][q], c[1][q], c[2][q], c[3][q], c[4][q], ph, t, S);
-    const bool smooth = (t[0] > ph.sens_lo * S) && (t[0] < ph.sens_hi * S);
-    const double c1 = k3[0] * c[0][q] + k3[1] * c[1][q] + k3[2] * c[2][q];
-    const double c2 = k3[3] * c[1][q] + k3[4] * c[2][q] + k3[5] * c[3][q];
-    const double c3 = k3[6] * c[2][q] + k3[7] * c[3][q] + k3[8] * c[4][q];
-    const double weighted = (t[0] * c1 + t[1] * c2 + t[2] * c3) * rcp64(S);
+    const double u[5] = {c[0][q], c[1][q], c[2][q], c[3][q], c[4][q]};
+    bool smooth;
+    const double weighted = weno64(u, k3, ph, smooth);
     if (((mine >> q) & 1u) && !(smooth && ph.force_branch != 2)) {
       C[q] = weighted;
       taken |= 1u << q;
@@ -1029,6 +1051,19 @@ __global__ void __launch_bounds__(kEdgeBlock, 4) k_edge64(int Ef, int V, const i
   edge_body64<true, FX>(e, Ef, V, sten, nrm, w5, w3, Ua, h, ph, err, dbg, fx, ws + threadIdx.x);
 }
 
+// One thread an edge for all branches (force_branch = "weno": there is no smooth edge to save the list for).
+template <bool FX>
+__global__ void __launch_bounds__(128, 3) k_edge64_weno(int Ef, int V, const int32_t* __restrict__ sten,
+                                                        const double* __restrict__ nrm,
+                                                        const double* __restrict__ w5,
+                                                        const double* __restrict__ w3,
+                                                        const double* __restrict__ Ua, double* __restrict__ h,
+                                                        Phys ph, unsigned* err, uint8_t* __restrict__ dbg,
+                                                        EdgeFx fx) {
+  const int e = blockIdx.x * blockDim.x + threadIdx.x;
+  if (e < Ef) edge_body64<false, FX>(e, Ef, V, sten, nrm, w5, w3, Ua, h, ph, err, dbg, fx);
+}
+
 // edge_fixed64's 5-node sum of one side's component q (the same integers, so the same bits).
 __device__ __forceinline__ bool lane_fixed64(int e, int Ef, const int* s, int side, int q, const EdgeFx& fx,
                                              double& W5) {
@@ -1168,17 +1203,12 @@ __global__ void __launch_bounds__(128) k_edge_weno(int Ef, int V, const int32_t*
       double u[5];
 #pragma unroll
       for (int j = 0; j < 5; ++j) u[j] = charac(c[j]);
-      double C = charac(w), t[3], S;
-      sensor64(u[0], u[1], u[2], u[3], u[4], ph, t, S);
-      const bool smooth = (t[0] > ph.sens_lo * S) && (t[0] < ph.sens_hi * S);
-      const bool three = mine && !(smooth && ph.force_branch != 2);
-      double k3[9];
+      double C = charac(w), k3[9];
 #pragma unroll
       for (int k = 0; k < 9; ++k) k3[k] = ld_stream(w3 + (size_t)(9 * side + k) * Ef + e);
-      const double c1 = k3[0] * u[0] + k3[1] * u[1] + k3[2] * u[2];
-      const double c2 = k3[3] * u[1] + k3[4] * u[2] + k3[5] * u[3];
-      const double c3 = k3[6] * u[2] + k3[7] * u[3] + k3[8] * u[4];
-      const double weighted = (t[0] * c1 + t[1] * c2 + t[2] * c3) * rcp64(S);
+      bool smooth;
+      const double weighted = weno64(u, k3, ph, smooth);
+      const bool three = mine && !(smooth && ph.force_branch != 2);
       if (three) C = weighted;
       taken = (__ballot_sync(0xffffffffu, three) >> (threadIdx.x & 24)) & 0xffu;
       double Cs[4];
@@ -2133,12 +2163,16 @@ cudaError_t launch_vertex(const DevMesh& m, const double* U, const Phys& ph, cud
 // edges 36 and 30 us.  Before (one kernel, sums in FP64, 341 FP64 instructions a smooth edge): 45 us for
 // 1728 edges, 125 us for 196,600 (now 87 us, 128 FP64 instructions), 330 us for 512,000 (237 us, its listed edges included; 248 us
 // with the weights loaded where they are used instead of copied to shared memory at the start).
+// Where every edge takes 3-node values (force_branch), the front of k_edge64 and 60 FP64 instructions an edge in
+// 8 lanes cost more than 32 in one thread: k_edge64_weno, a residual with 60 us for 7500 edges (8 lanes 68; 4800
+// edges 60 and 45), 64 for 15,552 (102), 267 for 109,443 (520 in 8 lanes, 596 listed) and 981 for
+// 480,000 (2132, listed 2741).
 // Threads per block: an SM partition has its own FP64 unit, so blocks of 32 spread a small mesh best.
-constexpr int kEdge8Max = 8000;
+constexpr int kEdge8Max = 8000, kEdge8MaxWeno = 6500;
 static int edge_threads(int Ef) { return Ef <= 152 * 64 ? 32 : Ef <= 152 * 128 ? 64 : 128; }
 
-int edge_launches(const DevMesh& m) {
-  return m.Ef == 0 ? 0 : m.precision == 0 && m.Ef > kEdge8Max ? 2 : 1;
+int edge_launches(const DevMesh& m, const Phys& ph) {
+  return m.Ef == 0 ? 0 : m.precision == 0 && ph.force_branch != 2 && m.Ef > kEdge8Max ? 2 : 1;
 }
 
 cudaError_t launch_edge(const DevMesh& m, const Phys& ph, cudaStream_t s) {
@@ -2157,13 +2191,20 @@ cudaError_t launch_edge(const DevMesh& m, const Phys& ph, cudaStream_t s) {
     }
     fx.list = m.weno_list;
     fx.count = m.weno_count;
-    if (m.Ef <= kEdge8Max) {
+    if (m.Ef <= (ph.force_branch == 2 ? kEdge8MaxWeno : kEdge8Max)) {
       k_edge_weno<true><<<blocks((long long)m.Ef * 8, 32), 32, 0, s>>>(
           m.Ef, m.V, m.sten, (const double*)m.nrm, (const double*)m.w5, (const double*)m.w3,
           (const double*)m.Ua, (double*)m.h, ph, m.err, m.dbg_branch, fx);
       return cudaGetLastError();
     }
     const int nt = edge_threads(m.Ef);
+    if (ph.force_branch == 2) {
+      auto* k = fx.uf ? k_edge64_weno<true> : k_edge64_weno<false>;
+      k<<<blocks(m.Ef, nt), nt, 0, s>>>(m.Ef, m.V, m.sten, (const double*)m.nrm, (const double*)m.w5,
+                                        (const double*)m.w3, (const double*)m.Ua, (double*)m.h, ph, m.err,
+                                        m.dbg_branch, fx);
+      return cudaGetLastError();
+    }
     auto* k = fx.uf ? k_edge64<true> : k_edge64<false>;
     k<<<blocks(m.Ef, nt), nt, 0, s>>>(m.Ef, m.V, m.sten, (const double*)m.nrm, (const double*)m.w5,
                                       (const double*)m.w3, (const double*)m.Ua, (double*)m.h, ph, m.err,

@@ -201,7 +201,7 @@ cudaError_t launch_conversions(int64_t n, const double* x, float* f_int, float* 
                                double* d_int, double* d_hw, cudaStream_t s);
 cudaError_t launch_vertex(const DevMesh& m, const double* U, const Phys& ph, cudaStream_t s);
 cudaError_t launch_edge(const DevMesh& m, const Phys& ph, cudaStream_t s);
-int edge_launches(const DevMesh& m);      // kernels that launch_edge launches
+int edge_launches(const DevMesh& m, const Phys& ph);      // kernels that launch_edge launches
 // out = R (residual mode) or out = a*Un + b*(Us + dt*R) (stage mode); dt_fixed <= 0 selects
 // dt_member[mesh] when dt_member is given (device array, one step per batch member), else
 // dt = cfl * (device minimum of the vertex's mesh).
