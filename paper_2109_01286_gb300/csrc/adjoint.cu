@@ -101,8 +101,10 @@ __device__ __forceinline__ void adj_edge_w5(int e, int Ef, const int* s, const d
 
 // Shared front of the edge reverse pass: hbar at the edge (k_adj_hbar), the stencil, the end
 // states and the FP32 sensor decisions exactly as k_edge takes them (bit side*4+q of `rough`:
-// 3-node branch; of `amb`: inside the guard band, re-decided in FP64).
-__device__ __forceinline__ void adj_edge_front(
+// 3-node branch; of `amb`: inside the guard band, re-decided in FP64).  FX: 5-node sums in fixed point only,
+// false where these do not hold the edge (nothing is decided then); else FP64 sums.
+template <bool FX>
+__device__ __forceinline__ bool adj_edge_front(
     int e, int Ef, const int32_t* __restrict__ sten, const double* __restrict__ nrm,
     const double* __restrict__ w5, const double* __restrict__ Ua, const double* __restrict__ hbar,
     const Phys& ph, const EdgeFx& fx, double* hb, int* s, double& nx, double& ny, double* wi, double* wj,
@@ -115,9 +117,10 @@ __device__ __forceinline__ void adj_edge_front(
   for (int r = 0; r < 4; ++r) { wi[r] = Ua[(size_t)s[2] * 12 + r]; wj[r] = Ua[(size_t)s[3] * 12 + r]; }
   // ---- forward: the 5-node sums and the FP32 sensor exactly as the edge kernel takes them
   float cf6[6][4];
-  if (fx.uf && edge_fixed64<false>(e, Ef, s, fx, (float)nx, (float)ny, ph, W5, cf6)) {
+  if (FX) {
+    if (!edge_fixed64<false>(e, Ef, s, fx, (float)nx, (float)ny, ph, W5, cf6)) return false;
     sensor32(cf6, ph, rough, amb);
-    return;
+    return true;
   }
   adj_edge_w5(e, Ef, s, w5, Ua, W5);
   rough = 0;
@@ -165,13 +168,16 @@ __device__ __forceinline__ void adj_edge_front(
         if (!(fabsf(mlo) > 1e-3f * S && fabsf(mhi) > 1e-3f * S)) amb |= bit;
       }
   }
+  return true;
 }
 
 // One thread per flux edge, edges whose sides both took the 5-node branch: the reverse of the
 // Roe flux and of the 5-node sums; each node's 12 sensitivities are formed in registers and
 // stored once to Ge[e][72].  Edges with a 3-node or re-decided component are appended to
 // `list` for k_adj_edge_full (the order of the list does not matter: each edge writes only
-// its own Ge row).
+// its own Ge row), with those that fixed point does not hold (FX; without FP64 sums in this kernel 0.6% less a
+// rollout step at 160x160).
+template <bool FX>
 __global__ void __launch_bounds__(128, 3) k_adj_edge(
     int Ef, const int32_t* __restrict__ sten, const double* __restrict__ nrm,
     const double* __restrict__ w5, const double* __restrict__ w3, const double* __restrict__ Ua,
@@ -182,8 +188,8 @@ __global__ void __launch_bounds__(128, 3) k_adj_edge(
   int s[6];
   unsigned rough, amb;
   double W5[2][4];
-  adj_edge_front(e, Ef, sten, nrm, w5, Ua, hbar, ph, fx, hb, s, nx, ny, wi, wj, W5, rough, amb);
-  if (rough | amb) {
+  if (!adj_edge_front<FX>(e, Ef, sten, nrm, w5, Ua, hbar, ph, fx, hb, s, nx, ny, wi, wj, W5, rough, amb) ||
+      (rough | amb)) {
     list[atomicAdd(count, 1)] = e;
     return;
   }
@@ -256,7 +262,8 @@ __global__ void __launch_bounds__(128) k_adj_edge_full(
   int s[6];
   unsigned rough, amb;
   double W5[2][4];
-  adj_edge_front(e, Ef, sten, nrm, w5, Ua, hbar, ph, fx, hb, s, nx, ny, wi, wj, W5, rough, amb);
+  if (!fx.uf || !adj_edge_front<true>(e, Ef, sten, nrm, w5, Ua, hbar, ph, fx, hb, s, nx, ny, wi, wj, W5, rough, amb))
+    adj_edge_front<false>(e, Ef, sten, nrm, w5, Ua, hbar, ph, fx, hb, s, nx, ny, wi, wj, W5, rough, amb);
   double* ge = Ge + (size_t)e * 72;
   const double g1 = ph.g1;
   for (int i = 0; i < 72; ++i) ge[i] = 0.0;
@@ -737,7 +744,8 @@ hfd_status residual_vjp(hfd_mesh* m, const double* Us, const double* mu, double*
   }
   // edges with both sides on the 5-node branch, then the listed remainder
   ACK(cudaMemsetAsync(m->adj_count, 0, sizeof(int32_t), s));
-  hfd::k_adj_edge<<<(d.Ef + 127) / 128, 128, 0, s>>>(
+  auto* adj_edge = fx.uf ? hfd::k_adj_edge<true> : hfd::k_adj_edge<false>;
+  adj_edge<<<(d.Ef + 127) / 128, 128, 0, s>>>(
       d.Ef, d.sten, (const double*)d.nrm, (const double*)d.w5, (const double*)d.w3,
       (const double*)d.Ua, m->adj_hbar, m->adj_Ge, m->ph, fx, m->adj_list, m->adj_count);
   ACK(cudaGetLastError());
