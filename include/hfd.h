@@ -355,8 +355,9 @@ hfd_status hfd_check_conversions(int64_t n, const double* x, float* f_int, float
  * the exact ones than those of FP64 multiply-adds (rms error 0.15 to 0.35 of theirs); they do not depend
  * on the order of the entries or the lane count, nor on the other rows of the mesh or batch.  Rows
  * that read a flux that is not finite are evaluated in FP64.  Meshes with a coefficient that is not
- * finite or outside 2^+-500, or with a tile of rows too large for shared memory (128 KB: a valence of several
- * hundred), take the plain FP64 form, as do meshes with 1 or 2 lanes (hfd_mesh_set_lanes) and the
+ * finite or outside 2^+-500, with a tile of rows too large for shared memory (128 KB: a valence of several
+ * hundred), or for whose second form (rows and edge weights are then held in both, 1.5 times the bytes)
+ * more than half of the memory left would be needed, take the plain FP64 form, as do meshes with 1 or 2 lanes (hfd_mesh_set_lanes) and the
  * persistent launch: 24 FP64 multiply-adds per stencil vertex and 12 per stencil edge.  Drops
  * captured graphs.
  * Errors: HFD_ERR_ARG (folded not 0 or 1), HFD_ERR_UNSUPPORTED (folded = 1 on an FP32 mesh). */

@@ -116,7 +116,8 @@ hfd_status hfd3_steps_profiled(hfd3_mesh* mesh, double* U, double dt, int32_t ns
 /* Lanes (consecutive threads) per vertex in the divergence gather: 1, 2 or 4 (default 4).  1 and 2 run the
  * FP64 gather; 4 runs the fixed-point one (8 threads share a row, exact sums of rounded products; a
  * 24^3 box's stage 102 us against 294 us with FP64 sums), or the FP64 gather with 4 lanes where the rows do
- * not fit fixed point (coefficients that are not finite).  FP64 lanes take the vertex's entries in turn
+ * not fit fixed point (coefficients that are not finite, or more than half of the memory left needed to hold rows
+ * and weights in both forms, 1.9 times the bytes).  FP64 lanes take the vertex's entries in turn
  * and their sums are combined by a fixed butterfly, so every count gives deterministic results that agree
  * with the others to rounding.  Errors: HFD_ERR_ARG (another count or a null mesh). */
 hfd_status hfd3_mesh_set_lanes(hfd3_mesh* mesh, int32_t lanes);

@@ -111,7 +111,9 @@ hfd_status dev_alloc(hfd_mesh* m, void** dst, size_t bytes) {
 // The fixed-point form of an FP64 mesh's divergence (d.fx, d.div_fx): chunk pointers and tile
 // records here, the coefficients packed on the device from the uploaded rows.  Meshes whose rows
 // have no such form (coefficients that are not finite or outside the exponent field, a tile too large
-// for shared memory) keep the plain FP64 kernel.
+// for shared memory) keep the plain FP64 kernel, and so do meshes whose second form would take more than
+// half of the memory that is left: rows and weights are then held twice, 1.5 times the bytes a vertex, and what
+// fitted with one form has to fit.
 hfd_status build_div_fx(hfd_mesh* m, const std::vector<int32_t>& vptr, const std::vector<int32_t>& vidx,
                         const std::vector<int32_t>& eptr, const std::vector<int32_t>& eidx) {
   DevMesh& d = m->dm;
@@ -174,6 +176,16 @@ hfd_status build_div_fx(hfd_mesh* m, const std::vector<int32_t>& vptr, const std
   if (most > hfd::kFxSmemMax) return HFD_OK;
   f.smem = (int)((most + 15) & ~(int64_t)15);
   const size_t nv = (size_t)cv[A], ne = (size_t)ce[A];
+  if (!m->want_fixed) return HFD_OK;
+  if (!m->opts.dev_alloc) {
+    const size_t V = d.V, Ef = d.Ef, both = d.viscous ? 2 : 1;
+    const size_t need = 4 * rec.size() + 192 * both * nv + 96 * ne + 16 * (size_t)A + 8 * (both + 14) * V + 256 * Ef;
+    const size_t rest = (12 * 8 * 3 + 8 * 8 * both) * V + 4 * 8 * Ef;      // fluxes and states, still to come
+    size_t left = 0, all = 0;
+    CK(cudaMemGetInfo(&left, &all));
+    if (left < rest || need > (left - rest) / 2) return HFD_OK;
+  }
+  m->began_fixed = true;
   int32_t* flag = nullptr;
   TRY(dev_upload(m, (void**)&f.head, head));
   TRY(dev_upload(m, (void**)&f.rec, rec));
@@ -698,18 +710,27 @@ hfd_status hfd_mesh_upload(const hfd_prep* prep, int32_t precision, hfd_mesh** o
   }
   *out = nullptr;
   hfd::NvtxRange range("hfd_mesh_upload");
-  hfd_mesh* m = new (std::nothrow) hfd_mesh();
-  if (!m) { set_error("hfd_mesh_upload: out of host memory"); return HFD_ERR_ARG; }
-  hfd_status st;
-  try {
-    st = upload(*prep, precision, m);
-  } catch (const std::exception& e) {
-    set_error("hfd_mesh_upload: %s", e.what());
-    st = HFD_ERR_ARG;
+  for (bool fixed : {true, false}) {
+    hfd_mesh* m = new (std::nothrow) hfd_mesh();
+    if (!m) { set_error("hfd_mesh_upload: out of host memory"); return HFD_ERR_ARG; }
+    m->want_fixed = fixed;
+    hfd_status st;
+    try {
+      st = upload(*prep, precision, m);
+    } catch (const std::exception& e) {
+      set_error("hfd_mesh_upload: %s", e.what());
+      st = HFD_ERR_ARG;
+    }
+    if (st == HFD_OK) {
+      *out = m;
+      return HFD_OK;
+    }
+    const bool again = m->began_fixed && m->out_of_memory;    // without the second form it may fit
+    hfd_mesh_destroy(m);
+    if (!again) return st;
+    cudaGetLastError();
   }
-  if (st != HFD_OK) { hfd_mesh_destroy(m); return st; }
-  *out = m;
-  return HFD_OK;
+  return HFD_ERR_CUDA;                // not reached: the second pass does not begin the form
 }
 
 hfd_status hfd_mesh_create(const hfd_mesh_desc* desc, const hfd_options* opts, hfd_mesh** out) {

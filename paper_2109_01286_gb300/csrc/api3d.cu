@@ -70,6 +70,48 @@ hfd_status put(const std::vector<T>& h, T* dptr) {
     if (s_ != HFD_OK) return s_;         \
   } while (0)
 
+// The blocks of the fixed-point forms, rows and weights a second time (1.9 times the bytes a vertex): left off,
+// and FP64 sums run, where they would take more than half of the memory that is left, or cannot be had.
+hfd_status alloc_fixed(hfd3_mesh* m) {
+  hfd::DevMesh3& d = m->d;
+  const hfd::Prep3& P = m->P;
+  const size_t V = P.V, E = P.E, held = m->allocs.size();
+  if (d.V == 0) return HFD_OK;
+  std::vector<int32_t> ptr(V + 1, 0);
+  for (size_t v = 0; v < V; ++v)
+    ptr[v + 1] = ptr[v] + (3 * (P.vptr[v + 1] - P.vptr[v]) + P.eptr[v + 1] - P.eptr[v] + 15) / 16;
+  const size_t n = (size_t)ptr[V];
+  const size_t need = 576 * n + 48 * (3 * V + E) + 12 * V + 192 * V + 328 * E;
+  size_t left = 0, all = 0;
+  CK3(cudaMemGetInfo(&left, &all));
+  if (need > left / 2) return HFD_OK;
+  auto blocks = [&]() {
+    TRY3(dalloc(m, (void**)&d.ex.uf, 10 * V * sizeof(int4)));
+    TRY3(dalloc(m, (void**)&d.ex.uc, 2 * V * sizeof(uint4)));
+    TRY3(dalloc(m, (void**)&d.ex.w5f, 40 * E * sizeof(int2)));
+    TRY3(dalloc(m, (void**)&d.ex.w5e, E * sizeof(int2)));
+    if (3 * (int64_t)V + (int64_t)E > INT32_MAX) return HFD_OK;
+    TRY3(dalloc(m, (void**)&d.fx.id, 4 * n * sizeof(int4)));
+    TRY3(dalloc(m, (void**)&d.fx.c, 32 * n * sizeof(int4)));
+    TRY3(dalloc(m, (void**)&d.fx.cexp, V * sizeof(int2)));
+    TRY3(dalloc(m, (void**)&d.fx.rec, 3 * (3 * V + E) * sizeof(int4)));
+    TRY3(dalloc(m, (void**)&d.fx.ptr, ptr.size() * sizeof(int32_t)));
+    return put(ptr, d.fx.ptr);
+  };
+  if (blocks() == HFD_OK) return HFD_OK;
+  cudaGetLastError();
+  while (m->allocs.size() > held) {
+    cudaFree(m->allocs.back());
+    m->allocs.pop_back();
+  }
+  d.fx = hfd::Div3Fx();
+  d.ex.uf = nullptr;
+  d.ex.uc = nullptr;
+  d.ex.w5f = nullptr;
+  d.ex.w5e = nullptr;
+  return HFD_OK;
+}
+
 // The edges' weights in fixed point; left off (the sums run in FP64) where a weight does not fit.
 hfd_status pack_edges(hfd3_mesh* m) {
   hfd::DevMesh3& d = m->d;
@@ -78,7 +120,7 @@ hfd_status pack_edges(hfd3_mesh* m) {
   CK3(cudaMemset(m->fx_flag, 0, sizeof(int)));
   CK3(hfd::launch3_pack_w5(d, m->fx_flag, nullptr));
   CK3(cudaMemcpy(&flag, m->fx_flag, sizeof flag, cudaMemcpyDeviceToHost));
-  d.ex_ok = flag == 0;
+  d.ex_ok = flag == 0 && d.ex.w5f;
   return HFD_OK;
 }
 
@@ -91,29 +133,17 @@ hfd_status upload_edges(hfd3_mesh* m) {
   return pack_edges(m);
 }
 
-// The fixed-point divergence: allocates m->d.fx on the first call and packs the coefficients.  Left off
-// (the FP64 gather runs) if an index is out of range or a coefficient does not fit.
+// Packs the coefficients of the fixed-point divergence.  Left off (the FP64 gather runs) if an index is out of
+// range or a coefficient does not fit.
 hfd_status pack_fx(hfd3_mesh* m) {
   hfd::DevMesh3& d = m->d;
   const hfd::Prep3& P = m->P;
   d.fx_ok = false;
-  if (d.V == 0 || 3 * (int64_t)d.V + d.E > INT32_MAX) return HFD_OK;
-  if (!d.fx.ptr) {
-    std::vector<int32_t> ptr(d.V + 1, 0);
-    for (int v = 0; v < d.V; ++v)
-      ptr[v + 1] = ptr[v] + (3 * (P.vptr[v + 1] - P.vptr[v]) + P.eptr[v + 1] - P.eptr[v] + 15) / 16;
-    for (int32_t u : P.vidx)
-      if (u < 0 || u >= d.V) return HFD_OK;
-    for (int32_t e : P.eidx)
-      if (e < 0 || e >= d.E) return HFD_OK;
-    const size_t n = (size_t)ptr[d.V];
-    TRY3(dalloc(m, (void**)&d.fx.id, 4 * n * sizeof(int4)));
-    TRY3(dalloc(m, (void**)&d.fx.c, 32 * n * sizeof(int4)));
-    TRY3(dalloc(m, (void**)&d.fx.cexp, (size_t)d.V * sizeof(int2)));
-    TRY3(dalloc(m, (void**)&d.fx.rec, 3 * (3 * (size_t)d.V + d.E) * sizeof(int4)));
-    TRY3(dalloc(m, (void**)&d.fx.ptr, ptr.size() * sizeof(int32_t)));
-    TRY3(put(ptr, d.fx.ptr));
-  }
+  if (!d.fx.ptr) return HFD_OK;
+  for (int32_t u : P.vidx)
+    if (u < 0 || u >= d.V) return HFD_OK;
+  for (int32_t e : P.eidx)
+    if (e < 0 || e >= d.E) return HFD_OK;
   int flag = 0;
   CK3(cudaMemset(m->fx_flag, 0, sizeof(int)));
   CK3(hfd::launch3_pack(d, m->fx_flag, nullptr));
@@ -148,15 +178,12 @@ hfd_status create(const hfd3_mesh_desc* desc, const hfd3_options* o, hfd3_mesh* 
   TRY3(dalloc(m, (void**)&d.err, sizeof(unsigned)));
   CK3(cudaMemset(d.err, 0, sizeof(unsigned)));
   TRY3(dalloc(m, (void**)&m->fx_flag, sizeof(int)));
-  TRY3(dalloc(m, (void**)&d.ex.uf, 10 * V * sizeof(int4)));
-  TRY3(dalloc(m, (void**)&d.ex.uc, 2 * V * sizeof(uint4)));
-  TRY3(dalloc(m, (void**)&d.ex.w5f, 40 * E * sizeof(int2)));
-  TRY3(dalloc(m, (void**)&d.ex.w5e, E * sizeof(int2)));
   TRY3(dalloc(m, (void**)&d.ex.framef, 9 * E * sizeof(float)));
   TRY3(dalloc(m, (void**)&d.ex.list, E * sizeof(int2)));
   TRY3(dalloc(m, (void**)&d.ex.listw, 12 * E * sizeof(double)));
   TRY3(dalloc(m, (void**)&d.ex.count, sizeof(int)));
   CK3(cudaMemset(d.ex.count, 0, sizeof(int)));
+  TRY3(alloc_fixed(m));
   TRY3(upload_edges(m));
   TRY3(put(P.vptr, d.vptr));
   TRY3(put(P.eptr, d.eptr));

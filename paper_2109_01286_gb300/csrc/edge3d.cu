@@ -582,6 +582,7 @@ __global__ void k3_pack_w5(int E, const double* __restrict__ w5, const double* _
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
   if (e >= E) return;
   for (int k = 0; k < 9; ++k) fx.framef[(size_t)k * E + e] = d2f_rn(frame[(size_t)k * E + e]);
+  if (!fx.w5f) return;
   int ev[2] = {-10000, -10000}, off = -10000;
   bool bad = false;
   for (int s = 0; s < 2; ++s) {

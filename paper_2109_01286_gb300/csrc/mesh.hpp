@@ -33,6 +33,8 @@ struct hfd_mesh {
   hfd::Phys ph{};
   int lanes = 4;                        // lanes per vertex in the divergence kernel (1, 2, 4, 8)
   bool fixed_point = false;             // FP64: the divergence has a fixed-point form (4 and 8 lanes)
+  // creating the mesh: the fixed-point form is wanted, was begun, and some block could not be had
+  bool want_fixed = true, began_fixed = false, out_of_memory = false;
   int persistent = 0;                   // 1: one cooperative launch per RK stage
   int grid = 0;                         // blocks of the persistent launch (0: all resident)
   std::vector<int32_t> perm;            // internal -> input
@@ -75,6 +77,7 @@ struct hfd_mesh {
 // one, else cudaMalloc; recorded for hfd_mesh_destroy.  Blocks must be 256-byte aligned.
 inline cudaError_t mesh_malloc(hfd_mesh* m, void** p, size_t bytes) {
   *p = nullptr;
+  m->out_of_memory = true;
   if (m->opts.dev_alloc) {
     void* q = m->opts.dev_alloc(bytes, m->opts.alloc_ctx);
     if (!q) return cudaErrorMemoryAllocation;
@@ -87,6 +90,7 @@ inline cudaError_t mesh_malloc(hfd_mesh* m, void** p, size_t bytes) {
     cudaError_t e = cudaMalloc(p, bytes);
     if (e != cudaSuccess) return e;
   }
+  m->out_of_memory = false;
   m->allocs.push_back(*p);
   m->stats.device_bytes += (int64_t)bytes;
   return cudaSuccess;
