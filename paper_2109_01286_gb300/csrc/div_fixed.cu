@@ -186,7 +186,7 @@ __device__ __forceinline__ void reduce_rows(FxAcc& A, unsigned* lo, int lane) {
 __device__ __forceinline__ int coef_exp(int packed, int k) { return (packed << (22 - 10 * k)) >> 22; }
 
 // One sum (row d_k, component q) of a row some of whose fluxes are not finite, in FP64 as the plain
-// kernel evaluates it: -div f + div f_vis.
+// kernel evaluates it: -div f + div f_vis.  NaN stays NaN, so the first one ends the sum.
 __device__ __noinline__ double fallback_sum(const DivFx& m, int r, int k, int q, bool visc) {
   const int half = q >> 1;
   double R = 0.0;
@@ -208,10 +208,12 @@ __device__ __noinline__ double fallback_sum(const DivFx& m, int r, int k, int q,
       const unsigned e = ex[2 * u + half];
       R = fma(sign * coef(c.x, c.y, ke), flux(FG, 4 * u, e), R);
       R = fma(sign * coef(c.z, c.w, ke), flux(FG, 4 * u + 2, e), R);
+      if (isnan(R)) return;
     }
   };
   const int2 ke = m.cexp[r];
   vertices(m.cv, m.FG, mex, ke.x, -1.0);
+  if (isnan(R)) return R;
   const int m0 = m.neptr[r], M = m.neptr[r + 1] - m0;
   for (int j = 0; j < M; ++j) {
     const size_t s = m.neidx[m0 + j];
@@ -221,6 +223,7 @@ __device__ __noinline__ double fallback_sum(const DivFx& m, int r, int k, int q,
     const double c = k == 0 ? coef(k01.x, k01.y, ke.x) : k == 1 ? coef(k01.z, k01.w, ke.x)
                                                                 : coef(k2.x, k2.y, ke.x);
     R = fma(-c, flux(m.h, 2 * s, mee[2 * s + half]), R);
+    if (isnan(R)) return R;
   }
   if (visc) vertices(m.cvis, m.FGv, mexv, ke.y, 1.0);
   return R;

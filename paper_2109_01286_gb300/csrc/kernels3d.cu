@@ -226,11 +226,11 @@ __device__ __noinline__ double fallback3(const Fx3Args& m, int V, int v, int k, 
     return fx_decode(p[q], c, kBits3);
   };
   double s = 0.0;
-  for (int j = m.vptr[v]; j < m.vptr[v + 1]; ++j)
+  for (int j = m.vptr[v]; j < m.vptr[v + 1] && !isnan(s); ++j)      // NaN stays NaN
 #pragma unroll 1
     for (int d = 2; d >= 0; --d)
       s = fma(m.cv[(size_t)12 * j + 3 * k + d], value((size_t)3 * m.vidx[j] + d), s);
-  for (int j = m.eptr[v]; j < m.eptr[v + 1]; ++j)
+  for (int j = m.eptr[v]; j < m.eptr[v + 1] && !isnan(s); ++j)
     s = fma(m.ce[(size_t)4 * j + k], value((size_t)3 * V + m.eidx[j]), s);
   return s;
 }
