@@ -267,7 +267,7 @@ __device__ __forceinline__ bool sums_fixed(int e, int E, const int* s, const Edg
   const Codes3 M0 = max_codes3(M, ld_codes3(fx.uc, s[0])), M1 = max_codes3(M, ld_codes3(fx.uc, s[5]));
   if (any_raw3(max_codes3(M0, M1))) return false;
   const int2 we = __ldg(fx.w5e + e);
-  // a component may lie one code below the scale, a momentum as far as sqrt(rho E) of its side reaches (as in 2D,
+  // a component may lie two codes below the scale, a momentum as far as sqrt(rho E) of its side reaches (as in 2D,
   // edge64.cuh: FP64 sums are the more accurate ones below that)
   int top[5], t0[5], t1[5];
   float unit[5];                                   // FP32 value of 2^-(L-1) of the scale
@@ -283,7 +283,7 @@ __device__ __forceinline__ bool sums_fixed(int e, int E, const int* s, const Edg
 #pragma unroll
   for (int q = 0; q < 5; ++q) {
     const bool mom = q >= 1 && q < 4;
-    apart |= top[q] - min(mom ? max(t0[q], m0) : t0[q], mom ? max(t1[q], m1) : t1[q]) > 1;
+    apart |= top[q] - min(mom ? max(t0[q], m0) : t0[q], mom ? max(t1[q], m1) : t1[q]) > 2;
   }
   if (apart) return false;
   // a pair's limbs at its component's scale (far: some shift of the node is 32 or more)

@@ -126,9 +126,9 @@ __device__ __forceinline__ bool any_raw8(uint4 a) {
 }
 
 // A side's sum is cut at 2^-57 of the scale that it shares with the other side, whose far node it does not
-// read.  True if no component of either side lies more than one code (a factor of two) below that scale: over the
-// weights of a 16x16 mesh and values within a factor e, the sums' errors in units of 2^-53 of the value
-// are then 0.50 rms and 1.6 at most, those of FP64 sums 1.07 and 5.1 (at the scale itself 0.43 and
+// read.  True if no component of either side lies more than two codes (a factor of four) below that scale:
+// over the weights of a 16x16 mesh and values within a factor e, the sums' errors in units of 2^-53 of the
+// value are then 0.70 rms and 3.0 at most, those of FP64 sums 1.07 and 5.1 (at the scale itself 0.43 and
 // 1.2, three codes below it 1.17 and 5.7).  A momentum is compared with sqrt(rho E) of its side
 // too, the size of the terms that it is added to in the flux, so that momenta around zero send no edge to
 // FP64.  m: codes of the four middle nodes, a, b: of the far ones (values, then derivatives), d: how far the
@@ -145,8 +145,8 @@ __device__ __forceinline__ bool sides_in_range(uint4 m, uint4 a, uint4 b, int d,
   };
   const uint2 ta = tops(a), tb = tops(b), ra = refs(ta), rb = refs(tb);
   top = make_uint2(__vmaxs2(ta.x, tb.x), __vmaxs2(ta.y, tb.y));
-  return (__vcmpgts2(__vsub2(top.x, __vmins2(ra.x, rb.x)), 0x00010001u) |
-          __vcmpgts2(__vsub2(top.y, __vmins2(ra.y, rb.y)), 0x00010001u)) == 0u;
+  return (__vcmpgts2(__vsub2(top.x, __vmins2(ra.x, rb.x)), 0x00020002u) |
+          __vcmpgts2(__vsub2(top.y, __vmins2(ra.y, rb.y)), 0x00020002u)) == 0u;
 }
 
 // The 5-node sums of both sides in fixed point (fixed_point.cuh): 120 DFMA, half of the smooth edge's
