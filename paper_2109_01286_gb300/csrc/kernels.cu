@@ -777,7 +777,7 @@ __device__ __forceinline__ void edge_body64(int e, int Ef, int V, const int32_t*
   ld4(Ua + (size_t)s[3] * 12, wj);
   double W[2][4];
   float cf[6][4];
-  if (!FX || !edge_fixed64<LIST>(e, Ef, s, fx, d2f_rn(nx), d2f_rn(ny), ph, W, cf, ws)) {
+  if (!FX || (!LIST && !fx.uf) || !edge_fixed64<LIST>(e, Ef, s, fx, d2f_rn(nx), d2f_rn(ny), ph, W, cf, ws)) {
     if (LIST && FX) {             // FP64 sums with 8 lanes; every component is decided again
       asm volatile("cp.async.wait_all;" ::: "memory");
       fx.list[atomicAdd(fx.count, 1)] = make_int2(e, ph.force_branch == 1 ? 0 : 0xff);
@@ -1052,7 +1052,6 @@ __global__ void __launch_bounds__(kEdgeBlock, 4) k_edge64(int Ef, int V, const i
 }
 
 // One thread an edge for all branches (force_branch = "weno": there is no smooth edge to save the list for).
-template <bool FX>
 __global__ void __launch_bounds__(128, 3) k_edge64_weno(int Ef, int V, const int32_t* __restrict__ sten,
                                                         const double* __restrict__ nrm,
                                                         const double* __restrict__ w5,
@@ -1061,7 +1060,7 @@ __global__ void __launch_bounds__(128, 3) k_edge64_weno(int Ef, int V, const int
                                                         Phys ph, unsigned* err, uint8_t* __restrict__ dbg,
                                                         EdgeFx fx) {
   const int e = blockIdx.x * blockDim.x + threadIdx.x;
-  if (e < Ef) edge_body64<false, FX>(e, Ef, V, sten, nrm, w5, w3, Ua, h, ph, err, dbg, fx);
+  if (e < Ef) edge_body64<false, true>(e, Ef, V, sten, nrm, w5, w3, Ua, h, ph, err, dbg, fx);
 }
 
 // edge_fixed64's 5-node sum of one side's component q (the same integers, so the same bits).
@@ -1106,19 +1105,40 @@ __device__ __forceinline__ bool lane_fixed64(int e, int Ef, const int* s, int si
 __device__ __forceinline__ double lane_xor(double x, int o) { return __shfl_xor_sync(0xffffffffu, x, o, 8); }
 __device__ __forceinline__ double lane_of(double x, int l) { return __shfl_sync(0xffffffffu, x, l, 8); }
 
+// Edges with 3-node values up to which they take 8 lanes each, and one thread each above (in a list, whose
+// edges lie apart in memory): 60 FP64 instructions an edge in 8 lanes and 32 in one thread, but the chain of one warp
+// is three times as long (see launch_edge).  A residual with 9,400 listed edges 165 us in 8 lanes and 185 in
+// one thread each (191x191), 18,600 215 and 206, 40,800 578 and 491 (400x400), 80,000 815 and 579.
+constexpr int kEdge8MaxWeno = 6500, kList8Max = 20000;
+
+// Long lists: one thread an edge.  A function of its own, so that the registers of the 8-lane form stay as they are
+// (inlined, it spilled them: 10 of 127 us a residual at 191x191 with 0.7% of the edges listed).
+__device__ __noinline__ void listed_edges_by_thread(int n, int Ef, int V, const int32_t* __restrict__ sten,
+                                                    const double* __restrict__ nrm, const double* __restrict__ w5,
+                                                    const double* __restrict__ w3, const double* __restrict__ Ua,
+                                                    double* __restrict__ h, const Phys& ph, unsigned* err,
+                                                    uint8_t* __restrict__ dbg, const EdgeFx& fx) {
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < n; i += gridDim.x * blockDim.x)
+    edge_body64<false, true>(fx.list[i].x, Ef, V, sten, nrm, w5, w3, Ua, h, ph, err, dbg, fx);
+}
+
 // The listed edges (ALL: every edge of a small mesh), 8 lanes each: lane side * 4 + q holds component q of one side, so that Alg. 1's FP64
 // chain is an eighth as long.  An SM partition takes 64 clocks for one FP64 warp instruction, and in a
 // warp of the edge kernel a few listed edges would hold up all (690 FP64 instructions for both sides
 // and all components; 240 here).
 template <bool ALL>
-__global__ void __launch_bounds__(128) k_edge_weno(int Ef, int V, const int32_t* __restrict__ sten,
+__global__ void __launch_bounds__(128, 3) k_edge_weno(int Ef, int V, const int32_t* __restrict__ sten,
                                                    const double* __restrict__ nrm,
                                                    const double* __restrict__ w5,
                                                    const double* __restrict__ w3,
                                                    const double* __restrict__ Ua, double* __restrict__ h,
-                                                   Phys ph, unsigned* err, uint8_t* __restrict__ dbg,
-                                                   EdgeFx fx) {
+                                                   const __grid_constant__ Phys ph, unsigned* err, uint8_t* __restrict__ dbg,
+                                                   const __grid_constant__ EdgeFx fx) {
   const int n = ALL ? Ef : *fx.count;
+  if (!ALL && n > kList8Max) {                   // one thread an edge, the same bits
+    listed_edges_by_thread(n, Ef, V, sten, nrm, w5, w3, Ua, h, ph, err, dbg, fx);
+    return;
+  }
   const int l8 = threadIdx.x & 7, side = l8 >> 2, q = l8 & 3;
   const double g1 = ph.g1;
   const int groups = gridDim.x * (blockDim.x >> 3);
@@ -2168,7 +2188,7 @@ cudaError_t launch_vertex(const DevMesh& m, const double* U, const Phys& ph, cud
 // edges 60 and 45), 64 for 15,552 (102), 267 for 109,443 (520 in 8 lanes, 596 listed) and 981 for
 // 480,000 (2132, listed 2741).
 // Threads per block: an SM partition has its own FP64 unit, so blocks of 32 spread a small mesh best.
-constexpr int kEdge8Max = 8000, kEdge8MaxWeno = 6500;
+constexpr int kEdge8Max = 8000;
 static int edge_threads(int Ef) { return Ef <= 152 * 64 ? 32 : Ef <= 152 * 128 ? 64 : 128; }
 
 int edge_launches(const DevMesh& m, const Phys& ph) {
@@ -2199,8 +2219,7 @@ cudaError_t launch_edge(const DevMesh& m, const Phys& ph, cudaStream_t s) {
     }
     const int nt = edge_threads(m.Ef);
     if (ph.force_branch == 2) {
-      auto* k = fx.uf ? k_edge64_weno<true> : k_edge64_weno<false>;
-      k<<<blocks(m.Ef, nt), nt, 0, s>>>(m.Ef, m.V, m.sten, (const double*)m.nrm, (const double*)m.w5,
+      k_edge64_weno<<<blocks(m.Ef, nt), nt, 0, s>>>(m.Ef, m.V, m.sten, (const double*)m.nrm, (const double*)m.w5,
                                         (const double*)m.w3, (const double*)m.Ua, (double*)m.h, ph, m.err,
                                         m.dbg_branch, fx);
       return cudaGetLastError();
