@@ -618,21 +618,30 @@ __device__ __forceinline__ void sensor64(T u0, T u1, T u2, T u3, T u4, const Phy
 // weights), and whether the sensor finds them smooth.  Every rounding is written out, so that the kernels agree.
 __device__ __forceinline__ double weno64(const double* u, const double* k3, const Phys& ph, bool& smooth) {
   double s[3];
-  auto square = [&](int i, double a, double e) {     // (eps + 13/12 a^2 + e^2/4)^2
-    const double x = __dadd_rn(ph.eps, __fma_rn(__dmul_rn(13.0 / 12.0, a), a, __dmul_rn(__dmul_rn(0.25, e), e)));
+  // (eps + 13/12 a^2 + e^2/4)^2
+  auto square = [&](int i, double b) {
+    const double x = __dadd_rn(ph.eps, b);
     s[i] = __dmul_rn(x, x);
   };
-  square(0, __dadd_rn(__fma_rn(-2.0, u[1], u[0]), u[2]), __fma_rn(3.0, u[2], __fma_rn(-4.0, u[1], u[0])));
-  square(1, __dadd_rn(__fma_rn(-2.0, u[2], u[1]), u[3]), __dadd_rn(u[1], -u[3]));
-  square(2, __dadd_rn(__fma_rn(-2.0, u[3], u[2]), u[4]), __dadd_rn(__fma_rn(3.0, u[2], __dmul_rn(-4.0, u[3])), u[4]));
+  auto a2 = [](double a) { return __dmul_rn(13.0 / 12.0, a); };
+  auto e2 = [](double e) { return __dmul_rn(0.25, e); };
+  double a = __dadd_rn(__fma_rn(-2.0, u[1], u[0]), u[2]);
+  double e = __dadd_rn(__fma_rn(-4.0, u[1], u[0]), __dmul_rn(3.0, u[2]));
+  square(0, __fma_rn(a2(a), a, __dmul_rn(e2(e), e)));
+  a = __dadd_rn(__fma_rn(-2.0, u[2], u[1]), u[3]);
+  e = __dadd_rn(u[1], -u[3]);
+  square(1, __fma_rn(e2(e), e, __dmul_rn(a2(a), a)));
+  a = __dadd_rn(__fma_rn(-2.0, u[3], u[2]), u[4]);
+  e = __dadd_rn(__fma_rn(-4.0, u[3], __dmul_rn(3.0, u[2])), u[4]);
+  square(2, __fma_rn(a2(a), a, __dmul_rn(e2(e), e)));
   const double t0 = __dmul_rn(__dmul_rn(1.0 / 16.0, s[1]), s[2]), t1 = __dmul_rn(__dmul_rn(10.0 / 16.0, s[0]), s[2]);
   const double t2 = __dmul_rn(__dmul_rn(5.0 / 16.0, s[0]), s[1]), S = __dadd_rn(__dadd_rn(t0, t1), t2);
   smooth = t0 > __dmul_rn(ph.sens_lo, S) && t0 < __dmul_rn(ph.sens_hi, S);
   double c[3];
 #pragma unroll
   for (int i = 0; i < 3; ++i)
-    c[i] = __fma_rn(k3[3 * i + 2], u[i + 2], __fma_rn(k3[3 * i + 1], u[i + 1], __dmul_rn(k3[3 * i], u[i])));
-  return __dmul_rn(__fma_rn(t2, c[2], __fma_rn(t1, c[1], __dmul_rn(t0, c[0]))), rcp64(S));
+    c[i] = __fma_rn(k3[3 * i + 2], u[i + 2], __fma_rn(k3[3 * i], u[i], __dmul_rn(k3[3 * i + 1], u[i + 1])));
+  return __dmul_rn(__fma_rn(t2, c[2], __fma_rn(t0, c[0], __dmul_rn(t1, c[1]))), rcp64(S));
 }
 
 // Characteristic values of the conservative values v: rows q_n - c, entropy, shear, q_n + c of the
