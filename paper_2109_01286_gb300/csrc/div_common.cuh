@@ -33,7 +33,7 @@ __device__ __forceinline__ bool finite_bits(double x) {
   return ((unsigned)(__double_as_longlong(x) >> 52) & 0x7ffu) != 0x7ffu;
 }
 
-// G lanes per active vertex (G in {1, 2, 4}); lanes stride over the CSR entries; the 12 partial
+// G lanes per active vertex (G in {1, 2, 4, 8}); lanes stride over the CSR entries; the 12 partial
 // sums are combined by a fixed reduce-scatter over the group (each level halves the values a
 // lane holds), so the result is deterministic and every add is useful.  acc = div(f) -
 // div(f_vis) for the 12 rows; R = -acc.

@@ -19,9 +19,12 @@
 // [entry] x {d0 hi, d0 lo, dx hi, dx lo} and [entry] x {dy hi, dy lo}: the bytes of the FP64
 // coefficients.  k_vertex and k_edge write the fluxes in the stored form of fixed_point.cuh with
 // codes per vertex and per edge; an edge's codes cover its end vertices, so the row's scale is the
-// largest over its edges.  Tiles of 16 rows (8 in meshes of fewer than kFxSmallRows, where more
-// blocks matter more than shared fluxes): a tile of 16 reads about 60 distinct vertices and 190
-// edges, a quarter of its rows' entries.
+// largest over its edges.  Tiles of 16 rows: a tile reads about 60 distinct vertices and 190 edges, a
+// quarter of its rows' entries; 8 in meshes of fewer than kFxSmallRows, for more blocks.  The line is not
+// sharp: a residual with tiles of 8 and 16 and the better lane count took 35.2 and 33.2 us with 576 rows, 49.7 and
+// 49.5 with 10,000, 75.2 and 74.5 with 19,881, 85.2 and 83.2 with 25,600, 226 and 225 with 90,000;
+// with 4 and 8 lanes 37 and 35 us with 576 rows, 50 and 52 with 10,000, 76 and 75 with 19,881, 126 and 124
+// with 40,000, 225 and 235 with 90,000.
 #include <algorithm>
 
 #include "div_common.cuh"
@@ -229,14 +232,9 @@ __device__ __noinline__ double fallback_sum(const DivFx& m, int r, int k, int q,
   return R;
 }
 
-// 16 bytes global -> shared, asynchronously (cp.async).
-__device__ __forceinline__ void copy16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
 __device__ __forceinline__ void copy8(void* dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 8;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
 }
-__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // One block: the rows of tile blockIdx.x, G lanes each.  Three rounds of loads: the tile's record
 // (the ids of the vertices and edges its rows read, each once, and the entries' positions in them)

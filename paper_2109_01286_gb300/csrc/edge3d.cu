@@ -8,7 +8,7 @@
 // warp alone 64.  So the sums run on the integer pipe (fixed_point.cuh; nodes as pairs with codes per
 // component, weights as limbs), the sensor's differences are integer differences rounded once to
 // FP32, the flux is formed from primitive jumps (150 FP64 instructions), and edges with a 3-node (or
-// undecided) component are listed for a second kernel of 16 lanes an edge.
+// undecided) component are listed for a second kernel of two lanes an edge.
 // 24^3 (96,768 edges, 1.5% listed): 93 us, before (one kernel, one thread an edge) 150 us; 12^3: 50 against 67 us.
 #include <cuda_runtime.h>
 
@@ -18,6 +18,7 @@
 #include "fp64_roots.cuh"
 #include "fp_convert.cuh"
 #include "kernels3d.hpp"
+#include "mbar.cuh"
 #include "record3.cuh"
 
 namespace hfd {
@@ -29,13 +30,6 @@ constexpr unsigned kErrIndex = 4u;
 constexpr float kGuard3 = 4e-3f;
 
 constexpr int kEdgeThreads3 = 128;
-
-// 16 bytes global -> shared, asynchronously.
-__device__ __forceinline__ void copy16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((unsigned)__cvta_generic_to_shared(dst)), "l"(src)
-               : "memory");
-}
-__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // ---- states
 struct Prim3 {       // of a state w: 1/rho, sqrt(rho), velocity, pressure, E + p, enthalpy
@@ -623,12 +617,12 @@ cudaError_t launch3_edge(const DevMesh3& m, const Phys3& ph, cudaStream_t s) {
   if (m.E == 0) return cudaSuccess;
   const Edge3Fx fx = edge3_fx(m);
   int4* rec = div3_lanes(m) == 0 ? m.fx.rec : nullptr;
-  const int nt = m.E <= 152 * 64 ? 32 : m.E <= 152 * 128 ? 64 : kEdgeThreads3;
+  const int nt = m.E <= kSms * 64 ? 32 : m.E <= kSms * 128 ? 64 : kEdgeThreads3;
   k3_edge<<<(unsigned)((m.E + nt - 1) / nt), nt, 0, s>>>(m.E, m.V, m.sten, m.frame, m.w5, m.Ua, m.h, rec, fx, ph,
                                                          m.err);
   const cudaError_t st = cudaGetLastError();
   if (st != cudaSuccess) return st;
-  const int64_t blocks = std::min<int64_t>(((int64_t)m.E * 2 + 63) / 64, 152 * 8);
+  const int64_t blocks = std::min<int64_t>(((int64_t)m.E * 2 + 63) / 64, kSms * 8);
   k3_edge_weno<<<(unsigned)blocks, 64, 0, s>>>(m.E, m.V, m.sten, m.frame, m.w3, m.Ua, m.h, rec, fx, ph);
   return cudaGetLastError();
 }

@@ -1,4 +1,4 @@
-// Fixed-point dot products for the FP64 divergence kernels.
+// Fixed-point dot products for the FP64 divergence and 5-node sums.
 //
 // GB300 issues FP64 multiply-adds at 2 lanes per clock and SM, and 32x32+64-bit integer
 // multiply-adds at 64 (measured; FP32 at 128).  A divergence row is a sum of products with one
@@ -9,10 +9,12 @@
 //   sum a b = 2^(2 L) sum ah bh + 2^L sum (ah bl + al bh)     (+ sum al bl, left out: below
 //                                                              2^(1-2L) of the scale per product)
 // is three integer multiply-adds per product instead of one DFMA: 3/64 against 1/2 clock.
-// The sums are exact, so they do not depend on the order of the entries or on how lanes share
-// them.  Only the factors are rounded, to 2^-57 of the row's largest (L = 29), against one rounding
-// of 2^-53 of the running sum per product in FP64: over random rows of 60 to 110 products the rms
-// error is 0.15 to 0.35 of the FP64 sum's.
+// The sums of the three are exact, so they do not depend on the order of the entries or on how lanes share
+// them.  The factors are rounded to 2^-57 of their row's scale and the fourth product is left out, against one
+// rounding of 2^-53 of the running sum per product in FP64: over random rows of 60 to 110 products the rms
+// error is 0.15 to 0.35 of the FP64 sum's, and 0.2 to 0.7 where the fluxes vary by a factor e to e^2.
+// Values far below the scale lose bits: the scale has to be that of values that are added (see
+// sides_in_range).
 //
 // Bounds: a row's coefficients take a scale of which they add up to kFxCoefSum = 127 at most, which for rows
 // of up to 127 products is the largest one's; with |bh| <= 2^(L-1) the high products then add up to
@@ -24,6 +26,7 @@
 
 namespace hfd {
 
+constexpr int kSms = 152;          // SMs of a GB300, for the grids and block sizes of the kernels that use these sums
 constexpr int kFxBits = 29;        // L
 constexpr int kFxCoefSum = 127, kFxCarry = 40;
 constexpr int kFxRaw = 0x7ff;      // code of a group stored as raw FP64 values

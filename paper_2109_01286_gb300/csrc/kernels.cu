@@ -2,18 +2,20 @@
 // (arXiv 2109.01286) for sm_103a, and the SSP-RK3 stage update fused into the divergence.
 //
 //   k_vertex : analytic Euler (and viscous) fluxes at every vertex (Sec. 2.3) plus an AoS copy
-//              of the state for the edge gathers.
-//   k_edge   : Alg. 1 on both sides of every flux edge -- Roe average of the end states,
+//              of the state for the edge gathers, and the stored pairs of the fixed-point kernels.
+//   k_edge   : (FP32; FP64: k_edge64 for edges whose sides take 5-node values and k_edge_weno for the
+//              others, or for all edges of a small mesh; k_edge64_weno where the branch is forced) Alg. 1 on both sides of every flux edge -- Roe average of the end states,
 //              characteristic projection of the 6 stencil nodes, uniform-WENO5 sensor,
 //              5-node Hermite value or omega-weighted 3-node values (Eq. (2d_hweno_intp)),
 //              back-projection -- then the Riemann (Roe) flux along the edge.
-//   k_div    : least-squares divergence rows d_0, d_x, d_y (Eq. (flux_polynomials)) as a CSR
+//   k_div    : (FP32 and FP64 sums; FP64's default is k_div_fx in div_fixed.cu) least-squares divergence rows d_0, d_x, d_y (Eq. (flux_polynomials)) as a CSR
 //              gather over stencil vertices and edges by a group of lanes per vertex with a
 //              fixed shuffle reduction (deterministic, no atomics), fused with the
 //              Runge-Kutta stage combination (Sec. 2.3, end).
 //
-// No step is a dense contraction, so no tensor-core path exists: the kernels are bound by
-// FP64 issue (FP64 path) or by memory traffic (FP32-bulk path).  The bulk precision T is
+// No step is a dense contraction, so no tensor-core path exists.  FP64 sums of products are bound by the FP64
+// pipe (2 multiply-adds per clock and SM), the fixed-point kernels by latency at 10 to 14 warps an SM, the
+// FP32-bulk divergence by memory traffic and gather latency.  The bulk precision T is
 // double or float; the state, the stage combination and the WENO weight ratios are double.
 #include <cuda_runtime.h>
 
@@ -2198,7 +2200,7 @@ cudaError_t launch_vertex(const DevMesh& m, const double* U, const Phys& ph, cud
 // 480,000 (2132, listed 2741).
 // Threads per block: an SM partition has its own FP64 unit, so blocks of 32 spread a small mesh best.
 constexpr int kEdge8Max = 8000;
-static int edge_threads(int Ef) { return Ef <= 152 * 64 ? 32 : Ef <= 152 * 128 ? 64 : 128; }
+static int edge_threads(int Ef) { return Ef <= kSms * 64 ? 32 : Ef <= kSms * 128 ? 64 : 128; }
 
 int edge_launches(const DevMesh& m, const Phys& ph) {
   return m.Ef == 0 ? 0 : m.precision == 0 && ph.force_branch != 2 && m.Ef > kEdge8Max ? 2 : 1;
@@ -2238,7 +2240,7 @@ cudaError_t launch_edge(const DevMesh& m, const Phys& ph, cudaStream_t s) {
                                       (const double*)m.w3, (const double*)m.Ua, (double*)m.h, ph, m.err,
                                       m.dbg_branch, fx);
     // the list's length is known on the device only: enough blocks for a full GPU, or the whole mesh
-    const int nb = std::min(blocks((long long)m.Ef * 8, nt), 152 * 4 * (128 / nt));
+    const int nb = std::min(blocks((long long)m.Ef * 8, nt), kSms * 4 * (128 / nt));
     k_edge_weno<false><<<nb, nt, 0, s>>>(m.Ef, m.V, m.sten, (const double*)m.nrm, (const double*)m.w5,
                                          (const double*)m.w3, (const double*)m.Ua, (double*)m.h, ph,
                                          m.err, m.dbg_branch, fx);

@@ -213,7 +213,7 @@ cudaError_t launch_div(const DevMesh& m, const double* Us, const double* Un, dou
 cudaError_t pack_w5_fx(const DevMesh& m, int* flag, cudaStream_t s);
 cudaError_t pack_div_fx(const DevMesh& m, int* flag, cudaStream_t s);
 // Raises the kernels' shared-memory limit for m.fx.smem (at most kFxSmemMax).
-constexpr int kFxSmallRows = 20000;     // meshes of fewer rows take tiles of 8 rows
+constexpr int kFxSmallRows = 20000;     // meshes of fewer rows take tiles of 8 rows (div_fixed.cu)
 constexpr int kFxSmemMax = 128 * 1024;
 cudaError_t prepare_div_fx(const DevMesh& m);
 cudaError_t launch_div_fx(const DevMesh& m, const StageArgs& sa, const Phys& ph, int lanes,

@@ -6,7 +6,7 @@
 //   k3_div_fx  8 lanes per vertex: the CSR gather of the least-squares divergence rows
 //              d_0, d_x, d_y, d_z over the vertex fluxes and edge fluxes (Eq.
 //              (flux_polynomials) in 3D) in fixed point, fused with the SSP-RK3 stage update;
-//   k3_div     the same gather in FP64, 1, 2 or 4 lanes per vertex (chosen lanes, long rows).
+//   k3_div     the same gather in FP64, 1, 2 or 4 lanes per vertex (chosen lanes; meshes without the fixed-point form).
 #include <cuda_runtime.h>
 
 #include "fixed_point.cuh"
@@ -235,12 +235,9 @@ __device__ __noinline__ double fallback3(const Fx3Args& m, int V, int v, int k, 
   return s;
 }
 
-// 16 bytes global -> shared, asynchronously, with and without a copy left in L1.
+// copy16 with a copy left in L1.
 __device__ __forceinline__ void copy16_l1(void* dst, const void* src) {
   asm volatile("cp.async.ca.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
-__device__ __forceinline__ void copy16(void* dst, const void* src) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
 }
 __device__ __forceinline__ void copies_commit() { asm volatile("cp.async.commit_group;" ::: "memory"); }
 __device__ __forceinline__ void copies_wait_but_one() { asm volatile("cp.async.wait_group 1;" ::: "memory"); }

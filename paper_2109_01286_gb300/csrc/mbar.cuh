@@ -1,4 +1,5 @@
-// mbarriers and 1D bulk copies (cp.async.bulk) with bounded waits.
+// Asynchronous copies to shared memory: mbarriers and 1D bulk copies (cp.async.bulk) with bounded waits, and
+// copies of a thread's own (cp.async).
 #pragma once
 #include <cuda_runtime.h>
 
@@ -36,6 +37,11 @@ __device__ __forceinline__ void bulk_g2s(void* dst, const void* src, unsigned by
 __device__ __forceinline__ void bulk_prefetch(const void* src, unsigned bytes) {
   asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(src), "r"(bytes) : "memory");
 }
+// 16 bytes global -> shared by this thread, past L1, and the wait for all such copies of it.
+__device__ __forceinline__ void copy16(void* dst, const void* src) {
+  asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void copies_wait() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 // Bounded wait for the phase of `bar` with parity `parity`; false if the bound ran out.
 __device__ __forceinline__ bool mbar_wait(unsigned long long* bar, unsigned parity) {
   const unsigned a = smem_addr(bar);
