@@ -39,13 +39,13 @@ import synth  # noqa: E402
 METRIC = "vertex-stage updates/s"
 CPU_PATCH_N = 32                 # bounded oracle sample: 32 x 32 patch of the same workload
 # DRAM bytes (read + write) per launch of each kernel on the default 1024 x 1024 workload, from
-# one ncu capture per kernel (one launch, one-pass metrics; profiles/traffic_four_quadrant_1024x1024.md),
-# valid for the kernel and data-layout sources they were taken on: when their hash
-# differs the figures are stale and the line reports traffic as null
+# one ncu capture per kernel (one launch, one-pass metrics), valid for the kernel and data-layout sources they
+# were taken on: when their hash differs the figures are stale and the line reports traffic as null
 TRAFFIC_SOURCES = tuple("paper_2109_01286_gb300/csrc/" + f for f in
-                        ("kernels.cu", "div_fixed.cu", "edge64.cuh", "fixed_point.cuh", "api.cu"))
-TRAFFIC_SHA = "ed41e003f9d1e831"
-DRAM_TRAFFIC_1024 = {"k_div_fx": 2964.6e6, "k_edge64": 1279.1e6, "k_div<float>": 1794.5e6, "k_div_df": 2923.1e6}
+                        ("kernels.cu", "div_fixed.cu", "edge64.cuh", "fixed_point.cuh", "api.cu", "div_common.cuh",
+                         "kernels.hpp", "mbar.cuh", "fp64_roots.cuh", "fp_convert.cuh"))
+TRAFFIC_SHA = "3862551025f808d9"
+DRAM_TRAFFIC_1024 = {"k_div_fx": 2964.5e6, "k_edge64": 1285.4e6, "k_div<float>": 1794.7e6, "k_div_df": 2923.0e6}
 # The FP64 kernels' sums of products run on the integer pipe, so their FLOPs are no share of the FP64
 # peak: they are set against the HBM, with the FP64-equivalent rate beside it
 FP64_KERNELS = {"vertex": "k_vertex<double>", "edge": "k_edge64", "div": "k_div_fx", "ghost": "k_ghost"}
