@@ -80,3 +80,24 @@ def test_3d_side_does_not_lose_bits_to_the_other_sides_far_node(ratio):
     for g in range(4):
         d = slice(5 * g, 5 * g + 5)
         assert torch.linalg.norm(R[d] - P[d]) <= TOL * torch.linalg.norm(P[d])
+
+
+@pytest.mark.parametrize("nx", [40, 60])
+def test_adjoint_of_edges_in_fp64_sums(nx):
+    """One vertex 8 times the others: some edges lie outside the fixed-point range of the sums.  lambda_n is lambda
+    and dt (1e-3) times sums whose terms are off by up to 110 units of 2^-53 and cancel by up to 1e2: the
+    norms agree to 1e-3 x 110 x 1.1e-16 x 1e2 and lambda's own rounding, below 1e-13."""
+    import paper_2109_01286_gb300 as pkg
+    m = synth.jittered_grid(nx, nx, 10.0, 10.0, seed=1)
+    U = synth.isentropic_vortex(m)
+    U[:, int(np.argmin(np.hypot(m["x"] - 4.0, m["y"] - 4.5)))] *= 8.0
+    mesh = pkg.Mesh(m)
+    Ui = mesh.import_state(torch.from_numpy(U).cuda())
+    lam = torch.randn(Ui.shape, dtype=torch.float64, device="cuda", generator=torch.Generator("cuda").manual_seed(1))
+    out = {}
+    for lanes in (8, 1):
+        mesh.set_lanes(lanes)
+        out[lanes] = mesh.adjoint(Ui, lam, dt=1e-3)
+    mesh.check()
+    assert not torch.equal(out[8], out[1])
+    assert torch.linalg.norm(out[8] - out[1]) <= 1e-13 * torch.linalg.norm(out[1])
